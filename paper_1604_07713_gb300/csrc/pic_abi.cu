@@ -362,6 +362,7 @@ pic_status pic_create(const pic_config *cfg, int32_t n_instances, pic_ctx **out)
             Instance &in = ctx->inst[i];
             in.cfg = cfg[i];
             in.mesh_mem.cache = &ctx->cache;
+            in.inv_mem.cache = &ctx->cache;
             in.part_mem[0].cache = &ctx->cache;
             in.part_mem[1].cache = &ctx->cache;
             GB_CUDA(cudaMallocHost(&in.red_host, 64));
@@ -394,6 +395,7 @@ pic_status pic_destroy(pic_ctx *ctx) {
         if (in.mg_cycle) cudaGraphExecDestroy(in.mg_cycle);
         repairs_release(in);
         in.mesh_mem.release_all();
+        in.inv_mem.release_all();
         in.part_mem[0].release_all();
         in.part_mem[1].release_all();
         if (in.red_host) cudaFreeHost(in.red_host);

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <array>
 #include <string>
 #include <map>
 #include <unordered_map>
@@ -216,8 +217,11 @@ struct Instance {
     bool mg_on_device = false;     // last solve ran its loop on the device (stats below)
     double *mg_stats = nullptr;    // device: [cycles, rel. residual, max rel. since reset]
     double *coarse_inv = nullptr;        // coarsest multigrid level: dense FP64 inverse (small levels)
+    double *coarse_inv_mem = nullptr;    // its memory, kept over mesh rebuilds, and the root grid
+    std::array<int, 4> coarse_inv_key = {0, 0, 0, 0};  // (nx, ny, walls) it was formed for
+    DeviceArena inv_mem;
     void *small_item = nullptr;          // meshes that fit one block: the solve's work item
-    size_t small_smem = 0;               // and its dynamic shared memory
+    size_t small_smem = 0;               // and the shared memory of its levels
     int small_cluster = 1;               // CTAs of its cluster when solved alone
     cudaGraphExec_t mg_cycle = nullptr;  // multi-block meshes: one captured cycle (V-cycle,
     int64_t mg_cycle_nodes = 0;          // correction, residual, norm read-back) and its launches
@@ -287,7 +291,9 @@ struct pic_ctx {
     int64_t mesh_epoch = 0, batch_epoch = -1;
     int batch_n = 0;
     void *batch_items = nullptr;
-    size_t batch_smem = 0;
+    size_t batch_smem = 0;   // the largest instance's levels
+    int batch_cells = 0;     // the largest instance's cells
+    int batch_cluster = 1;   // CTAs per instance
     gbpic::DeviceArena batch_mem;
     gbpic::BlockCache cache;  // device blocks released by this context, for reuse
     // captured multi-instance step (pic_graph.cu)

@@ -10,6 +10,7 @@
 // that spreads the FP64 work over its SMs (one CTA per instance in a batch).  Larger meshes
 // run one CUDA graph per solve whose WHILE node repeats the cycle until the device decides.
 #include <algorithm>
+#include <array>
 #include <cmath>
 
 #include <cooperative_groups.h>
@@ -375,8 +376,15 @@ __global__ void __launch_bounds__(1024) k_coarse_cg(int64_t n, const int32_t *__
 // ---- levels held in shared memory by one block (n <= kSmallN cells each) ----------------
 constexpr int kSmallN = 8192;          // 8 cells per thread of a 1024-thread block
 constexpr int kMaxSmallLevels = 16;
-constexpr int kSmallSmemCap = 200 * 1024;
+constexpr int kSmallSmemCap = 201 * 1024;  // the levels' vectors
+constexpr int kSmallSmemMax = 222 * 1024;  // with the sums' buffers and the coarsest inverse
+constexpr int kDirectN = 128;  // coarsest levels up to this size are solved by a dense inverse
 
+// A level of root boxes only (no refinement) is a row-major nx x ny grid whose operator is the
+// 5-point stencil, applied from the cell index without the ELL arrays (`uniform`).  Every such
+// level but the coarsest has even nx and ny, so its red-black colouring is proper (also across
+// a periodic wrap), and its vectors are stored by colour (`fast`): cell (ix, iy) of colour
+// c = (ix + iy) & 1 at c * hs + iy * nx / 2 + ix / 2.
 struct SmallLevel {
     int32_t n;
     const int32_t *col;
@@ -384,20 +392,22 @@ struct SmallLevel {
     const uint8_t *color;
     const int32_t *child4;  // children (in the finer level) of this level's cells
     const int32_t *parent;  // this level's cells -> cells of the next coarser level
-    int32_t off;            // smem offset (floats) of x; b follows at off + n
-    // A level of root boxes only (no refinement) is a row-major nx x ny grid whose operator
-    // is the 5-point stencil; it is applied from the cell index, without the ELL arrays.
+    int32_t off;            // smem offset (floats) of x; b follows at off + boff
+    int32_t boff;
     int32_t uniform, nx, ny;
     uint32_t nx_magic;   // floor(i / nx) == mdiv(i, nx_magic) for every cell index i < n
     uint32_t nxh_magic;  // the same for nx / 2 (uniform levels with even nx)
+    int32_t fast, half, hs;  // stored by colour: cells per colour, stride between the colours (half + 4)
+    int32_t nthr, kc;        // threads that sweep the level, cells of each colour per thread (1, 2 or 4)
 };
 struct SmallDesc {
     int nlev;  // levels g0 .. g0 + nlev - 1 live in shared memory
     int bcx, bcy;
     SmallLevel lv[kMaxSmallLevels];
     int32_t off_cg;  // smem offset of the coarsest CG vectors r, p, q (3 n)
-    int32_t smem_floats;
-    const double *cinv;  // coarsest level: dense FP64 inverse (n x n, row-major), or null (CG)
+    int32_t smem_floats;  // a multiple of 4
+    const double *cinv;  // coarsest level: dense FP64 inverse (n x n, symmetric), or null (CG)
+    int32_t inv_words;   // its words if it is copied to shared memory, else 0
 };
 
 // floor(i / d) by a multiply-high reciprocal m = floor((2^32 - 1) / d) + 1; m = 0 stands for
@@ -405,33 +415,41 @@ struct SmallDesc {
 __host__ __device__ __forceinline__ uint32_t mdiv_magic(uint32_t d) { return d <= 1u ? 0u : 0xFFFFFFFFu / d + 1u; }
 __device__ __forceinline__ int mdiv(int i, uint32_t m) { return m ? (int)__umulhi((uint32_t)i, m) : i; }
 
+// Where cell i of a level sits in its x (and b) vector.
+__device__ __forceinline__ int sm_pos(const SmallLevel &L, int i) {
+    if (!L.fast) return i;
+    const int iy = mdiv(i, L.nx_magic), ix = i - iy * L.nx;
+    return ((ix + iy) & 1) * L.hs + iy * (L.nx >> 1) + (ix >> 1);
+}
+
 // Neighbour sum s and diagonal d of row i, so that (A x)_i = d x_i - s.  Uniform levels:
 // face conductance 1 to each neighbour, 2 to a Dirichlet wall, none at a Neumann wall.
 template <typename T>
-__device__ __forceinline__ T uni_row(int nx, int ny, uint32_t magic, int bcx, int bcy, const T *x, int i, T &d) {
+__device__ __forceinline__ T uni_row(int nx, int ny, uint32_t magic, int bcx, int bcy, const T *x, int i, int &dd) {
     const int iy = mdiv(i, magic), ix = i - iy * nx;
-    T s = 0;
-    int dd = 0;  // counted in integers: the diagonal is converted once
-    if (ix > 0) { s += x[i - 1]; dd += 1; }
-    else if (bcx == PIC_BC_PERIODIC) { s += x[i + nx - 1]; dd += 1; }
+    T l = 0, r = 0, dn = 0, up = 0;
+    dd = 0;
+    if (ix > 0) { l = x[i - 1]; dd += 1; }
+    else if (bcx == PIC_BC_PERIODIC) { l = x[i + nx - 1]; dd += 1; }
     else if (bcx == PIC_BC_DIRICHLET) dd += 2;
-    if (ix < nx - 1) { s += x[i + 1]; dd += 1; }
-    else if (bcx == PIC_BC_PERIODIC) { s += x[i - nx + 1]; dd += 1; }
+    if (ix < nx - 1) { r = x[i + 1]; dd += 1; }
+    else if (bcx == PIC_BC_PERIODIC) { r = x[i - nx + 1]; dd += 1; }
     else if (bcx == PIC_BC_DIRICHLET) dd += 2;
-    if (iy > 0) { s += x[i - nx]; dd += 1; }
-    else if (bcy == PIC_BC_PERIODIC) { s += x[i + (ny - 1) * nx]; dd += 1; }
+    if (iy > 0) { dn = x[i - nx]; dd += 1; }
+    else if (bcy == PIC_BC_PERIODIC) { dn = x[i + (ny - 1) * nx]; dd += 1; }
     else if (bcy == PIC_BC_DIRICHLET) dd += 2;
-    if (iy < ny - 1) { s += x[i + nx]; dd += 1; }
-    else if (bcy == PIC_BC_PERIODIC) { s += x[i - (ny - 1) * nx]; dd += 1; }
+    if (iy < ny - 1) { up = x[i + nx]; dd += 1; }
+    else if (bcy == PIC_BC_PERIODIC) { up = x[i - (ny - 1) * nx]; dd += 1; }
     else if (bcy == PIC_BC_DIRICHLET) dd += 2;
-    d = (T)dd;
-    return s;
+    return ((l + r) + dn) + up;
 }
 
 __device__ __forceinline__ float sm_row(const SmallDesc &D, const SmallLevel &L, const float *x, int i, float &d,
                                         float &dinv) {
     if (L.uniform) {
-        const float s = uni_row<float>(L.nx, L.ny, L.nx_magic, D.bcx, D.bcy, x, i, d);
+        int dd;
+        const float s = uni_row<float>(L.nx, L.ny, L.nx_magic, D.bcx, D.bcy, x, i, dd);
+        d = (float)dd;
         dinv = __frcp_rn(d);
         return s;
     }
@@ -450,47 +468,15 @@ __device__ __forceinline__ float sm_row(const SmallDesc &D, const SmallLevel &L,
     return sm_row(D, L, x, i, d, dinv);
 }
 
-__device__ __forceinline__ int sm_color(const SmallLevel &L, int i) {
-    if (!L.uniform) return L.color[i];
-    const int iy = mdiv(i, L.nx_magic);
-    return (i - iy * L.nx + iy) & 1;
-}
-
-// Red-black Gauss-Seidel sweep in shared memory; each colour's new values are computed from
-// the current vector before any is written (deterministic on non-uniform meshes).  The block
-// has 1024 threads; thread t owns cells t + 1024 k, k < 8, so the new values stay in registers.
+// Red-black Gauss-Seidel sweep of an ELL level in shared memory; each colour's new values are
+// computed from the current vector before any is written (cells of one colour can touch on a
+// non-uniform mesh, and the result must not depend on thread order).  The block has 1024
+// threads; thread t owns cells t + 1024 k, k < 8, so the new values stay in registers.
 constexpr int kPerThread = kSmallN / 1024;
 __device__ void sm_smooth(const SmallDesc &D, const SmallLevel &L, float *x, const float *b, bool first) {
     if (first) {
         for (int i = threadIdx.x; i < L.n; i += blockDim.x) x[i] = 0.0f;
         __syncthreads();
-    }
-    if (L.uniform && (L.nx & 1) == 0) {
-        // colour c of an even-width grid: in row iy the cells ix = 2m + ((c + iy) & 1)
-        const int half = L.n >> 1, nxh = L.nx >> 1;
-        for (int c = 0; c < 2; ++c) {
-            float t[kPerThread / 2];
-            int cell[kPerThread / 2];
-#pragma unroll
-            for (int k = 0; k < kPerThread / 2; ++k) {
-                const int j = threadIdx.x + 1024 * k;
-                cell[k] = -1;
-                if (j < half) {
-                    const int iy = mdiv(j, L.nxh_magic), m = j - iy * nxh;
-                    const int i = iy * L.nx + 2 * m + ((c + iy) & 1);
-                    float d, dinv;
-                    const float sn = sm_row(D, L, x, i, d, dinv);
-                    t[k] = (b[i] + sn) * dinv;
-                    cell[k] = i;
-                }
-            }
-            __syncthreads();
-#pragma unroll
-            for (int k = 0; k < kPerThread / 2; ++k)
-                if (cell[k] >= 0) x[cell[k]] = t[k];
-            __syncthreads();
-        }
-        return;
     }
     for (int c = 0; c < 2; ++c) {
         float t[kPerThread];
@@ -498,7 +484,7 @@ __device__ void sm_smooth(const SmallDesc &D, const SmallLevel &L, float *x, con
 #pragma unroll
         for (int k = 0; k < kPerThread; ++k) {
             const int i = threadIdx.x + 1024 * k;
-            mine[k] = i < L.n && sm_color(L, i) == c;
+            mine[k] = i < L.n && L.color[i] == c;
             t[k] = 0.0f;
             if (mine[k]) {
                 float d, dinv;
@@ -513,8 +499,6 @@ __device__ void sm_smooth(const SmallDesc &D, const SmallLevel &L, float *x, con
         __syncthreads();
     }
 }
-
-
 
 __device__ __forceinline__ float warp_sumf(float v) {
 #pragma unroll
@@ -618,157 +602,321 @@ __device__ void sm_coarse_cg(const SmallDesc &D, const SmallLevel &L, float *x, 
     __syncthreads();
 }
 
-// Coarsest level by its dense inverse C (at most kDirectN cells), applied in FP64:
-// x = C (b - mean(b)) with the mean taken out when the mesh is periodic in both directions (C
-// then inverts A + 1 1^T / n, which maps a zero-mean right-hand side to the zero-mean
-// solution).  Warp w forms rows w, w + 32, ...; all threads of the block call it.
-__device__ void sm_coarse_direct(const SmallDesc &D, const SmallLevel &L, float *x, const float *b, bool singular,
-                                 float *red) {
-    const int n = L.n, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-    double mb = 0.0;
-    if (singular) {
-        // every lane of warp 0 sums the (at most 64) values in the same order
-        __shared__ double mean_sh;
-        if (threadIdx.x < 32) {
-            double sb = 0.0;
-            for (int i = 0; i < n; ++i) sb += (double)b[i];
-            if (threadIdx.x == 0) mean_sh = sb / (double)n;
-        }
-        __syncthreads();
-        mb = mean_sh;
-    }
-    for (int r = threadIdx.x >> 5; r < n; r += nwarp) {
+// Barrier `id` (1 .. 15) over the first `nthr` threads of the block.
+__device__ __forceinline__ void part_bar(int id, int nthr) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthr) : "memory");
+}
+
+// Coarsest level by its dense inverse C (at most kDirectN cells), applied in FP64 by the first
+// nthr >= 256 threads: thread (part, row) sums a run of columns of its row (C is symmetric, so
+// lanes read consecutive words), then the parts are added in order.  The FP64 pipe retires two
+// lanes per clock and SM, so one multiply-add per matrix word and no shuffle trees is the
+// cheapest form.  Singular (periodic in both directions): C inverts A + 1 1^T / n, whose
+// inverse maps 1 to 1, so C (b - mean(b) 1) = C b - mean(b).  `scr` holds n + 512 doubles.
+__device__ void sm_coarse_direct(const SmallLevel &L, const double *inv, float *x, const float *b, bool singular,
+                                 int nthr, int bar, double *scr) {
+    const int n = L.n, t = threadIdx.x;
+    double *ps = scr + n;
+    if (t < n) scr[t] = (double)b[t];
+    part_bar(bar, nthr);
+    const int n32 = (n + 31) & ~31, parts = min(nthr, 512) / n32;
+    const int part = t / n32, r = t - part * n32;
+    if (part < parts && r < n) {
+        const int per = (n + parts - 1) / parts, c1 = min(n, (part + 1) * per);
         double acc = 0.0;
-        for (int c = lane; c < n; c += 32) acc = fma(__ldg(D.cinv + r * n + c), (double)b[c] - mb, acc);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-        if (lane == 0) x[r] = (float)acc;
+        for (int c = part * per; c < c1; ++c) acc = fma(inv[c * n + r], scr[c], acc);
+        ps[part * n32 + r] = acc;
     }
-    __syncthreads();
+    part_bar(bar, nthr);
+    if (part == 0) {
+        double m = 0.0;
+        if (singular) {  // the warps of part 0 are whole (n32 is a multiple of 32)
+            for (int c = t & 31; c < n; c += 32) m += scr[c];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xFFFFFFFFu, m, o);
+            m /= (double)n;
+        }
+        if (r < n) {
+            double acc = ps[r];
+            for (int p = 1; p < parts; ++p) acc += ps[p * n32 + r];
+            x[r] = (float)(acc - m);
+        }
+    }
+}
+
+// ---- levels stored by colour --------------------------------------------------------------
+// Thread t sweeps the positions j = t + nthr k (k < K) of both colours.  The horizontal
+// neighbours of the cell at position j of one colour sit at j and at one of j - 1, j + 1 of the
+// other colour, the vertical ones at j - nx/2 and j + nx/2; a missing neighbour points to the
+// zero word at `half`.  The offsets and the reciprocal diagonals of a thread's cells are formed
+// once per leg and serve its four half sweeps, each of which costs 5 shared loads, 4 adds, a
+// multiply and one store per cell and one barrier (a colour reads only the other colour, so
+// values are updated in place).
+//
+// What bounds the solve is this serial chain of half sweeps.  512 x 16 cells, 4 cycles: 0.283 ms
+// when each cell's index division and wall tests were done in every half sweep and two barriers
+// ended it, 0.118 ms so (with the FP64 sums of small_sums and the three cluster barriers of
+// k_small_solve); 64 x 64 periodic, 7 cycles: 0.508 and 0.170 ms.
+template <int K> struct RbCells {
+    int oh0[K], oh1[K], od[K], ou[K];
+    float di0[K], di1[K];
+};
+template <int K> __device__ __forceinline__ void rb_cells(const SmallDesc &D, const SmallLevel &L, RbCells<K> &c) {
+    const int nxh = L.nx >> 1, half = L.half;
+    const bool px = D.bcx == PIC_BC_PERIODIC, py = D.bcy == PIC_BC_PERIODIC;
+    const int wx = D.bcx == PIC_BC_DIRICHLET ? 2 : (px ? 1 : 0), wy = D.bcy == PIC_BC_DIRICHLET ? 2 : (py ? 1 : 0);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int j = (int)threadIdx.x + L.nthr * k;
+        const int iy = mdiv(j, L.nxh_magic), m = j - iy * nxh;
+        const bool p = iy & 1;  // colour 0 of this row is at odd ix
+        const int hl = m > 0 ? j - 1 : (px ? j + nxh - 1 : half), hr = m < nxh - 1 ? j + 1 : (px ? j - nxh + 1 : half);
+        const int dl = m > 0 ? 1 : wx, dr = m < nxh - 1 ? 1 : wx;
+        c.od[k] = iy > 0 ? j - nxh : (py ? j + (L.ny - 1) * nxh : half);
+        c.ou[k] = iy < L.ny - 1 ? j + nxh : (py ? j - (L.ny - 1) * nxh : half);
+        const int dv = 1 + (iy > 0 ? 1 : wy) + (iy < L.ny - 1 ? 1 : wy);
+        c.oh0[k] = p ? hr : hl;
+        c.oh1[k] = p ? hl : hr;
+        c.di0[k] = __frcp_rn((float)(dv + (p ? dr : dl)));
+        c.di1[k] = __frcp_rn((float)(dv + (p ? dl : dr)));
+    }
+}
+// xs: this colour's values, xo: the other colour's
+template <int K>
+__device__ __forceinline__ void rb_half(float *xs, const float *xo, const int (&oh)[K], const int (&od)[K],
+                                        const int (&ou)[K], const float (&b)[K], const float (&di)[K], int nthr, int half) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int j = (int)threadIdx.x + nthr * k;
+        if (j < half) xs[j] = (b[k] + (((xo[j] + xo[oh[k]]) + xo[od[k]]) + xo[ou[k]])) * di[k];
+    }
+}
+
+// Pre-smoothing from x = 0 and the residual's restriction.
+template <int K>
+__device__ __forceinline__ void rb_down(const SmallDesc &D, const SmallLevel &L, const SmallLevel &Cc, float *sm, int bar) {
+    const int nthr = L.nthr, half = L.half;
+    float *x0 = sm + L.off, *x1 = x0 + L.hs;
+    const float *b0 = x0 + L.boff, *b1 = b0 + L.hs;
+    {
+        RbCells<K> c;
+        float bb0[K], bb1[K];
+        rb_cells<K>(D, L, c);
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int j = (int)threadIdx.x + nthr * k;
+            bb0[k] = bb1[k] = 0.0f;
+            if (j < half) {
+                bb0[k] = b0[j]; bb1[k] = b1[j];
+                x0[j] = bb0[k] * c.di0[k];  // the first half sweep reads zeros only
+            }
+        }
+        if (threadIdx.x == 0) x0[half] = x1[half] = 0.0f;  // missing neighbours
+        part_bar(bar, nthr);
+        rb_half<K>(x1, x0, c.oh1, c.od, c.ou, bb1, c.di1, nthr, half);
+        part_bar(bar, nthr);
+        for (int s = 1; s < kNu; ++s) {
+            rb_half<K>(x0, x1, c.oh0, c.od, c.ou, bb0, c.di0, nthr, half);
+            part_bar(bar, nthr);
+            rb_half<K>(x1, x0, c.oh1, c.od, c.ou, bb1, c.di1, nthr, half);
+            part_bar(bar, nthr);
+        }
+    }
+    // coarse cell p: the residuals of its children (0,0), (1,0), (0,1), (1,1) summed in this order
+    const int nxh = L.nx >> 1;
+    const bool px = D.bcx == PIC_BC_PERIODIC, py = D.bcy == PIC_BC_PERIODIC;
+    const int wx = D.bcx == PIC_BC_DIRICHLET ? 2 : (px ? 1 : 0), wy = D.bcy == PIC_BC_DIRICHLET ? 2 : (py ? 1 : 0);
+    float *bc = sm + Cc.off + Cc.boff;
+    for (int p = threadIdx.x; p < Cc.n; p += nthr) {
+        const int qy = mdiv(p, L.nxh_magic), qx = p - qy * nxh;
+        const int j0 = 2 * qy * nxh + qx, j1 = j0 + nxh;
+        const bool le = qx > 0, re = qx < nxh - 1, de = qy > 0, ue = 2 * qy + 2 < L.ny;
+        const bool hl = le || px, hr = re || px;
+        const int wl = le ? -1 : nxh - 1, wr = re ? 1 : 1 - nxh;
+        const int jd = de ? j0 - nxh : (py ? j0 + (L.ny - 1) * nxh : half);
+        const int ju = ue ? j1 + nxh : (py ? j1 - (L.ny - 1) * nxh : half);
+        const float x00 = x0[j0], x10 = x1[j0], x01 = x1[j1], x11 = x0[j1];
+        const float l0 = hl ? x1[j0 + wl] : 0.0f, l1 = hl ? x0[j1 + wl] : 0.0f;
+        const float r0 = hr ? x0[j0 + wr] : 0.0f, r1 = hr ? x1[j1 + wr] : 0.0f;
+        const float dl = (float)(1 + (le ? 1 : wx)), dr = (float)(1 + (re ? 1 : wx));
+        const float dd = (float)(1 + (de ? 1 : wy)), du = (float)(1 + (ue ? 1 : wy));
+        float s = b0[j0] - ((dl + dd) * x00 - (((l0 + x10) + x1[jd]) + x01));
+        s += b1[j0] - ((dr + dd) * x10 - (((x00 + r0) + x0[jd]) + x11));
+        s += b1[j1] - ((dl + du) * x01 - (((l1 + x11) + x00) + x0[ju]));
+        s += b0[j1] - ((dr + du) * x11 - (((x01 + r1) + x10) + x1[ju]));
+        bc[sm_pos(Cc, p)] = s;
+    }
+    part_bar(bar, nthr);
+}
+
+// The coarse correction (needed on colour 1 only: the first half sweep overwrites colour 0
+// without reading it) and the post-smoothing.
+template <int K>
+__device__ __forceinline__ void rb_up(const SmallDesc &D, const SmallLevel &L, const SmallLevel &Cc, float *sm, int bar) {
+    const int nthr = L.nthr, half = L.half, nxh = L.nx >> 1;
+    float *x0 = sm + L.off, *x1 = x0 + L.hs;
+    const float *b0 = x0 + L.boff, *b1 = b0 + L.hs;
+    const float *xc = sm + Cc.off;
+    RbCells<K> c;
+    float bb0[K], bb1[K];
+    rb_cells<K>(D, L, c);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int j = (int)threadIdx.x + nthr * k;
+        bb0[k] = bb1[k] = 0.0f;
+        if (j < half) {
+            bb0[k] = b0[j]; bb1[k] = b1[j];
+            const int iy = mdiv(j, L.nxh_magic), m = j - iy * nxh, cy = iy >> 1;
+            const int q = Cc.fast ? ((m + cy) & 1) * Cc.hs + cy * (nxh >> 1) + (m >> 1) : cy * nxh + m;
+            x1[j] += xc[q];
+        }
+    }
+    part_bar(bar, nthr);
+    for (int s = 0; s < kNu; ++s) {
+        rb_half<K>(x0, x1, c.oh0, c.od, c.ou, bb0, c.di0, nthr, half);
+        part_bar(bar, nthr);
+        rb_half<K>(x1, x0, c.oh1, c.od, c.ou, bb1, c.di1, nthr, half);
+        if (s + 1 < kNu) part_bar(bar, nthr);
+    }
 }
 
 // V-cycle over the shared-memory levels; b of the first level must be in place, x of the
-// first level holds the correction on return.
-__device__ void sm_vcycle(const SmallDesc &D, float *sm, bool singular, float *red) {
+// first level holds the correction on return (after a block barrier).  All 1024 threads call
+// it.  ELL levels are swept by the whole block; a level stored by colour by its nthr threads,
+// whose other warps wait at the next finer level's barrier (barrier ids count from the first
+// such level).  `inv` is the coarsest inverse (null: CG), `scr` kDirectN + 512 doubles.
+__device__ void sm_vcycle(const SmallDesc &D, float *sm, bool singular, float *red, const double *inv, double *scr) {
     const int last = D.nlev - 1;
-    for (int g = 0; g < last; ++g) {
+    int g = 0;
+    for (; g < last && !D.lv[g].fast; ++g) {
         const SmallLevel &L = D.lv[g], &Cc = D.lv[g + 1];
-        float *x = sm + L.off, *b = x + L.n;
+        float *x = sm + L.off, *b = x + L.boff;
         for (int k = 0; k < kNu; ++k) sm_smooth(D, L, x, b, k == 0);
-        float *bc = sm + Cc.off + Cc.n;
+        float *bc = sm + Cc.off + Cc.boff;
         for (int p = threadIdx.x; p < Cc.n; p += blockDim.x) {
             float s = 0.0f;
-            if (L.uniform && Cc.uniform) {
-                const int py = mdiv(p, Cc.nx_magic), px = p - py * Cc.nx;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int i = (2 * py + (k >> 1)) * L.nx + 2 * px + (k & 1);
-                    float d;
-                    const float sn = sm_row(D, L, x, i, d);
-                    s += b[i] - (d * x[i] - sn);
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int32_t i = Cc.child4[4 * p + k];
-                    if (i < 0) continue;
-                    float d;
-                    const float sn = sm_row(D, L, x, i, d);
-                    s += b[i] - (d * x[i] - sn);
-                }
+            for (int k = 0; k < 4; ++k) {
+                const int32_t i = Cc.child4[4 * p + k];
+                if (i < 0) continue;
+                float d;
+                const float sn = sm_row(D, L, x, i, d);
+                s += b[i] - (d * x[i] - sn);
             }
-            bc[p] = s;
+            bc[sm_pos(Cc, p)] = s;
         }
         __syncthreads();
     }
-    {
+    const int gf = g;
+    for (; g < last; ++g) {
+        const SmallLevel &L = D.lv[g], &Cc = D.lv[g + 1];
+        if ((int)threadIdx.x >= L.nthr) break;
+        if (L.kc == 1) rb_down<1>(D, L, Cc, sm, 1 + g - gf);
+        else if (L.kc == 2) rb_down<2>(D, L, Cc, sm, 1 + g - gf);
+        else rb_down<4>(D, L, Cc, sm, 1 + g - gf);
+    }
+    if (g == last) {
         const SmallLevel &L = D.lv[last];
-        float *x = sm + L.off, *b = x + L.n;
+        float *x = sm + L.off, *b = x + L.boff;
         float *r = sm + D.off_cg;
-        if (D.cinv) sm_coarse_direct(D, L, x, b, singular, red);
+        if (inv) sm_coarse_direct(L, inv, x, b, singular, last > gf ? D.lv[last - 1].nthr : 1024, 1 + last - gf, scr);
         else sm_coarse_cg(D, L, x, b, r, r + L.n, r + 2 * L.n, singular, red);
     }
-    for (int g = last - 1; g >= 0; --g) {
+    for (--g; g >= gf; --g) {
         const SmallLevel &L = D.lv[g], &Cc = D.lv[g + 1];
-        float *x = sm + L.off, *b = x + L.n;
+        part_bar(1 + g - gf, L.nthr);  // the coarser level's correction is complete
+        if (L.kc == 1) rb_up<1>(D, L, Cc, sm, 1 + g - gf);
+        else if (L.kc == 2) rb_up<2>(D, L, Cc, sm, 1 + g - gf);
+        else rb_up<4>(D, L, Cc, sm, 1 + g - gf);
+    }
+    if (gf > 0) __syncthreads();
+    for (g = gf - 1; g >= 0; --g) {
+        const SmallLevel &L = D.lv[g], &Cc = D.lv[g + 1];
+        float *x = sm + L.off, *b = x + L.boff;
         const float *xc = sm + Cc.off;
-        if (L.uniform && Cc.uniform) {
-            for (int i = threadIdx.x; i < L.n; i += blockDim.x) {
-                const int iy = mdiv(i, L.nx_magic), ix = i - iy * L.nx;
-                x[i] += xc[(iy >> 1) * Cc.nx + (ix >> 1)];
-            }
-        } else {
-            for (int i = threadIdx.x; i < L.n; i += blockDim.x) x[i] += xc[L.parent[i]];
-        }
+        for (int i = threadIdx.x; i < L.n; i += blockDim.x) x[i] += xc[sm_pos(Cc, L.parent[i])];
         __syncthreads();
         for (int k = 0; k < kNu; ++k) sm_smooth(D, L, x, b, false);
     }
 }
 
 // Tail of a V-cycle started by the multi-block levels: b from global, x back to global.
-__global__ void __launch_bounds__(1024, 1) k_tail_vcycle(SmallDesc D, const float *__restrict__ gb,
-                                                       float *__restrict__ gx, int singular) {
-    pdl_chain();
-    extern __shared__ float sm[];
+__global__ void __launch_bounds__(1024, 1) k_tail_vcycle(const __grid_constant__ SmallDesc Dp,
+                                                       const float *__restrict__ gb, float *__restrict__ gx,
+                                                       int singular) {
+    extern __shared__ __align__(16) float sm[];
     __shared__ float redf[33];
-    const SmallLevel &L = D.lv[0];
-    for (int i = threadIdx.x; i < L.n; i += blockDim.x) sm[L.off + L.n + i] = gb[i];
+    __shared__ double scr[kDirectN + 512];
+    __shared__ SmallDesc D;
+    // constant data before the wait for the kernel before this one
+    for (int k = threadIdx.x; k < (int)(sizeof(SmallDesc) / 4); k += 1024)
+        reinterpret_cast<uint32_t *>(&D)[k] = reinterpret_cast<const uint32_t *>(&Dp)[k];
     __syncthreads();
-    sm_vcycle(D, sm, singular != 0, redf);
-    for (int i = threadIdx.x; i < L.n; i += blockDim.x) gx[i] = sm[L.off + i];
+    const double *inv = D.cinv;
+    if (D.inv_words) {
+        double *cs = reinterpret_cast<double *>(sm + D.smem_floats);
+        for (int k = threadIdx.x; k < D.inv_words; k += 1024) cs[k] = inv[k];
+        inv = cs;
+    }
+    pdl_chain();
+    const SmallLevel &L = D.lv[0];
+    for (int i = threadIdx.x; i < L.n; i += blockDim.x) sm[L.off + L.boff + sm_pos(L, i)] = gb[i];
+    __syncthreads();
+    sm_vcycle(D, sm, singular != 0, redf, inv, scr);
+    __syncthreads();
+    for (int i = threadIdx.x; i < L.n; i += blockDim.x) gx[i] = sm[L.off + sm_pos(L, i)];
 }
-
 
 // FP64 sums over the cells of a small solve that come out the same whatever the number C of
 // CTAs in the instance's cluster: chunk c (cells 1024 c .. 1024 c + 1023) is summed by CTA
-// c mod C as a fixed tree (warp shuffles, then the 32 warp sums in order), and the chunk
-// sums by the leader CTA in chunk order.  f(i, a, b) adds cell i's terms to a and b; every
-// thread of the cluster receives both totals.  Collective over the cluster.
+// c mod C as a fixed tree into four words part[4 c .. 4 c + 3] of the leader's shared memory,
+// and small_total adds the (at most 32) words as a fixed tree.  f(i) is cell i's term.  A
+// chunk's terms go through shared memory and 128 threads add eight each before any shuffle:
+// 52 FP64 warp instructions per chunk instead of the 160 of a shuffle tree in every warp (the
+// FP64 pipe takes 16 clocks for each).
 constexpr int kSmallChunks = kSmallN / 1024;
 template <typename F>
-__device__ void cl_sums(cooperative_groups::cluster_group &cl, int C, int rank, int n, double *wsum, double *lpart,
-                        double *louts, F f, double &s0, double &s1) {
+__device__ __forceinline__ void small_sums(int C, int rank, int n, double *vbuf, int nbuf, double *part, F f) {
     const int nch = (n + 1023) >> 10;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int c = rank; c < nch; c += C) {
-        const int i = (c << 10) + (int)threadIdx.x;
-        double a = 0.0, b = 0.0;
-        if (i < n) f(i, a, b);
+    const int nq = rank < nch ? (nch - rank + C - 1) / C : 0;  // this CTA's chunks
+    const int u = threadIdx.x & 127;
+    for (int q0 = 0; q0 < nq; q0 += nbuf) {
+        const int m = min(nbuf, nq - q0);
+        if (q0) __syncthreads();
+        for (int q = 0; q < m; ++q) {
+            const int i = ((rank + (q0 + q) * C) << 10) + (int)threadIdx.x;
+            vbuf[1024 * q + threadIdx.x] = i < n ? f(i) : 0.0;
+        }
+        __syncthreads();
+        for (int q = threadIdx.x >> 7; q < m; q += 8) {
+            double s = vbuf[1024 * q + u];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_down_sync(0xFFFFFFFFu, a, o);
-            b += __shfl_down_sync(0xFFFFFFFFu, b, o);
+            for (int k = 1; k < 8; ++k) s += vbuf[1024 * q + u + 128 * k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, o);
+            if ((u & 31) == 0) part[4 * (rank + (q0 + q) * C) + (u >> 5)] = s;
         }
-        if (lane == 0) { wsum[wid] = a; wsum[32 + wid] = b; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double x = 0.0, y = 0.0;
-            for (int w = 0; w < 32; ++w) { x += wsum[w]; y += wsum[32 + w]; }
-            lpart[2 * c] = x;
-            lpart[2 * c + 1] = y;
-        }
-        __syncthreads();
     }
-    cl.sync();
-    if (rank == 0 && threadIdx.x == 0) {
-        double x = 0.0, y = 0.0;
-        for (int c = 0; c < nch; ++c) { x += lpart[2 * c]; y += lpart[2 * c + 1]; }
-        louts[0] = x;
-        louts[1] = y;
-    }
-    cl.sync();
-    s0 = louts[0];
-    s1 = louts[1];
+}
+// The total of a sum's words, on every lane of the calling warp of the leader CTA.
+__device__ __forceinline__ double small_total(const double *part, int n) {
+    const int lane = threadIdx.x & 31;
+    double s = lane < 4 * ((n + 1023) >> 10) ? part[lane] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+    return s;
 }
 
 // Whole solve for a mesh whose every level fits: FP64 residual and correction, FP32 V-cycles
-// in shared memory, convergence test on the device.  One cluster of C CTAs per item (C = 1
-// for a batch of instances, one launch for all; up to 8 for an instance alone): the leader
+// in shared memory, convergence test on the device.  One cluster of C CTAs per item: the leader
 // CTA holds the levels and runs the V-cycles, and the FP64 work (warm start, residual,
 // correction, norms) is split by chunks of 1024 cells over the cluster, each CTA writing its
 // chunks' FP32 residual straight into the leader's shared memory.  GB300's FP64 rate per SM
-// is low, so spreading it over the cluster's SMs is what bounds the solve.  The result does
-// not depend on C.  stats: [cycles, rel. residual, max rel. since reset].
+// is low (two lanes a clock), so a cycle's FP64 work (7 operations per cell and the norm) is
+// spread over the cluster's SMs.  A cycle crosses three cluster barriers: residual and norm
+// words with the leader; correction (or the decision to stop) with the others; potential
+// complete.  The result does not depend on C.  stats: [cycles, rel. residual, max rel. since
+// reset].
 struct SmallSolve {
     SmallDesc D;
     const double *diag64, *val64;
@@ -779,19 +927,31 @@ struct SmallSolve {
     double tol;
 };
 
-__global__ void __launch_bounds__(1024, 1) k_small_solve(const SmallSolve *__restrict__ items) {
+// `nbuf`: chunk buffers of the sums that fit behind every item's levels.
+__global__ void __launch_bounds__(1024, 1) k_small_solve(const SmallSolve *__restrict__ items, int nbuf) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
-    extern __shared__ float sm[];
+    extern __shared__ __align__(16) float sm[];
     __shared__ float redf[33];
     __shared__ SmallDesc D;
-    __shared__ double wsum[64], part[2 * kSmallChunks], outs[2];
+    __shared__ double part[64], outs[2];
+    __shared__ double rel_sh;
+    __shared__ int stop_sh;
     const SmallSolve &it = items[blockIdx.x / C];
-    if (threadIdx.x == 0) D = it.D;
+    for (int k = threadIdx.x; k < (int)(sizeof(SmallDesc) / 4); k += 1024)
+        reinterpret_cast<uint32_t *>(&D)[k] = reinterpret_cast<const uint32_t *>(&it.D)[k];
     __syncthreads();
+    double *vbuf = reinterpret_cast<double *>(sm + D.smem_floats);
+    const double *inv = D.cinv;
+    if (rank == 0 && D.inv_words) {
+        double *cs = vbuf + 1024 * nbuf;
+        for (int k = threadIdx.x; k < D.inv_words; k += 1024) cs[k] = inv[k];
+        inv = cs;
+    }
     float *lsm = cl.map_shared_rank(sm, 0);  // the leader's levels
     double *lpart = cl.map_shared_rank(part, 0), *louts = cl.map_shared_rank(outs, 0);
+    const int *lstop = cl.map_shared_rank(&stop_sh, 0);
     const double *__restrict__ diag64 = it.diag64;
     const double *__restrict__ val64 = it.val64;
     double *phi = it.phi;
@@ -804,44 +964,45 @@ __global__ void __launch_bounds__(1024, 1) k_small_solve(const SmallSolve *__res
 #define CL_FOR(i)                                                                    \
     for (int c_ = rank; c_ < nch; c_ += C)                                           \
         for (int i = (c_ << 10) + (int)threadIdx.x; i < n && i < ((c_ + 1) << 10); i += 1 << 30)
-    {
-        const int ns = *it.n_solves;
-        if (ns >= 1)
-            CL_FOR(i) {
-                const double p = phi[i];
-                if (ns >= 2) phi[i] = 2.0 * p - it.phi_prev[i];
-                it.phi_prev[i] = p;
-            }
-        cl.sync();  // every CTA has read the counter and its chunks of phi
-        if (rank == 0 && threadIdx.x == 0) *it.n_solves = ns + 1;
-    }
-    if (singular) {  // right-hand side compatibility: remove an area-proportional share
-        double sb, sa;
-        cl_sums(cl, C, rank, n, wsum, lpart, louts, [&](int i, double &a, double &b) {
-            const double s = (double)(1 << (lmax - lev[i]));
-            a += bvec[i];
-            b += s * s;
-        }, sb, sa);
-        CL_FOR(i) {
-            const double s = (double)(1 << (lmax - lev[i]));
-            bvec[i] -= sb / sa * s * s;
+    // two sums over all cells, known to every thread of the cluster
+    auto area = [&](int i) { const double s = (double)(1 << (lmax - lev[i])); return s * s; };
+    auto moments = [&](auto f, double &s0, double &s1) {
+        small_sums(C, rank, n, vbuf, nbuf, lpart, f);
+        __syncthreads();
+        small_sums(C, rank, n, vbuf, nbuf, lpart + 32, area);
+        cl.sync();
+        if (rank == 0 && threadIdx.x < 32) {
+            const double a = small_total(part, n), b = small_total(part + 32, n);
+            if (threadIdx.x == 0) { outs[0] = a; outs[1] = b; }
         }
         cl.sync();
+        s0 = louts[0];
+        s1 = louts[1];
+    };
+    const int ns = *it.n_solves;
+    if (ns >= 1)
+        CL_FOR(i) {
+            const double p = phi[i];
+            if (ns >= 2) phi[i] = 2.0 * p - it.phi_prev[i];
+            it.phi_prev[i] = p;
+        }
+    if (singular) {  // right-hand side compatibility: remove an area-proportional share
+        double sb, sa;
+        moments([&](int i) { return bvec[i]; }, sb, sa);
+        const double k = sb / sa;
+        CL_FOR(i) bvec[i] -= k * area(i);
     }
-    double bb, unused;
-    cl_sums(cl, C, rank, n, wsum, lpart, louts, [&](int i, double &a, double &) { a += bvec[i] * bvec[i]; }, bb,
-            unused);
-    float *b0 = lsm + L.off + n, *x0 = lsm + L.off;
-    int cyc = 0;
-    double rel = 0.0;
-    for (;;) {
-        double rr;
-        cl_sums(cl, C, rank, n, wsum, lpart, louts, [&](int i, double &a, double &) {
+    small_sums(C, rank, n, vbuf, nbuf, lpart + 32, [&](int i) { return bvec[i] * bvec[i]; });
+    cl.sync();  // every CTA has read the counter; phi is complete
+    if (rank == 0 && threadIdx.x == 0) *it.n_solves = ns + 1;
+    float *lb = lsm + L.off + L.boff, *lx = lsm + L.off;
+    for (int cyc = 0;; ++cyc) {
+        small_sums(C, rank, n, vbuf, nbuf, lpart, [&](int i) {
             double ax;
             if (L.uniform) {
-                double d;
-                const double sn = uni_row<double>(L.nx, L.ny, L.nx_magic, D.bcx, D.bcy, phi, i, d);
-                ax = d * phi[i] - sn;
+                int dd;
+                const double sn = uni_row<double>(L.nx, L.ny, L.nx_magic, D.bcx, D.bcy, phi, i, dd);
+                ax = (dd == 4 ? 4.0 : (double)dd) * phi[i] - sn;
             } else {
                 ax = diag64[i] * phi[i];
 #pragma unroll
@@ -851,70 +1012,86 @@ __global__ void __launch_bounds__(1024, 1) k_small_solve(const SmallSolve *__res
                 }
             }
             const double ri = bvec[i] - ax;
-            b0[i] = (float)ri;
-            a += ri * ri;
-        }, rr, unused);
-        rel = bb > 0.0 ? sqrt(rr / bb) : sqrt(rr);
-        if (rel <= tol || (bb == 0.0 && rr == 0.0) || cyc >= maxc) break;
-        if (rank == 0) sm_vcycle(D, sm, singular != 0, redf);
-        cl.sync();  // the correction is in the leader's x0
-        CL_FOR(i) phi[i] += (double)x0[i];
-        cl.sync();  // phi complete before the next residual (and x0 read before the next V-cycle)
-        if (singular) {
-            double sv, sa;
-            cl_sums(cl, C, rank, n, wsum, lpart, louts, [&](int i, double &a, double &b) {
-                const double s = (double)(1 << (lmax - lev[i]));
-                a += s * s * phi[i];
-                b += s * s;
-            }, sv, sa);
-            CL_FOR(i) phi[i] -= sv / sa;
-            cl.sync();
+            lb[sm_pos(L, i)] = (float)ri;
+            return ri * ri;
+        });
+        cl.sync();
+        if (rank == 0) {
+            if (threadIdx.x < 32) {
+                const double rr = small_total(part, n), bb = small_total(part + 32, n);
+                if (threadIdx.x == 0) {
+                    const double rel = bb > 0.0 ? sqrt(rr / bb) : sqrt(rr);
+                    rel_sh = rel;
+                    stop_sh = rel <= tol || (bb == 0.0 && rr == 0.0) || cyc >= maxc;
+                    if (stop_sh) {
+                        it.stats[0] = (double)cyc;
+                        it.stats[1] = rel;
+                        it.stats[2] = worst_residual(it.stats[2], rel);
+                    }
+                }
+            }
+            __syncthreads();
+            if (!stop_sh) sm_vcycle(D, sm, singular != 0, redf, inv, vbuf);
         }
-        ++cyc;
+        cl.sync();  // the correction is in the leader's x
+        if (*lstop) break;
+        CL_FOR(i) phi[i] += (double)lx[sm_pos(L, i)];
+        cl.sync();  // phi complete before the next residual (and x read before the next V-cycle)
+    }
+    if (singular) {  // zero area-weighted mean (a constant changes no residual)
+        double sv, sa;
+        moments([&](int i) { return area(i) * phi[i]; }, sv, sa);
+        const double k = sv / sa;
+        CL_FOR(i) phi[i] -= k;
     }
 #undef CL_FOR
-    if (rank == 0 && threadIdx.x == 0) {
-        it.stats[0] = (double)cyc;
-        it.stats[1] = rel;
-        it.stats[2] = worst_residual(it.stats[2], rel);
-    }
+    cl.sync();  // the leader's shared memory outlives every read of it
 }
 
-// One launch of the small solve: n_items clusters of C CTAs.
-void launch_small_solve(const void *items, int n_items, int C, size_t smem, cudaStream_t st) {
+// A solve's shared memory holds the levels and the coarsest inverse (lv_bytes) and, per chunk of
+// a CTA, one 8 KB buffer of the sums (as many as fit, at least one).
+int small_bufs(int n, int C, size_t lv_bytes) {
+    const int nch = (n + 1023) / 1024;
+    return std::max(1, std::min((nch + C - 1) / C, ((int)kSmallSmemMax - (int)lv_bytes) / 8192));
+}
+
+cudaLaunchConfig_t small_config(int n_items, int C, size_t smem, cudaLaunchAttribute *attr) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(n_items * C));
     cfg.blockDim = dim3(1024);
     cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)C;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    GB_CUDA(cudaLaunchKernelEx(&cfg, k_small_solve, (const SmallSolve *)items));
+    return cfg;
 }
 
-// The cluster size for an instance solved alone: one CTA per 1024-cell chunk, at most 8,
-// reduced until the GPU can hold such a cluster.
-int small_cluster(int n, size_t smem) {
-    int C = std::min(8, std::max(1, (n + 1023) / 1024));
+// One launch of the small solve: n_items clusters of C CTAs.
+void launch_small_solve(const void *items, int n_items, int C, int nbuf, size_t smem, cudaStream_t st) {
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = small_config(n_items, C, smem, attr);
+    cfg.stream = st;
+    GB_CUDA(cudaLaunchKernelEx(&cfg, k_small_solve, (const SmallSolve *)items, nbuf));
+}
+
+// The cluster size for n_items instances solved in one launch: one CTA per 1024-cell chunk of
+// the largest, at most 8, as many as the GPU's SMs hold side by side (a CTA fills an SM),
+// reduced until the GPU can hold such clusters.  32 instances of up to 8192 cells: 0.61 ms with
+// one CTA each and the old sweeps, 0.133 ms with 4.
+int small_cluster(int n, int n_items, size_t lv_bytes) {
+    int sms = 0, dev = 0;
+    GB_CUDA(cudaGetDevice(&dev));
+    GB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    int C = 1;
+    while (2 * C <= std::min(8, (n + 1023) / 1024) && 2 * C * n_items <= sms) C *= 2;
     for (; C > 1; C >>= 1) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)C);
-        cfg.blockDim = dim3(1024);
-        cfg.dynamicSmemBytes = smem;
         cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)C;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
+        cudaLaunchConfig_t cfg = small_config(n_items, C, lv_bytes + (size_t)small_bufs(n, C, lv_bytes) * 8192, attr);
         int nc = 0;
-        if (cudaOccupancyMaxActiveClusters(&nc, k_small_solve, &cfg) == cudaSuccess && nc >= 1) break;
+        if (cudaOccupancyMaxActiveClusters(&nc, k_small_solve, &cfg) == cudaSuccess && nc >= n_items) break;
         cudaGetLastError();
     }
     return C;
@@ -926,7 +1103,7 @@ int small_from(const Instance &in) {
     int64_t floats = 0;
     for (int g = (int)in.lv.size() - 1; g >= 0; --g) {
         const Level &L = in.lv[g];
-        const int64_t add = 2 * L.n + (g == (int)in.lv.size() - 1 ? 3 * L.n + 8 : 0);
+        const int64_t add = 2 * L.n + 16 + (g == (int)in.lv.size() - 1 ? 3 * L.n + 8 : 0);
         if (L.n > kSmallN || (int)in.lv.size() - g > kMaxSmallLevels || (floats + add) * 4 > kSmallSmemCap) break;
         floats += add;
         g0 = g;
@@ -957,12 +1134,23 @@ SmallDesc small_desc(const Instance &in, int g0) {
         for (int64_t i = 0; i < L.n; ++i)
             if (q(i, S.nx_magic) != i / L.nx0 || q(i, S.nxh_magic) != i / (int64_t)nxh)
                 fail(PIC_EINVAL, "index division check failed");
-        off += 2 * (int32_t)L.n;
+        S.fast = S.uniform && k + 1 < D.nlev ? 1 : 0;  // (such a level coarsens: nx and ny are even)
+        S.half = (int32_t)L.n / 2;
+        S.hs = S.half + 4;
+        S.boff = S.fast ? 2 * S.hs : (int32_t)L.n;
+        // at least 8 warps (the coarsest solve runs on the last level's), every warp when the
+        // coarsest level is solved by CG, which uses the whole block
+        S.nthr = in.coarse_inv ? std::min(1024, std::max(256, (S.half + 31) / 32 * 32)) : 1024;
+        const int kc = (S.half + S.nthr - 1) / S.nthr;
+        S.kc = kc > 2 ? 4 : kc;
+        off += S.fast ? 4 * S.hs : 2 * (int32_t)L.n;
     }
     D.off_cg = off;
     off += 3 * (int32_t)in.lv.back().n + 8;
-    D.smem_floats = off;
+    D.smem_floats = (off + 3) & ~3;
     D.cinv = in.coarse_inv;
+    const int64_t words = in.lv.back().n * in.lv.back().n;
+    D.inv_words = D.cinv && (int64_t)D.smem_floats * 4 + words * 8 + 8192 <= kSmallSmemMax ? (int32_t)words : 0;
     return D;
 }
 
@@ -972,7 +1160,7 @@ void vcycle(pic_ctx *ctx, Instance &in, size_t g, bool singular) {
     const int g0 = small_from(in);
     if ((int)g >= g0) {
         const SmallDesc D = small_desc(in, (int)g);
-        const size_t bytes = (size_t)D.smem_floats * 4;
+        const size_t bytes = (size_t)D.smem_floats * 4 + (size_t)D.inv_words * 8;
         pdl(k_tail_vcycle, 1, 1024, bytes, s, D, L.b, L.x, singular);
         count_launch(ctx);
         return;
@@ -1012,46 +1200,30 @@ void vcycle(pic_ctx *ctx, Instance &in, size_t g, bool singular) {
 }  // namespace
 
 namespace {
-constexpr int kDirectN = 64;  // coarsest levels up to this size are solved by a dense inverse
-
-// Dense inverse of the coarsest level's operator as the shared-memory V-cycle applies it
-// (uniform levels: the 5-point stencil with the wall rules; otherwise the ELL rows with the
-// diagonal 1 / dinv rounded to FP32), plus 1 1^T / n when the mesh is periodic in both
-// directions.  Gauss-Jordan with partial pivoting in FP64; null (the CG is used) for a
-// level larger than kDirectN cells or a singular matrix.
+// Dense inverse of the coarsest level's operator (a uniform grid of root boxes: the 5-point
+// stencil with the wall rules), plus 1 1^T / n when the mesh is periodic in both directions.
+// Gauss-Jordan with partial pivoting in FP64, made symmetric (the solve reads columns as rows);
+// null (the CG is used) for a level larger than kDirectN cells or a singular matrix.  It depends
+// on the root grid and the walls only, so an adaptation keeps it.
 double *coarse_inverse(pic_ctx *ctx, Instance &in, bool singular) {
     const Level &L = in.lv.back();
     const int n = (int)L.n;
     if (n > kDirectN || n < 1) return nullptr;
+    const std::array<int, 4> key = {L.nx0, L.ny0, in.cfg.bc_x, in.cfg.bc_y};
+    if (in.coarse_inv_key == key) return in.coarse_inv_mem;
     std::vector<double> A((size_t)n * n, 0.0);
     auto at = [&](int i, int j) -> double & { return A[(size_t)i * n + j]; };
-    if (L.lmax == 0) {
-        const int nx = L.nx0, ny = L.ny0, bx = in.cfg.bc_x, by = in.cfg.bc_y;
-        for (int i = 0; i < n; ++i) {
-            const int ix = i % nx, iy = i / nx;
-            auto face = [&](bool inside, int j, int bc) {
-                if (inside || bc == PIC_BC_PERIODIC) { at(i, j) -= 1.0; at(i, i) += 1.0; }
-                else if (bc == PIC_BC_DIRICHLET) at(i, i) += 2.0;
-            };
-            face(ix > 0, ix > 0 ? i - 1 : i + nx - 1, bx);
-            face(ix < nx - 1, ix < nx - 1 ? i + 1 : i - nx + 1, bx);
-            face(iy > 0, iy > 0 ? i - nx : i + (ny - 1) * nx, by);
-            face(iy < ny - 1, iy < ny - 1 ? i + nx : i - (ny - 1) * nx, by);
-        }
-    } else {
-        std::vector<int32_t> col((size_t)kEll * n);
-        std::vector<float> val((size_t)kEll * n), dinv(n);
-        GB_CUDA(cudaMemcpyAsync(col.data(), L.col, col.size() * 4, cudaMemcpyDeviceToHost, ctx->stream));
-        GB_CUDA(cudaMemcpyAsync(val.data(), L.val, val.size() * 4, cudaMemcpyDeviceToHost, ctx->stream));
-        GB_CUDA(cudaMemcpyAsync(dinv.data(), L.dinv, dinv.size() * 4, cudaMemcpyDeviceToHost, ctx->stream));
-        GB_CUDA(cudaStreamSynchronize(ctx->stream));
-        for (int i = 0; i < n; ++i) {
-            at(i, i) += (double)(1.0f / dinv[i]);
-            for (int j = 0; j < kEll; ++j) {
-                const int32_t c = col[(size_t)j * n + i];
-                if (c >= 0) at(i, c) += (double)val[(size_t)j * n + i];
-            }
-        }
+    const int nx = L.nx0, ny = L.ny0, bx = in.cfg.bc_x, by = in.cfg.bc_y;
+    for (int i = 0; i < n; ++i) {
+        const int ix = i % nx, iy = i / nx;
+        auto face = [&](bool inside, int j, int bc) {
+            if (inside || bc == PIC_BC_PERIODIC) { at(i, j) -= 1.0; at(i, i) += 1.0; }
+            else if (bc == PIC_BC_DIRICHLET) at(i, i) += 2.0;
+        };
+        face(ix > 0, ix > 0 ? i - 1 : i + nx - 1, bx);
+        face(ix < nx - 1, ix < nx - 1 ? i + 1 : i - nx + 1, bx);
+        face(iy > 0, iy > 0 ? i - nx : i + (ny - 1) * nx, by);
+        face(iy < ny - 1, iy < ny - 1 ? i + nx : i - (ny - 1) * nx, by);
     }
     if (singular)
         for (double &a : A) a += 1.0 / n;
@@ -1082,10 +1254,16 @@ double *coarse_inverse(pic_ctx *ctx, Instance &in, bool singular) {
             }
         }
     }
-    double *d = dalloc<double>(in.mesh_mem, Inv.size());
-    GB_CUDA(cudaMemcpyAsync(d, Inv.data(), Inv.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
+    for (int i = 0; i < n; ++i)
+        for (int j = 0; j < i; ++j) {
+            const double m = 0.5 * (Inv[(size_t)i * n + j] + Inv[(size_t)j * n + i]);
+            Inv[(size_t)i * n + j] = Inv[(size_t)j * n + i] = m;
+        }
+    if (!in.coarse_inv_mem) in.coarse_inv_mem = dalloc<double>(in.inv_mem, kDirectN * kDirectN);
+    GB_CUDA(cudaMemcpyAsync(in.coarse_inv_mem, Inv.data(), Inv.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
     GB_CUDA(cudaStreamSynchronize(ctx->stream));
-    return d;
+    in.coarse_inv_key = key;
+    return in.coarse_inv_mem;
 }
 }  // namespace
 
@@ -1094,8 +1272,9 @@ void poisson_setup(pic_ctx *ctx, Instance &in) {
         cudaGraphExecDestroy(in.mg_cycle);
         in.mg_cycle = nullptr;
     }
-    GB_CUDA(cudaFuncSetAttribute(k_tail_vcycle, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmemCap));
-    GB_CUDA(cudaFuncSetAttribute(k_small_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmemCap));
+    // (the tail has no sums' buffers, and more static shared memory)
+    GB_CUDA(cudaFuncSetAttribute(k_tail_vcycle, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmemMax - 8192));
+    GB_CUDA(cudaFuncSetAttribute(k_small_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmemMax));
     DeviceArena &A = in.mesh_mem;
     const int64_t n = in.lv[0].n;
     in.phi = dalloc<double>(A, n);
@@ -1138,8 +1317,8 @@ void poisson_setup(pic_ctx *ctx, Instance &in) {
         GB_CUDA(cudaMemcpyAsync(d, &it, sizeof(SmallSolve), cudaMemcpyHostToDevice, ctx->stream));
         GB_CUDA(cudaStreamSynchronize(ctx->stream));
         in.small_item = d;
-        in.small_smem = (size_t)it.D.smem_floats * 4;
-        in.small_cluster = small_cluster((int)L.n, in.small_smem);
+        in.small_smem = (size_t)it.D.smem_floats * 4 + (size_t)it.D.inv_words * 8;
+        in.small_cluster = small_cluster((int)L.n, 1, in.small_smem);
     }
     ++ctx->mesh_epoch;
 }
@@ -1154,7 +1333,6 @@ void poisson_reset_warm_start(pic_ctx *ctx, Instance &in) {
     if (in.d_n_solves) GB_CUDA(cudaMemsetAsync(in.d_n_solves, 0, 4, ctx->stream));
 }
 
-// One launch for every instance whose mesh fits one block: block b solves instance b.
 // The batched solver's item table for `list` (copies issued on the context's stream, so a
 // step captured afterwards finds the table current and captures no copy).
 void poisson_batch_items(pic_ctx *ctx, const std::vector<Instance *> &list) {
@@ -1162,9 +1340,11 @@ void poisson_batch_items(pic_ctx *ctx, const std::vector<Instance *> &list) {
         ctx->batch_mem.release_all();
         ctx->batch_items = ctx->batch_mem.alloc(list.size() * sizeof(SmallSolve));
         ctx->batch_smem = 0;
-        // largest meshes first: the blocks start in this order, one per SM (each reserves the
-        // largest instance's shared memory), so the longest solves begin in the first wave
-        // and the short ones fill in behind them (every item writes only its own instance)
+        ctx->batch_cells = 0;
+        // largest meshes first: the clusters start in this order (a CTA reserves the largest
+        // instance's shared memory, so it has an SM to itself), so the longest solves begin in
+        // the first wave and the short ones fill in behind them (every item writes only its
+        // own instance)
         std::vector<size_t> order(list.size());
         for (size_t k = 0; k < order.size(); ++k) order[k] = k;
         std::stable_sort(order.begin(), order.end(),
@@ -1173,7 +1353,9 @@ void poisson_batch_items(pic_ctx *ctx, const std::vector<Instance *> &list) {
             GB_CUDA(cudaMemcpyAsync((SmallSolve *)ctx->batch_items + k, list[order[k]]->small_item, sizeof(SmallSolve),
                                     cudaMemcpyDeviceToDevice, ctx->stream));
             ctx->batch_smem = std::max(ctx->batch_smem, list[order[k]]->small_smem);
+            ctx->batch_cells = std::max(ctx->batch_cells, (int)list[order[k]]->lv[0].n);
         }
+        ctx->batch_cluster = small_cluster(ctx->batch_cells, (int)list.size(), ctx->batch_smem);
         ctx->batch_epoch = ctx->mesh_epoch;
         ctx->batch_n = (int)list.size();
     }
@@ -1186,7 +1368,9 @@ void poisson_solve_batch(pic_ctx *ctx, const std::vector<Instance *> &list, cons
         for (int w = 0; w < 4; ++w) list[k]->last_walls[w] = walls[k][w];
         list[k]->mg_on_device = true;
     }
-    launch_small_solve(ctx->batch_items, (int)list.size(), 1, ctx->batch_smem, ctx->stream);
+    const int nbuf = small_bufs(ctx->batch_cells, ctx->batch_cluster, ctx->batch_smem);
+    launch_small_solve(ctx->batch_items, (int)list.size(), ctx->batch_cluster, nbuf, ctx->batch_smem + (size_t)nbuf * 8192,
+                       ctx->stream);
     count_launch(ctx);
     check_launch("poisson_solve_batch");
 }
@@ -1199,7 +1383,8 @@ void poisson_solve(pic_ctx *ctx, Instance &in, const double walls[4]) {
     const int64_t n = L.n;
     const bool singular = in.cfg.bc_x == PIC_BC_PERIODIC && in.cfg.bc_y == PIC_BC_PERIODIC;
     if (in.small_item) {
-        launch_small_solve(in.small_item, 1, in.small_cluster, (size_t)in.small_smem, s);
+        const int nbuf = small_bufs((int)n, in.small_cluster, in.small_smem);
+        launch_small_solve(in.small_item, 1, in.small_cluster, nbuf, in.small_smem + (size_t)nbuf * 8192, s);
         count_launch(ctx);
         check_launch("poisson_solve");
         in.mg_on_device = true;
