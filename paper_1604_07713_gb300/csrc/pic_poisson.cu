@@ -398,7 +398,7 @@ struct SmallLevel {
     uint32_t nx_magic;   // floor(i / nx) == mdiv(i, nx_magic) for every cell index i < n
     uint32_t nxh_magic;  // the same for nx / 2 (uniform levels with even nx)
     int32_t fast, half, hs;  // stored by colour: cells per colour, stride between the colours (half + 4)
-    int32_t nthr, kc;        // threads that sweep the level, cells of each colour per thread (1, 2 or 4)
+    int32_t nthr, rows, strips;  // threads of the level, rows of a strip (2 or 4), strips per thread
 };
 struct SmallDesc {
     int nlev;  // levels g0 .. g0 + nlev - 1 live in shared memory
@@ -623,9 +623,14 @@ __device__ void sm_coarse_direct(const SmallLevel &L, const double *inv, float *
     const int part = t / n32, r = t - part * n32;
     if (part < parts && r < n) {
         const int per = (n + parts - 1) / parts, c1 = min(n, (part + 1) * per);
-        double acc = 0.0;
-        for (int c = part * per; c < c1; ++c) acc = fma(inv[c * n + r], scr[c], acc);
-        ps[part * n32 + r] = acc;
+        double a0 = 0.0, a1 = 0.0;  // two chains: a dependent FP64 operation takes tens of clocks
+        int c = part * per;
+        for (; c + 1 < c1; c += 2) {
+            a0 = fma(inv[c * n + r], scr[c], a0);
+            a1 = fma(inv[(c + 1) * n + r], scr[c + 1], a1);
+        }
+        if (c < c1) a0 = fma(inv[c * n + r], scr[c], a0);
+        ps[part * n32 + r] = a0 + a1;
     }
     part_bar(bar, nthr);
     if (part == 0) {
@@ -637,145 +642,177 @@ __device__ void sm_coarse_direct(const SmallLevel &L, const double *inv, float *
             m /= (double)n;
         }
         if (r < n) {
-            double acc = ps[r];
-            for (int p = 1; p < parts; ++p) acc += ps[p * n32 + r];
-            x[r] = (float)(acc - m);
+            double a0 = ps[r], a1 = 0.0;
+            int p = 1;
+            for (; p + 1 < parts; p += 2) { a0 += ps[p * n32 + r]; a1 += ps[(p + 1) * n32 + r]; }
+            if (p < parts) a0 += ps[p * n32 + r];
+            x[r] = (float)((a0 + a1) - m);
         }
     }
 }
 
 // ---- levels stored by colour --------------------------------------------------------------
-// Thread t sweeps the positions j = t + nthr k (k < K) of both colours.  The horizontal
-// neighbours of the cell at position j of one colour sit at j and at one of j - 1, j + 1 of the
-// other colour, the vertical ones at j - nx/2 and j + nx/2; a missing neighbour points to the
-// zero word at `half`.  The offsets and the reciprocal diagonals of a thread's cells are formed
-// once per leg and serve its four half sweeps, each of which costs 5 shared loads, 4 adds, a
-// multiply and one store per cell and one barrier (a colour reads only the other colour, so
-// values are updated in place).
+// A strip is one position m of a row and the K rows (K even) from an even one on: 2 K cells, two
+// in each row, held by one thread (S strips per thread).  In an even row colour 0 is at ix = 2 m
+// and colour 1 at 2 m + 1, in an odd row the other way round, so a cell's horizontal neighbours
+// are the strip's other cell of its row and one word of a neighbouring strip, and its vertical
+// neighbours are the strip's own cells except above and below it: K + 2 shared loads per half
+// sweep of K cells instead of 4 K.  A colour reads only the other colour, so values are updated
+// in place and one barrier ends a half sweep.  A missing neighbour is the zero word at `half`.
 //
-// What bounds the solve is this serial chain of half sweeps.  512 x 16 cells, 4 cycles: 0.283 ms
-// when each cell's index division and wall tests were done in every half sweep and two barriers
-// ended it, 0.118 ms so (with the FP64 sums of small_sums and the three cluster barriers of
-// k_small_solve); 64 x 64 periodic, 7 cycles: 0.508 and 0.170 ms.
-template <int K> struct RbCells {
-    int oh0[K], oh1[K], od[K], ou[K];
-    float di0[K], di1[K];
+// What bounds the solve is this serial chain of half sweeps; with four cells per thread the
+// finest level's is bound by shared-memory words.  512 x 16 cells, 4 cycles: 0.283 ms when each
+// cell's index division and wall tests were done in every half sweep and two barriers ended it,
+// 0.118 ms with the neighbour offsets formed once per leg (4 K loads), 0.105 ms so.
+template <int K, int S> struct RbStrips {
+    int j[S];            // position of the first row
+    int l[S], sl[S];     // word left of it and the step to the next row's (0: missing)
+    int r[S], sr[S];     // the same to the right
+    int dn[S], up[S];    // words below the first and above the last row
+    float di0[S][K], di1[S][K];  // reciprocal diagonals of the two colours
+    float b0[S][K], b1[S][K];    // right-hand side
+    bool ok[S];
 };
-template <int K> __device__ __forceinline__ void rb_cells(const SmallDesc &D, const SmallLevel &L, RbCells<K> &c) {
+template <int K, int S>
+__device__ __forceinline__ void rb_strips(const SmallDesc &D, const SmallLevel &L, const float *b0, const float *b1,
+                                          RbStrips<K, S> &c) {
     const int nxh = L.nx >> 1, half = L.half;
     const bool px = D.bcx == PIC_BC_PERIODIC, py = D.bcy == PIC_BC_PERIODIC;
     const int wx = D.bcx == PIC_BC_DIRICHLET ? 2 : (px ? 1 : 0), wy = D.bcy == PIC_BC_DIRICHLET ? 2 : (py ? 1 : 0);
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const int j = (int)threadIdx.x + L.nthr * k;
-        const int iy = mdiv(j, L.nxh_magic), m = j - iy * nxh;
-        const bool p = iy & 1;  // colour 0 of this row is at odd ix
-        const int hl = m > 0 ? j - 1 : (px ? j + nxh - 1 : half), hr = m < nxh - 1 ? j + 1 : (px ? j - nxh + 1 : half);
+    for (int i = 0; i < S; ++i) {
+        const int q = (int)threadIdx.x + L.nthr * i;
+        const int g = mdiv(q, L.nxh_magic), m = q - g * nxh, y0 = g * K;  // rows y0 .. y0 + K - 1
+        const int j = y0 * nxh + m;
+        c.ok[i] = y0 < L.ny;
+        c.j[i] = j;
+        const bool hl = m > 0 || px, hr = m < nxh - 1 || px;
+        c.l[i] = hl ? (m > 0 ? j - 1 : j + nxh - 1) : half;
+        c.r[i] = hr ? (m < nxh - 1 ? j + 1 : j - nxh + 1) : half;
+        c.sl[i] = hl ? nxh : 0;
+        c.sr[i] = hr ? nxh : 0;
+        const bool hd = y0 > 0, hu = y0 + K < L.ny;
+        c.dn[i] = hd ? j - nxh : (py ? j + (L.ny - 1) * nxh : half);
+        c.up[i] = hu ? j + K * nxh : (py ? m : half);
         const int dl = m > 0 ? 1 : wx, dr = m < nxh - 1 ? 1 : wx;
-        c.od[k] = iy > 0 ? j - nxh : (py ? j + (L.ny - 1) * nxh : half);
-        c.ou[k] = iy < L.ny - 1 ? j + nxh : (py ? j - (L.ny - 1) * nxh : half);
-        const int dv = 1 + (iy > 0 ? 1 : wy) + (iy < L.ny - 1 ? 1 : wy);
-        c.oh0[k] = p ? hr : hl;
-        c.oh1[k] = p ? hl : hr;
-        c.di0[k] = __frcp_rn((float)(dv + (p ? dr : dl)));
-        c.di1[k] = __frcp_rn((float)(dv + (p ? dl : dr)));
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int dv = 1 + (k > 0 || hd ? 1 : wy) + (k < K - 1 || hu ? 1 : wy);
+            c.di0[i][k] = __frcp_rn((float)(dv + (k & 1 ? dr : dl)));
+            c.di1[i][k] = __frcp_rn((float)(dv + (k & 1 ? dl : dr)));
+            c.b0[i][k] = c.ok[i] ? b0[j + k * nxh] : 0.0f;
+            c.b1[i][k] = c.ok[i] ? b1[j + k * nxh] : 0.0f;
+        }
     }
 }
-// xs: this colour's values, xo: the other colour's
-template <int K>
-__device__ __forceinline__ void rb_half(float *xs, const float *xo, const int (&oh)[K], const int (&od)[K],
-                                        const int (&ou)[K], const float (&b)[K], const float (&di)[K], int nthr, int half) {
+// One half sweep of colour C: xs its values, xo the other colour's in shared memory; v and o the
+// strips' own values of both.
+template <int K, int S, int C>
+__device__ __forceinline__ void rb_half(const RbStrips<K, S> &c, float *xs, const float *xo, float (&v)[S][K],
+                                        const float (&o)[S][K], int nxh) {
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const int j = (int)threadIdx.x + nthr * k;
-        if (j < half) xs[j] = (b[k] + (((xo[j] + xo[oh[k]]) + xo[od[k]]) + xo[ou[k]])) * di[k];
+    for (int i = 0; i < S; ++i) {
+        if (!c.ok[i]) continue;
+        const float below = xo[c.dn[i]], above = xo[c.up[i]];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const float h = (k & 1) == C ? xo[c.l[i] + k * c.sl[i]] : xo[c.r[i] + k * c.sr[i]];
+            const float s = ((h + o[i][k]) + (k > 0 ? o[i][k > 0 ? k - 1 : 0] : below)) +
+                            (k < K - 1 ? o[i][k < K - 1 ? k + 1 : k] : above);
+            v[i][k] = ((C ? c.b1[i][k] : c.b0[i][k]) + s) * (C ? c.di1[i][k] : c.di0[i][k]);
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k) xs[c.j[i] + k * nxh] = v[i][k];
     }
 }
 
 // Pre-smoothing from x = 0 and the residual's restriction.
-template <int K>
+template <int K, int S>
 __device__ __forceinline__ void rb_down(const SmallDesc &D, const SmallLevel &L, const SmallLevel &Cc, float *sm, int bar) {
-    const int nthr = L.nthr, half = L.half;
+    const int nthr = L.nthr, nxh = L.nx >> 1;
     float *x0 = sm + L.off, *x1 = x0 + L.hs;
-    const float *b0 = x0 + L.boff, *b1 = b0 + L.hs;
-    {
-        RbCells<K> c;
-        float bb0[K], bb1[K];
-        rb_cells<K>(D, L, c);
+    RbStrips<K, S> c;
+    float a[S][K], e[S][K];  // the strips' values of colour 0 and 1
+    rb_strips<K, S>(D, L, x0 + L.boff, x1 + L.boff, c);
+#pragma unroll
+    for (int i = 0; i < S; ++i)
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            const int j = (int)threadIdx.x + nthr * k;
-            bb0[k] = bb1[k] = 0.0f;
-            if (j < half) {
-                bb0[k] = b0[j]; bb1[k] = b1[j];
-                x0[j] = bb0[k] * c.di0[k];  // the first half sweep reads zeros only
-            }
+            a[i][k] = c.b0[i][k] * c.di0[i][k];  // the first half sweep reads zeros only
+            if (c.ok[i]) x0[c.j[i] + k * nxh] = a[i][k];
         }
-        if (threadIdx.x == 0) x0[half] = x1[half] = 0.0f;  // missing neighbours
+    if (threadIdx.x == 0) x0[L.half] = x1[L.half] = 0.0f;  // missing neighbours
+    part_bar(bar, nthr);
+    rb_half<K, S, 1>(c, x1, x0, e, a, nxh);
+    part_bar(bar, nthr);
+#pragma unroll
+    for (int s = 1; s < kNu; ++s) {
+        rb_half<K, S, 0>(c, x0, x1, a, e, nxh);
         part_bar(bar, nthr);
-        rb_half<K>(x1, x0, c.oh1, c.od, c.ou, bb1, c.di1, nthr, half);
+        rb_half<K, S, 1>(c, x1, x0, e, a, nxh);
         part_bar(bar, nthr);
-        for (int s = 1; s < kNu; ++s) {
-            rb_half<K>(x0, x1, c.oh0, c.od, c.ou, bb0, c.di0, nthr, half);
-            part_bar(bar, nthr);
-            rb_half<K>(x1, x0, c.oh1, c.od, c.ou, bb1, c.di1, nthr, half);
-            part_bar(bar, nthr);
-        }
     }
-    // coarse cell p: the residuals of its children (0,0), (1,0), (0,1), (1,1) summed in this order
-    const int nxh = L.nx >> 1;
-    const bool px = D.bcx == PIC_BC_PERIODIC, py = D.bcy == PIC_BC_PERIODIC;
-    const int wx = D.bcx == PIC_BC_DIRICHLET ? 2 : (px ? 1 : 0), wy = D.bcy == PIC_BC_DIRICHLET ? 2 : (py ? 1 : 0);
+    // coarse cells: the residuals of the children (0,0), (1,0), (0,1), (1,1) summed in this order
     float *bc = sm + Cc.off + Cc.boff;
-    for (int p = threadIdx.x; p < Cc.n; p += nthr) {
-        const int qy = mdiv(p, L.nxh_magic), qx = p - qy * nxh;
-        const int j0 = 2 * qy * nxh + qx, j1 = j0 + nxh;
-        const bool le = qx > 0, re = qx < nxh - 1, de = qy > 0, ue = 2 * qy + 2 < L.ny;
-        const bool hl = le || px, hr = re || px;
-        const int wl = le ? -1 : nxh - 1, wr = re ? 1 : 1 - nxh;
-        const int jd = de ? j0 - nxh : (py ? j0 + (L.ny - 1) * nxh : half);
-        const int ju = ue ? j1 + nxh : (py ? j1 - (L.ny - 1) * nxh : half);
-        const float x00 = x0[j0], x10 = x1[j0], x01 = x1[j1], x11 = x0[j1];
-        const float l0 = hl ? x1[j0 + wl] : 0.0f, l1 = hl ? x0[j1 + wl] : 0.0f;
-        const float r0 = hr ? x0[j0 + wr] : 0.0f, r1 = hr ? x1[j1 + wr] : 0.0f;
-        const float dl = (float)(1 + (le ? 1 : wx)), dr = (float)(1 + (re ? 1 : wx));
-        const float dd = (float)(1 + (de ? 1 : wy)), du = (float)(1 + (ue ? 1 : wy));
-        float s = b0[j0] - ((dl + dd) * x00 - (((l0 + x10) + x1[jd]) + x01));
-        s += b1[j0] - ((dr + dd) * x10 - (((x00 + r0) + x0[jd]) + x11));
-        s += b1[j1] - ((dl + du) * x01 - (((l1 + x11) + x00) + x0[ju]));
-        s += b0[j1] - ((dr + du) * x11 - (((x01 + r1) + x10) + x1[ju]));
-        bc[sm_pos(Cc, p)] = s;
+#pragma unroll
+    for (int i = 0; i < S; ++i) {
+        if (!c.ok[i]) continue;
+        const int q = (int)threadIdx.x + nthr * i;
+        const int g = mdiv(q, L.nxh_magic), m = q - g * nxh;
+        const float b0d = x0[c.dn[i]], b1d = x1[c.dn[i]], a0u = x0[c.up[i]], a1u = x1[c.up[i]];
+#pragma unroll
+        for (int k = 0; k < K; k += 2) {
+            const float l0 = x1[c.l[i] + k * c.sl[i]], l1 = x0[c.l[i] + (k + 1) * c.sl[i]];
+            const float r0 = x0[c.r[i] + k * c.sr[i]], r1 = x1[c.r[i] + (k + 1) * c.sr[i]];
+            const float x00 = a[i][k], x10 = e[i][k], x01 = e[i][k + 1], x11 = a[i][k + 1];
+            const float d1 = k > 0 ? e[i][k > 0 ? k - 1 : 0] : b1d, d0 = k > 0 ? a[i][k > 0 ? k - 1 : 0] : b0d;
+            const float u0 = k + 2 < K ? a[i][k + 2 < K ? k + 2 : k] : a0u, u1 = k + 2 < K ? e[i][k + 2 < K ? k + 2 : k] : a1u;
+            // the diagonals are small integers: exact from their reciprocals
+            const float g00 = rintf(__frcp_rn(c.di0[i][k])), g10 = rintf(__frcp_rn(c.di1[i][k]));
+            const float g01 = rintf(__frcp_rn(c.di1[i][k + 1])), g11 = rintf(__frcp_rn(c.di0[i][k + 1]));
+            float s = c.b0[i][k] - (g00 * x00 - (((l0 + x10) + d1) + x01));
+            s += c.b1[i][k] - (g10 * x10 - (((x00 + r0) + d0) + x11));
+            s += c.b1[i][k + 1] - (g01 * x01 - (((l1 + x11) + x00) + u0));
+            s += c.b0[i][k + 1] - (g11 * x11 - (((x01 + r1) + x10) + u1));
+            const int cy = (K / 2) * g + k / 2;
+            bc[Cc.fast ? ((m + cy) & 1) * Cc.hs + cy * (nxh >> 1) + (m >> 1) : cy * nxh + m] = s;
+        }
     }
     part_bar(bar, nthr);
 }
 
 // The coarse correction (needed on colour 1 only: the first half sweep overwrites colour 0
 // without reading it) and the post-smoothing.
-template <int K>
+template <int K, int S>
 __device__ __forceinline__ void rb_up(const SmallDesc &D, const SmallLevel &L, const SmallLevel &Cc, float *sm, int bar) {
-    const int nthr = L.nthr, half = L.half, nxh = L.nx >> 1;
+    const int nthr = L.nthr, nxh = L.nx >> 1;
     float *x0 = sm + L.off, *x1 = x0 + L.hs;
-    const float *b0 = x0 + L.boff, *b1 = b0 + L.hs;
     const float *xc = sm + Cc.off;
-    RbCells<K> c;
-    float bb0[K], bb1[K];
-    rb_cells<K>(D, L, c);
+    RbStrips<K, S> c;
+    float a[S][K], e[S][K];
+    rb_strips<K, S>(D, L, x0 + L.boff, x1 + L.boff, c);
+    part_bar(bar, nthr);  // the coarser level's correction is complete
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const int j = (int)threadIdx.x + nthr * k;
-        bb0[k] = bb1[k] = 0.0f;
-        if (j < half) {
-            bb0[k] = b0[j]; bb1[k] = b1[j];
-            const int iy = mdiv(j, L.nxh_magic), m = j - iy * nxh, cy = iy >> 1;
-            const int q = Cc.fast ? ((m + cy) & 1) * Cc.hs + cy * (nxh >> 1) + (m >> 1) : cy * nxh + m;
-            x1[j] += xc[q];
+    for (int i = 0; i < S; ++i) {
+        const int q = (int)threadIdx.x + nthr * i;
+        const int g = mdiv(q, L.nxh_magic), m = q - g * nxh;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            e[i][k] = 0.0f;
+            if (c.ok[i]) {
+                const int cy = (K / 2) * g + k / 2;
+                e[i][k] = x1[c.j[i] + k * nxh] +
+                          xc[Cc.fast ? ((m + cy) & 1) * Cc.hs + cy * (nxh >> 1) + (m >> 1) : cy * nxh + m];
+                x1[c.j[i] + k * nxh] = e[i][k];
+            }
         }
     }
     part_bar(bar, nthr);
+#pragma unroll
     for (int s = 0; s < kNu; ++s) {
-        rb_half<K>(x0, x1, c.oh0, c.od, c.ou, bb0, c.di0, nthr, half);
+        rb_half<K, S, 0>(c, x0, x1, a, e, nxh);
         part_bar(bar, nthr);
-        rb_half<K>(x1, x0, c.oh1, c.od, c.ou, bb1, c.di1, nthr, half);
+        rb_half<K, S, 1>(c, x1, x0, e, a, nxh);
         if (s + 1 < kNu) part_bar(bar, nthr);
     }
 }
@@ -811,9 +848,9 @@ __device__ void sm_vcycle(const SmallDesc &D, float *sm, bool singular, float *r
     for (; g < last; ++g) {
         const SmallLevel &L = D.lv[g], &Cc = D.lv[g + 1];
         if ((int)threadIdx.x >= L.nthr) break;
-        if (L.kc == 1) rb_down<1>(D, L, Cc, sm, 1 + g - gf);
-        else if (L.kc == 2) rb_down<2>(D, L, Cc, sm, 1 + g - gf);
-        else rb_down<4>(D, L, Cc, sm, 1 + g - gf);
+        if (L.rows == 4) rb_down<4, 1>(D, L, Cc, sm, 1 + g - gf);
+        else if (L.strips == 1) rb_down<2, 1>(D, L, Cc, sm, 1 + g - gf);
+        else rb_down<2, 2>(D, L, Cc, sm, 1 + g - gf);
     }
     if (g == last) {
         const SmallLevel &L = D.lv[last];
@@ -824,10 +861,9 @@ __device__ void sm_vcycle(const SmallDesc &D, float *sm, bool singular, float *r
     }
     for (--g; g >= gf; --g) {
         const SmallLevel &L = D.lv[g], &Cc = D.lv[g + 1];
-        part_bar(1 + g - gf, L.nthr);  // the coarser level's correction is complete
-        if (L.kc == 1) rb_up<1>(D, L, Cc, sm, 1 + g - gf);
-        else if (L.kc == 2) rb_up<2>(D, L, Cc, sm, 1 + g - gf);
-        else rb_up<4>(D, L, Cc, sm, 1 + g - gf);
+        if (L.rows == 4) rb_up<4, 1>(D, L, Cc, sm, 1 + g - gf);
+        else if (L.strips == 1) rb_up<2, 1>(D, L, Cc, sm, 1 + g - gf);
+        else rb_up<2, 2>(D, L, Cc, sm, 1 + g - gf);
     }
     if (gf > 0) __syncthreads();
     for (g = gf - 1; g >= 0; --g) {
@@ -889,9 +925,10 @@ __device__ __forceinline__ void small_sums(int C, int rank, int n, double *vbuf,
         }
         __syncthreads();
         for (int q = threadIdx.x >> 7; q < m; q += 8) {
-            double s = vbuf[1024 * q + u];
+            double v[8];
 #pragma unroll
-            for (int k = 1; k < 8; ++k) s += vbuf[1024 * q + u + 128 * k];
+            for (int k = 0; k < 8; ++k) v[k] = vbuf[1024 * q + u + 128 * k];
+            double s = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, o);
             if ((u & 31) == 0) part[4 * (rank + (q0 + q) * C) + (u >> 5)] = s;
@@ -935,8 +972,7 @@ __global__ void __launch_bounds__(1024, 1) k_small_solve(const SmallSolve *__res
     extern __shared__ __align__(16) float sm[];
     __shared__ float redf[33];
     __shared__ SmallDesc D;
-    __shared__ double part[64], outs[2];
-    __shared__ double rel_sh;
+    __shared__ double part[64], mean_sh;
     __shared__ int stop_sh;
     const SmallSolve &it = items[blockIdx.x / C];
     for (int k = threadIdx.x; k < (int)(sizeof(SmallDesc) / 4); k += 1024)
@@ -950,7 +986,8 @@ __global__ void __launch_bounds__(1024, 1) k_small_solve(const SmallSolve *__res
         inv = cs;
     }
     float *lsm = cl.map_shared_rank(sm, 0);  // the leader's levels
-    double *lpart = cl.map_shared_rank(part, 0), *louts = cl.map_shared_rank(outs, 0);
+    double *lpart = cl.map_shared_rank(part, 0);
+    const double *lmean = cl.map_shared_rank(&mean_sh, 0);
     const int *lstop = cl.map_shared_rank(&stop_sh, 0);
     const double *__restrict__ diag64 = it.diag64;
     const double *__restrict__ val64 = it.val64;
@@ -958,26 +995,29 @@ __global__ void __launch_bounds__(1024, 1) k_small_solve(const SmallSolve *__res
     double *bvec = it.bvec;
     const uint8_t *__restrict__ lev = it.lev;
     const int lmax = it.lmax, singular = it.singular, maxc = it.maxc;
-    const double tol = it.tol;
+    const double tol2 = it.tol * it.tol;
+    double bb = 0.0;  // ||b||^2 (the leader's first warp)
     const SmallLevel &L = D.lv[0];
     const int n = L.n, nch = (n + 1023) >> 10;
 #define CL_FOR(i)                                                                    \
     for (int c_ = rank; c_ < nch; c_ += C)                                           \
         for (int i = (c_ << 10) + (int)threadIdx.x; i < n && i < ((c_ + 1) << 10); i += 1 << 30)
-    // two sums over all cells, known to every thread of the cluster
+    // the area-weighted mean of f over all cells (areas in units of the finest cell's), known to
+    // every thread of the cluster (the division is done once: in FP64 it is ~25 operations)
     auto area = [&](int i) { const double s = (double)(1 << (lmax - lev[i])); return s * s; };
-    auto moments = [&](auto f, double &s0, double &s1) {
+    auto mean = [&](auto f) -> double {
         small_sums(C, rank, n, vbuf, nbuf, lpart, f);
-        __syncthreads();
-        small_sums(C, rank, n, vbuf, nbuf, lpart + 32, area);
-        cl.sync();
-        if (rank == 0 && threadIdx.x < 32) {
-            const double a = small_total(part, n), b = small_total(part + 32, n);
-            if (threadIdx.x == 0) { outs[0] = a; outs[1] = b; }
+        if (!L.uniform) {
+            __syncthreads();
+            small_sums(C, rank, n, vbuf, nbuf, lpart + 32, area);
         }
         cl.sync();
-        s0 = louts[0];
-        s1 = louts[1];
+        if (rank == 0 && threadIdx.x < 32) {
+            const double a = small_total(part, n), b = L.uniform ? (double)n : small_total(part + 32, n);
+            if (threadIdx.x == 0) mean_sh = a / b;
+        }
+        cl.sync();
+        return *lmean;
     };
     const int ns = *it.n_solves;
     if (ns >= 1)
@@ -987,10 +1027,8 @@ __global__ void __launch_bounds__(1024, 1) k_small_solve(const SmallSolve *__res
             it.phi_prev[i] = p;
         }
     if (singular) {  // right-hand side compatibility: remove an area-proportional share
-        double sb, sa;
-        moments([&](int i) { return bvec[i]; }, sb, sa);
-        const double k = sb / sa;
-        CL_FOR(i) bvec[i] -= k * area(i);
+        const double k = mean([&](int i) { return bvec[i]; });
+        CL_FOR(i) bvec[i] -= L.uniform ? k : k * area(i);
     }
     small_sums(C, rank, n, vbuf, nbuf, lpart + 32, [&](int i) { return bvec[i] * bvec[i]; });
     cl.sync();  // every CTA has read the counter; phi is complete
@@ -1018,12 +1056,14 @@ __global__ void __launch_bounds__(1024, 1) k_small_solve(const SmallSolve *__res
         cl.sync();
         if (rank == 0) {
             if (threadIdx.x < 32) {
-                const double rr = small_total(part, n), bb = small_total(part + 32, n);
+                // ||r|| <= tol ||b||, compared squared: the root and the division only once done
+                const double rr = small_total(part, n);
+                if (cyc == 0) bb = small_total(part + 32, n);
                 if (threadIdx.x == 0) {
-                    const double rel = bb > 0.0 ? sqrt(rr / bb) : sqrt(rr);
-                    rel_sh = rel;
-                    stop_sh = rel <= tol || (bb == 0.0 && rr == 0.0) || cyc >= maxc;
-                    if (stop_sh) {
+                    const bool stop = rr <= tol2 * (bb > 0.0 ? bb : 1.0) || cyc >= maxc;
+                    stop_sh = stop;
+                    if (stop) {
+                        const double rel = bb > 0.0 ? sqrt(rr / bb) : sqrt(rr);
                         it.stats[0] = (double)cyc;
                         it.stats[1] = rel;
                         it.stats[2] = worst_residual(it.stats[2], rel);
@@ -1039,9 +1079,7 @@ __global__ void __launch_bounds__(1024, 1) k_small_solve(const SmallSolve *__res
         cl.sync();  // phi complete before the next residual (and x read before the next V-cycle)
     }
     if (singular) {  // zero area-weighted mean (a constant changes no residual)
-        double sv, sa;
-        moments([&](int i) { return area(i) * phi[i]; }, sv, sa);
-        const double k = sv / sa;
+        const double k = mean([&](int i) { return L.uniform ? phi[i] : area(i) * phi[i]; });
         CL_FOR(i) phi[i] -= k;
     }
 #undef CL_FOR
@@ -1138,11 +1176,14 @@ SmallDesc small_desc(const Instance &in, int g0) {
         S.half = (int32_t)L.n / 2;
         S.hs = S.half + 4;
         S.boff = S.fast ? 2 * S.hs : (int32_t)L.n;
-        // at least 8 warps (the coarsest solve runs on the last level's), every warp when the
-        // coarsest level is solved by CG, which uses the whole block
-        S.nthr = in.coarse_inv ? std::min(1024, std::max(256, (S.half + 31) / 32 * 32)) : 1024;
-        const int kc = (S.half + S.nthr - 1) / S.nthr;
-        S.kc = kc > 2 ? 4 : kc;
+        // strips of 4 rows where 2-row strips would need more than 512 threads (fewer shared
+        // loads per cell, fewer warps at the barriers), of 2 rows on smaller levels (shorter
+        // chains).  At least 8 warps take part (the coarsest solve runs on the last level's), every
+        // warp when the coarsest level is solved by CG, which uses the whole block.
+        S.rows = S.ny % 4 == 0 && S.half > 1024 ? 4 : 2;
+        const int ns = S.half / S.rows;
+        S.strips = ns > 1024 ? 2 : 1;
+        S.nthr = in.coarse_inv ? std::min(1024, std::max(256, (ns + 31) / 32 * 32)) : 1024;
         off += S.fast ? 4 * S.hs : 2 * (int32_t)L.n;
     }
     D.off_cg = off;
