@@ -393,7 +393,6 @@ pic_status pic_destroy(pic_ctx *ctx) {
     cudaStreamSynchronize(ctx->stream);
     for (Instance &in : ctx->inst) {
         if (in.mg_cycle) cudaGraphExecDestroy(in.mg_cycle);
-        repairs_release(in);
         in.mesh_mem.release_all();
         in.inv_mem.release_all();
         in.part_mem[0].release_all();

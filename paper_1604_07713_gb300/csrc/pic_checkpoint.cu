@@ -154,7 +154,7 @@ template <typename R> void write_species(pic_ctx *ctx, Instance &in, int s, Writ
     int32_t *cnt = dalloc<int32_t>(T, nl);
     k_leaf_counts<<<blocks_for(nl), kT, 0, st>>>(nl, sp.start, sp.end, cnt);
     count_launch(ctx);
-    list_ranks(ctx, sp, nl);
+    list_ranks(ctx, in, s);
     SoA<R> o = dense_soa<R>(T, n);
     k_gather_records<R><<<warp_blocks(nl), kT, 0, st>>>(nl, sp.start, sp.end, sp.rank0, soa<R>(sp, sp.cur), o);
     count_launch(ctx);

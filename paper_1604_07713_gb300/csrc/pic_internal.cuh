@@ -31,6 +31,7 @@ void check_cuda(cudaError_t e, const char *what);
 constexpr int kEll = 8;           // off-diagonal slots per row of the Poisson operator
 constexpr int kMaxLevel = 8;      // deepest supported refinement level
 constexpr int kWarp = 32;
+constexpr int kPartWords = 1024;
 
 // ------------------------------------------------------------------------------------
 // Device memory.  A context keeps the blocks it releases in a size-class cache and hands
@@ -128,6 +129,7 @@ struct Species {
     int32_t *stay = nullptr, *inc = nullptr, *fill = nullptr;  // [nleaf + 1]
     int32_t *big = nullptr;    // [nleaf + 1] long entering regions, their count at [nleaf]
     int32_t *moved = nullptr;  // [nleaf + 1] leaves that ran out of free slots, count at [nleaf]
+    int32_t *spart = nullptr;  // tile totals of the list-rank and spawn scans (leaf_tiles(nleaf) words each)
     int32_t *spawn = nullptr, *spawn_base = nullptr;           // [nleaf], [nleaf + 1]
     // overflow store
     void *ovf[6] = {};
@@ -143,10 +145,7 @@ struct Species {
     void *stay_hi = nullptr, *stay_lo = nullptr;               // R [nleaf]
     void *ent_hi = nullptr, *ent_lo = nullptr;                 // R [nleaf]
     bool sums_valid = false;
-    // the per-step list repairs as a graph of two IF nodes (pic_lists.cu), valid for the
-    // mesh and list epochs it was built in
-    cudaGraphExec_t repair = nullptr;
-    int64_t repair_mesh_epoch = -1, repair_lists_epoch = -1;
+    int32_t *part = nullptr;  // [kPartWords] block totals of the re-layout's scan
 };
 
 template <typename R> struct SoA {
@@ -409,6 +408,34 @@ __device__ __forceinline__ uint32_t philox2x32_10_x(uint32_t c0, uint32_t c1, co
     return c0;  // the first output word
 }
 
+// Exclusive prefix of v over the block's threads (at most 1024, whole warps); *total their sum.
+__device__ __forceinline__ int32_t block_exclusive_scan(int32_t v, int32_t *total) {
+    __shared__ int32_t warp_sums[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        int32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) warp_sums[wid] = x;
+    __syncthreads();
+    if (wid == 0) {
+        int32_t s = (lane < (int)(blockDim.x >> 5)) ? warp_sums[lane] : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            int32_t y = __shfl_up_sync(0xFFFFFFFFu, s, o);
+            if (lane >= o) s += y;
+        }
+        warp_sums[lane] = s;
+    }
+    __syncthreads();
+    const int32_t before = (wid > 0 ? warp_sums[wid - 1] : 0) + x - v;
+    *total = warp_sums[(blockDim.x >> 5) - 1];
+    __syncthreads();
+    return before;
+}
+
 // Leaf geometry on its level's lattice.
 struct LeafGeom { int32_t ix, iy, s; };
 
@@ -475,10 +502,10 @@ void species_leaf_arrays(pic_ctx *ctx, Instance &in, int s, int64_t nl);
 void lists_from_counts(pic_ctx *ctx, Species &sp, int64_t nl, const int32_t *cnt, int32_t *start,
                        int32_t *end, int32_t *scratch);
 void lists_installed(pic_ctx *ctx, Species &sp, int64_t nl);  // lim, tail after start / end are set
-void list_ranks(pic_ctx *ctx, Species &sp, int64_t nl);       // rank0 from start / end
+void list_ranks(pic_ctx *ctx, Instance &in, int s);             // rank0 from start / end
 void count_totals(pic_ctx *ctx, Instance &in);  // flags[1] of every species, device side
-void place_overflow(pic_ctx *ctx, Instance &in, int s);  // tail moves, else re-layout
-void repairs_release(Instance &in);                       // the cached repair graphs
+void step_lists_prep(pic_ctx *ctx, Instance &in, bool ionize);  // list ranks of every species, step reset
+void step_repairs(pic_ctx *ctx, Instance &in, bool ionize);     // spawn offsets; tail moves, else re-layout
 BatchTab batch_prepare_lists(pic_ctx *ctx);                // per (instance, species) list arrays
 void lists_prep_batch(pic_ctx *ctx);                      // step reset and record counts
 void repairs_batch(pic_ctx *ctx);                         // overflow repairs of every instance
@@ -531,6 +558,14 @@ pic_status guarded_call(pic_ctx *ctx, pic_status (*fn)(void *), void *arg);
 void exclusive_scan_i32(pic_ctx *ctx, const int32_t *in, int32_t *out, int64_t n,
                         int32_t *scratch, const int32_t *gate = nullptr);
 int64_t scan_scratch_elems(int64_t n);
+// The step's scans over leaves: tiles of kLeafTile * leaf_runs(n) leaves, few enough that every
+// block can add up the totals of the tiles before its own.
+constexpr int kLeafTile = 1024;  // 256 threads x 4 leaves
+inline int leaf_runs(int64_t n) { return (int)((n + (int64_t)kLeafTile * 2048 - 1) / ((int64_t)kLeafTile * 2048)); }
+inline int leaf_tiles(int64_t n) {
+    const int64_t t = (int64_t)kLeafTile * leaf_runs(n);
+    return (int)((n + t - 1) / t);
+}
 // segments {in, out, n}: out[0..n) = exclusive scan of in, out[n] = total, one launch per pass
 // With gates, segment k does nothing while *gate[k] == 0.
 ScanPlan scan_plan(pic_ctx *ctx, const std::vector<const int32_t *> &in, const std::vector<int32_t *> &out,

@@ -1357,22 +1357,6 @@ template <typename R> SortArgs step_sort_args(Instance &in, int s, int mode = PU
     return a;
 }
 
-// Per species before a push: no entering records yet, nothing in the overflow store, no
-// moved leaves, the tail not used up, and (electrons with ionization) no spawns counted.
-__global__ void k_step_reset(int64_t nl, int32_t *__restrict__ fill, int32_t *__restrict__ flags,
-                             int32_t *__restrict__ moved, int32_t *__restrict__ spawn) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nl) {
-        fill[i] = 0;
-        if (spawn) spawn[i] = 0;
-    }
-    if (i == 0) {
-        flags[0] = 0;
-        flags[5] = 0;
-        moved[nl] = 0;
-    }
-}
-
 template <typename R> void step_impl(pic_ctx *ctx, Instance &in, int64_t step, int mode) {
     cudaStream_t st = ctx->stream;
     const int nsp = in.cfg.n_species;
@@ -1412,13 +1396,7 @@ template <typename R> void step_impl(pic_ctx *ctx, Instance &in, int64_t step, i
     Species &e = in.sp[0];
     {
         Phase ph(ctx, PIC_PHASE_LISTS);
-        for (int s = 0; s < nsp; ++s) {
-            Species &sp = in.sp[s];
-            k_step_reset<<<blocks_for(nl), kT, 0, st>>>(nl, sp.fill, sp.flags, sp.moved,
-                                                        s == 0 && ionize ? sp.spawn : nullptr);
-            count_launch(ctx);
-            list_ranks(ctx, sp, nl);
-        }
+        step_lists_prep(ctx, in, ionize);
     }
     {
         Phase ph(ctx, PIC_PHASE_MOVE);
@@ -1437,8 +1415,7 @@ template <typename R> void step_impl(pic_ctx *ctx, Instance &in, int64_t step, i
     }
     {
         Phase ph(ctx, PIC_PHASE_SCAN);
-        if (ionize) exclusive_scan_i32(ctx, e.spawn, e.spawn_base, nl, e.spawn_base + nl + 1 + scan_scratch_elems(nl));
-        for (int s = 0; s < nsp; ++s) place_overflow(ctx, in, s);
+        step_repairs(ctx, in, ionize);
     }
     {
         Phase ph(ctx, PIC_PHASE_SORT);
@@ -1732,7 +1709,7 @@ void particles_read(pic_ctx *ctx, Instance &in, int s, double *x, double *y, dou
     for (int k = 0; k < 6; ++k) d[k] = dalloc<double>(tmp, n);
     unsigned long long *did = dalloc<unsigned long long>(tmp, n);
     uint32_t *dleaf = dalloc<uint32_t>(tmp, n);
-    list_ranks(ctx, sp, nl);
+    list_ranks(ctx, in, s);
     const int32_t *out0 = sp.rank0;
     Level &g = in.lv[0];
     const double hf = in.h0 / (double)(1 << in.lmax);
