@@ -367,8 +367,8 @@ pic_status pic_create(const pic_config *cfg, int32_t n_instances, pic_ctx **out)
             in.part_mem[1].cache = &ctx->cache;
             GB_CUDA(cudaMallocHost(&in.red_host, 64));
             GB_CUDA(cudaMallocHost(&in.cnt_host, 64));
-            GB_CUDA(cudaMalloc(&in.d_next_id, 8));
-            GB_CUDA(cudaMemset(in.d_next_id, 0, 8));
+            GB_CUDA(cudaMalloc(&in.d_next_id, 16));
+            GB_CUDA(cudaMemset(in.d_next_id, 0, 16));
             GB_CUDA(cudaMalloc(&in.d_err, 4));
             GB_CUDA(cudaMemset(in.d_err, 0, 4));
         }

@@ -205,7 +205,7 @@ struct Instance {
     double *cic_part = nullptr;  // cloud-in-cell deposit: per leaf its charge on the 3 x 3 cells around it
     Species sp[2];
     int64_t next_id = 0;                     // host mirror (exact after a sync)
-    unsigned long long *d_next_id = nullptr; // device counter of the next particle id
+    unsigned long long *d_next_id = nullptr; // device: next particle id, [1] its value before the step
     int32_t *d_err = nullptr;                // device-side consistency flag (0 = fine)
     double *d_walls = nullptr;               // the context's wall array for this instance (4)
     int32_t report_err = 0;                  // consistency flag read by the last report

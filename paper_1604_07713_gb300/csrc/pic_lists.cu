@@ -75,10 +75,11 @@ __global__ void k_lists_installed(int64_t nl, const int32_t *__restrict__ start,
 struct RankEntry {
     const int32_t *start, *end;
     int32_t *rank0, *part;
-    int32_t *fill, *flags, *moved, *spawn;  // fill null: ranks only
+    int32_t *fill, *flags, *moved, *big, *spawn;  // fill null: ranks only
 };
 struct RankArgs {
     RankEntry e[2];
+    unsigned long long *next_id;  // [1] := [0], the next id before the step (null: ranks only)
     int64_t nl;
     int runs;
 };
@@ -111,6 +112,8 @@ __global__ void __launch_bounds__(kT) k_lists_sums(RankArgs A) {
             e.flags[0] = 0;
             e.flags[5] = 0;
             e.moved[A.nl] = 0;
+            e.big[A.nl] = 0;
+            if (blockIdx.y == 0) A.next_id[1] = A.next_id[0];
         }
     }
 }
@@ -454,6 +457,8 @@ template <typename R> __global__ void __launch_bounds__(kT) k_step_place(const _
         place_ovf<R>(e.end, e.cap, soa_of<R>(e.o), e.okey, e.oaux, e.odest, e.oslot, soa_of<R>(e.d), e.key, e.aux,
                      e.moved, e.nl, e.flags, (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
                      (int64_t)gridDim.x * blockDim.x, blockIdx.x == 0 && threadIdx.x == 0);
+        // (after its count is read) the array holds the sort's medium regions next
+        if (blockIdx.x == 0 && threadIdx.x == 0) e.moved[e.nl] = 0;
         return;
     }
     if ((int)blockIdx.x >= A.tiles) return;
@@ -862,7 +867,8 @@ RankArgs rank_args(Instance &in, int first, int last, bool reset, bool ionize) {
         RankEntry &e = A.e[s - first];
         e.start = sp.start; e.end = sp.end; e.rank0 = sp.rank0; e.part = sp.spart;
         if (!reset) continue;
-        e.fill = sp.fill; e.flags = sp.flags; e.moved = sp.moved;
+        e.fill = sp.fill; e.flags = sp.flags; e.moved = sp.moved; e.big = sp.big;
+        A.next_id = in.d_next_id;
         e.spawn = s == 0 && ionize ? sp.spawn : nullptr;
     }
     return A;

@@ -248,7 +248,7 @@ template <typename R> struct PushArgs {
     int32_t *err;
     int self_wrap;        // some leaf spans a whole periodic direction (a particle may wrap back)
     // collisions
-    int mcc, species;
+    int mcc;
     int drift_kick;  // the implicit scheme's corrector: drift by the kick's increment only
     R ng_dt, sig_el, sig_iz0, eps_th, half_m_over_qe, two_qe_over_m, two_m_over_mn;
     R vt_gas;       // neutral thermal speed sqrt(T qe / M)
@@ -301,7 +301,7 @@ template <typename R> struct Queue {
 // Electrons that spawn are ranked among their leaf's spawning particles in list order: the
 // entries are in list order, and (run_leaf, run_count) carry the count of the last leaf of
 // the previous batch, whose entries may continue in this one.
-template <typename R>
+template <typename R, int S>
 __device__ __forceinline__ void run_deferred(const PushArgs<R> &a, const Queue<R> &q, int e, bool valid, uint32_t span,
                                              uint32_t ion_span, uint32_t step, int32_t &run_leaf, int32_t &run_count) {
     R vx = 0, vy = 0, vz = 0, w = 0;
@@ -338,7 +338,7 @@ __device__ __forceinline__ void run_deferred(const PushArgs<R> &a, const Queue<R
         const R v2 = vx * vx + vy * vy + vz * vz;
         const R U0 = u24<R>(q.r0[e]);
         const U4 r0 = philox4x32_10(id, a.inst_word, step, 0u, a.keys);  // the other uniforms
-        if (a.species == 0) {
+        if constexpr (S == 0) {
             // the exact test, from the same quantities as the bound of the pass
             const R eps = a.half_m_over_qe * v2;
             const R siz = eps > a.eps_th ? a.sig_iz0 * ((R)1 - m_div(a.eps_th, eps)) : (R)0;
@@ -441,8 +441,9 @@ __device__ __forceinline__ void run_deferred(const PushArgs<R> &a, const Queue<R
 // (a 64-register build for 1024 threads spills and runs slower).
 // CIC: the field is gathered from the leaf's per-quarter cloud-in-cell coefficients (32 per
 // leaf, lane k holding coefficient k) instead of the bilinear corner field.
-// The warp walks the leaves first, first + nw, ... below last (all lanes call it).
-template <typename R, int NT, bool CIC>
+// The warp walks the leaves first, first + nw, ... below last (all lanes call it).  S: the
+// species, which decides the collision path (0 electrons, 1 ions).
+template <typename R, int NT, bool CIC, int S>
 __device__ __forceinline__ void push_leaves(const PushArgs<R> &a, Queue<R> &q, const int64_t first, const int64_t last,
                                             const int64_t nw) {
     const int lane = threadIdx.x & 31;
@@ -573,7 +574,7 @@ __device__ __forceinline__ void push_leaves(const PushArgs<R> &a, Queue<R> &q, c
                     const R U0 = u24<R>(r0x);
                     // 1 - exp(-x) <= x: a uniform at or above the bound x (with a rounding
                     // margin) means no collision; below it the deferred work makes the exact test
-                    if (a.species == 0) {
+                    if constexpr (S == 0) {
                         // x = n dt sigma(eps) |v| with eps sigma(eps) = sc T(eps), squared so that
                         // neither a root nor a division is needed: U0 < x pad iff
                         // (U0 eps)^2 < (n dt sc pad)^2 v^2 T^2 (a zero uniform always goes on)
@@ -613,7 +614,7 @@ __device__ __forceinline__ void push_leaves(const PushArgs<R> &a, Queue<R> &q, c
                 qn += __popc(defer_mask);
                 if (qn >= 32) {
                     __syncwarp();
-                    run_deferred(a, q, (qhead + lane) & (kQueue - 1), true, span, ion_span, step, run_leaf, run_count);
+                    run_deferred<R, S>(a, q, (qhead + lane) & (kQueue - 1), true, span, ion_span, step, run_leaf, run_count);
                     __syncwarp();
                     qhead = (qhead + 32) & (kQueue - 1);
                     qn -= 32;
@@ -629,22 +630,34 @@ __device__ __forceinline__ void push_leaves(const PushArgs<R> &a, Queue<R> &q, c
         }
     }
     __syncwarp();
-    if (qn > 0) run_deferred(a, q, (qhead + lane) & (kQueue - 1), lane < qn, span, ion_span, step, run_leaf, run_count);
+    if (qn > 0) run_deferred<R, S>(a, q, (qhead + lane) & (kQueue - 1), lane < qn, span, ion_span, step, run_leaf, run_count);
 }
 
-// One instance: persistent warps over all its leaves.
+// One instance, every species in one launch: the first n0 blocks are species 0's persistent
+// warps, the others species 1's, which start as soon as species 0's first blocks end (two
+// launches left the SMs idle while the last warps of the first finished).  The species touch
+// each other's lists only through spawned ions, which take atomic slots past every list's end
+// and are ordered by key afterwards.
+template <typename R> struct PushPair {
+    PushArgs<R> e[2];
+    unsigned n0;
+};
 template <typename R, int NT, bool CIC>
-__global__ void __launch_bounds__(NT, 768 / NT) k_push(const __grid_constant__ PushArgs<R> a) {
+__global__ void __launch_bounds__(NT, 768 / NT) k_push(const __grid_constant__ PushPair<R> P) {
     extern __shared__ unsigned char push_smem[];
     Queue<R> &q = reinterpret_cast<Queue<R> *>(push_smem)[threadIdx.x >> 5];
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    push_leaves<R, NT, CIC>(a, q, warp, a.nleaf, nw);
+    if (blockIdx.x < P.n0) {
+        const int64_t warp = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 5;
+        push_leaves<R, NT, CIC, 0>(P.e[0], q, warp, P.e[0].nleaf, ((int64_t)P.n0 * NT) >> 5);
+    } else {
+        const int64_t warp = ((int64_t)(blockIdx.x - P.n0) * NT + threadIdx.x) >> 5;
+        push_leaves<R, NT, CIC, 1>(P.e[1], q, warp, P.e[1].nleaf, ((int64_t)(gridDim.x - P.n0) * NT) >> 5);
+    }
 }
 
 // Every instance of an ensemble in one launch: block b takes the leaves [c.y, c.z) of
 // instance c.x (c = chunks[b]), the instance's arguments copied to shared memory.
-template <typename R, int NT, bool CIC>
+template <typename R, int NT, bool CIC, int S>
 __global__ void __launch_bounds__(NT, 768 / NT) k_push_batch(const PushArgs<R> *__restrict__ tab,
                                                              const int4 *__restrict__ chunks) {
     extern __shared__ unsigned char push_smem[];
@@ -657,11 +670,7 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_push_batch(const PushArgs<R> *
     }
     __syncthreads();
     Queue<R> &q = reinterpret_cast<Queue<R> *>(push_smem)[threadIdx.x >> 5];
-    push_leaves<R, NT, CIC>(sa, q, (int64_t)c.y + (threadIdx.x >> 5), (int64_t)c.z, NT / 32);
-}
-
-__global__ void k_bump_next_id(unsigned long long *next_id, const int32_t *__restrict__ spawn_total) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) *next_id += 2ull * (unsigned long long)(*spawn_total);
+    push_leaves<R, NT, CIC, S>(sa, q, (int64_t)c.y + (threadIdx.x >> 5), (int64_t)c.z, NT / 32);
 }
 
 // ------------------------------------------------------------------------------------
@@ -885,13 +894,6 @@ __device__ __forceinline__ void sort_big_leaves(const SortArgs &a, const SoA<R> 
     }
 }
 
-template <typename R>
-__global__ void __launch_bounds__(512) k_sort_big(SortArgs a, SoA<R> d, SoA<R> t) {
-    extern __shared__ unsigned long long bk[];
-    __shared__ R red_hi[16], red_lo[16];
-    sort_big_leaves<R>(a, d, t, blockIdx.x, gridDim.x, bk, red_hi, red_lo);
-}
-
 constexpr int kSortLane = 8;  // entering regions up to this long are sorted by a leaf's 8-lane group
 
 // Entering regions of every leaf, 8 lanes per leaf (4 leaves per warp pass): a short region
@@ -962,12 +964,6 @@ __device__ __forceinline__ void sort_entering_groups(const SortArgs &a, const So
     }
 }
 
-template <typename R>
-__global__ void __launch_bounds__(kT) k_sort_entering(SortArgs a, SoA<R> d, SoA<R> t) {
-    sort_entering_groups<R>(a, d, t, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, a.nleaf,
-                            ((int64_t)gridDim.x * blockDim.x) >> 5);
-}
-
 // Medium entering regions (kSortLane < k <= kSortSmem): one warp per listed leaf; the warp
 // takes the list entries first, first + stride, ... below last.  Lane 0 fetches the next
 // entry's leaf and region words while the current region is sorted.  A region sorted in
@@ -1026,18 +1022,39 @@ __device__ __forceinline__ void sort_medium_leaves(const SortArgs &a, const SoA<
     }
 }
 
-template <typename R>
-__global__ void __launch_bounds__(kT, 3) k_sort_medium(SortArgs a, SoA<R> d, SoA<R> t) {
-    __shared__ unsigned long long sm_keys[kWarpsPerBlock][kSortSmem];
-    sort_medium_leaves<R>(a, d, t, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, a.nleaf,
-                          ((int64_t)gridDim.x * blockDim.x) >> 5, sm_keys[threadIdx.x >> 5]);
-}
-
-// ---- the sorts of every (instance, species) of an ensemble, one launch per pass ----------
 template <typename R> struct SortEntry {
     SortArgs a;
     SoA<R> d, t;
 };
+// The sorts of an instance's species, one launch per pass (blockIdx.y: the species).
+template <typename R> struct SortPair {
+    SortEntry<R> e[2];
+    // after a step with ionization: the next id moves past its pairs (the sorts read next_id[1],
+    // its value before the step)
+    unsigned long long *next_id;
+    const int32_t *spawn_total;
+};
+template <typename R> __global__ void __launch_bounds__(kT) k_sort_entering(const __grid_constant__ SortPair<R> P) {
+    const SortEntry<R> &e = P.e[blockIdx.y];
+    if (P.next_id && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
+        P.next_id[0] = P.next_id[1] + 2ull * (unsigned long long)(*P.spawn_total);
+    sort_entering_groups<R>(e.a, e.d, e.t, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, e.a.nleaf,
+                            ((int64_t)gridDim.x * blockDim.x) >> 5);
+}
+template <typename R> __global__ void __launch_bounds__(kT, 3) k_sort_medium(const __grid_constant__ SortPair<R> P) {
+    __shared__ unsigned long long sm_keys[kWarpsPerBlock][kSortSmem];
+    const SortEntry<R> &e = P.e[blockIdx.y];
+    sort_medium_leaves<R>(e.a, e.d, e.t, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, e.a.nleaf,
+                          ((int64_t)gridDim.x * blockDim.x) >> 5, sm_keys[threadIdx.x >> 5]);
+}
+template <typename R> __global__ void __launch_bounds__(512) k_sort_big(const __grid_constant__ SortPair<R> P) {
+    extern __shared__ unsigned long long bk[];
+    __shared__ R red_hi[16], red_lo[16];
+    const SortEntry<R> &e = P.e[blockIdx.y];
+    sort_big_leaves<R>(e.a, e.d, e.t, blockIdx.x, gridDim.x, bk, red_hi, red_lo);
+}
+
+// ---- the sorts of every (instance, species) of an ensemble, one launch per pass ----------
 template <typename T> __device__ __forceinline__ void copy_words(T &dst, const T &src) {
     static_assert(sizeof(T) % 4 == 0, "word copy");
     const uint32_t *s = reinterpret_cast<const uint32_t *>(&src);
@@ -1210,21 +1227,21 @@ __global__ void k_read(int64_t nleaf, const int32_t *__restrict__ start, const i
     }
 }
 
-// Order the entering regions of every leaf: the warp-per-leaf pass (short regions, and the
-// entering weight sums when a.ent_hi is given), then the long regions (one block each).
-template <typename R> void sort_lists(pic_ctx *ctx, SortArgs a, SoA<R> d, SoA<R> t) {
-    GB_CUDA(cudaMemsetAsync(a.big + a.nleaf, 0, 4, ctx->stream));
-    GB_CUDA(cudaMemsetAsync(a.med + a.nleaf, 0, 4, ctx->stream));
-    k_sort_entering<R><<<(unsigned)std::max<int64_t>(1, std::min<int64_t>((a.nleaf + 31) / 32, 152 * 16)), kT, 0,
-                         ctx->stream>>>(a, d, t);
-    k_sort_medium<R><<<std::min<unsigned>(warp_blocks(a.nleaf), 152u * 8u), kT, 0, ctx->stream>>>(a, d, t);
+// Order the entering regions of every leaf of nsp species: the groups of lanes (short regions),
+// then the queued medium and long ones (their counts are zero before).
+template <typename R> void sort_lists(pic_ctx *ctx, const SortPair<R> &P, int nsp) {
+    const int64_t nl = P.e[0].a.nleaf;
     const size_t smem = (size_t)kSortBig * sizeof(unsigned long long);
     static bool attr = false;  // per R, set once (not while a step is being captured)
     if (!attr) {
         GB_CUDA(cudaFuncSetAttribute(k_sort_big<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         attr = true;
     }
-    k_sort_big<R><<<152, 512, smem, ctx->stream>>>(a, d, t);
+    const unsigned n = (unsigned)nsp;
+    const unsigned ge = (unsigned)std::max<int64_t>(1, std::min<int64_t>((nl + 31) / 32, 152 * 16));
+    k_sort_entering<R><<<dim3(ge, n), kT, 0, ctx->stream>>>(P);
+    k_sort_medium<R><<<dim3(std::min<unsigned>(warp_blocks(nl), 152u * 8u), n), kT, 0, ctx->stream>>>(P);
+    k_sort_big<R><<<dim3(152u / n, n), 512, smem, ctx->stream>>>(P);
     count_launch(ctx, 3);
 }
 
@@ -1288,7 +1305,6 @@ template <typename R> PushArgs<R> push_args(Instance &in, int s, int64_t step) {
     a.err = in.d_err;
     a.self_wrap = (a.px && in.nx0 == 1) || (a.py && in.ny0 == 1);
     a.mcc = c.mcc ? 1 : 0;
-    a.species = s;
     a.ng_dt = (R)(c.gas_density * c.dt);
     a.sig_el = (R)c.sigma_el;
     a.sig_iz0 = (R)c.sigma_iz0;
@@ -1393,25 +1409,27 @@ template <typename R> void step_impl(pic_ctx *ctx, Instance &in, int64_t step, i
     const unsigned full = (unsigned)(bps * sms);
     const unsigned pb = std::min<unsigned>(wb, ctx->capturing ? std::max(1u, full / (unsigned)std::max(1, ctx->tune.graph_div)) : full);
     const bool ionize = mode != PUSH_PREDICT && in.cfg.mcc && in.cfg.sigma_iz0 > 0.0;
-    Species &e = in.sp[0];
     {
         Phase ph(ctx, PIC_PHASE_LISTS);
         step_lists_prep(ctx, in, ionize);
     }
     {
         Phase ph(ctx, PIC_PHASE_MOVE);
+        PushPair<R> P{};
         for (int s = 0; s < nsp; ++s) {
-            PushArgs<R> a = step_push_args<R>(in, s, step, mode);
-            if (ctx->capturing) a.step_dev = ctx->d_step;  // a captured step reads its number on the device
-            if (cic) {
-                if (nt == 128) k_push<R, 128, true><<<pb, 128, push_smem, st>>>(a);
-                else k_push<R, 256, true><<<pb, 256, push_smem, st>>>(a);
-            } else {
-                if (nt == 128) k_push<R, 128, false><<<pb, 128, push_smem, st>>>(a);
-                else k_push<R, 256, false><<<pb, 256, push_smem, st>>>(a);
-            }
-            count_launch(ctx);
+            P.e[s] = step_push_args<R>(in, s, step, mode);
+            if (ctx->capturing) P.e[s].step_dev = ctx->d_step;  // a captured step reads its number on the device
         }
+        P.n0 = pb;
+        const unsigned grid = pb * (unsigned)nsp;
+        if (cic) {
+            if (nt == 128) k_push<R, 128, true><<<grid, 128, push_smem, st>>>(P);
+            else k_push<R, 256, true><<<grid, 256, push_smem, st>>>(P);
+        } else {
+            if (nt == 128) k_push<R, 128, false><<<grid, 128, push_smem, st>>>(P);
+            else k_push<R, 256, false><<<grid, 256, push_smem, st>>>(P);
+        }
+        count_launch(ctx);
     }
     {
         Phase ph(ctx, PIC_PHASE_SCAN);
@@ -1419,15 +1437,18 @@ template <typename R> void step_impl(pic_ctx *ctx, Instance &in, int64_t step, i
     }
     {
         Phase ph(ctx, PIC_PHASE_SORT);
+        SortPair<R> P{};
         for (int s = 0; s < nsp; ++s) {
             Species &sp = in.sp[s];
-            sort_lists<R>(ctx, step_sort_args<R>(in, s, mode), soa<R>(sp, sp.cur), soa<R>(sp, sp.cur ^ 1));
+            P.e[s] = SortEntry<R>{step_sort_args<R>(in, s, mode), soa<R>(sp, sp.cur), soa<R>(sp, sp.cur ^ 1)};
+            P.e[s].a.next_id = in.d_next_id + 1;
             sp.sums_valid = true;
         }
         if (ionize) {
-            k_bump_next_id<<<1, 32, 0, st>>>(in.d_next_id, e.spawn_base + nl);
-            count_launch(ctx);
+            P.next_id = in.d_next_id;
+            P.spawn_total = in.sp[0].spawn_base + nl;
         }
+        sort_lists<R>(ctx, P, nsp);
     }
     check_launch("particle_step");
 }
@@ -1566,10 +1587,17 @@ void particles_load(pic_ctx *ctx, Instance &in, int s, int64_t n, const double *
         }
         count_launch(ctx, 2);
     }
-    if (in.cfg.precision == PIC_FP64)
-        sort_lists<double>(ctx, sort_args<double>(in, sp), soa<double>(sp, 0), soa<double>(sp, 1));
-    else
-        sort_lists<float>(ctx, sort_args<float>(in, sp), soa<float>(sp, 0), soa<float>(sp, 1));
+    GB_CUDA(cudaMemsetAsync(sp.big + nl, 0, 4, st));
+    GB_CUDA(cudaMemsetAsync(sp.moved + nl, 0, 4, st));
+    if (in.cfg.precision == PIC_FP64) {
+        SortPair<double> P{};
+        P.e[0] = SortEntry<double>{sort_args<double>(in, sp), soa<double>(sp, 0), soa<double>(sp, 1)};
+        sort_lists<double>(ctx, P, 1);
+    } else {
+        SortPair<float> P{};
+        P.e[0] = SortEntry<float>{sort_args<float>(in, sp), soa<float>(sp, 0), soa<float>(sp, 1)};
+        sort_lists<float>(ctx, P, 1);
+    }
     unsigned long long nid = next_id;
     if (id) {
         for (int64_t i = 0; i < n; ++i) nid = std::max<unsigned long long>(nid, id[i] + 1);
@@ -1848,8 +1876,10 @@ template <typename R> void batch_prepare_impl(pic_ctx *ctx) {
 
     // shared-memory limits of the batched kernels (set outside the capture)
     const size_t q256 = 8 * sizeof(Queue<R>), q128 = 4 * sizeof(Queue<R>);
-    GB_CUDA(cudaFuncSetAttribute(k_push_batch<R, 256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)q256));
-    GB_CUDA(cudaFuncSetAttribute(k_push_batch<R, 128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)q128));
+    GB_CUDA(cudaFuncSetAttribute(k_push_batch<R, 256, false, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)q256));
+    GB_CUDA(cudaFuncSetAttribute(k_push_batch<R, 128, false, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)q128));
+    GB_CUDA(cudaFuncSetAttribute(k_push_batch<R, 256, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)q256));
+    GB_CUDA(cudaFuncSetAttribute(k_push_batch<R, 128, false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)q128));
     GB_CUDA(cudaFuncSetAttribute(k_sort_big_batch<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(kSortBig * sizeof(unsigned long long))));
 }
@@ -1870,8 +1900,9 @@ template <typename R> void particle_step_batch_impl(pic_ctx *ctx) {
             const BatchTab &t = B.push[s];
             if (!t.n) continue;
             const PushArgs<R> *tab = (const PushArgs<R> *)t.tab;
-            if (nt == 128) k_push_batch<R, 128, false><<<(unsigned)t.nchunks, 128, smem, st>>>(tab, t.chunks);
-            else k_push_batch<R, 256, false><<<(unsigned)t.nchunks, 256, smem, st>>>(tab, t.chunks);
+            auto *k128 = s == 0 ? k_push_batch<R, 128, false, 0> : k_push_batch<R, 128, false, 1>;
+            auto *k256 = s == 0 ? k_push_batch<R, 256, false, 0> : k_push_batch<R, 256, false, 1>;
+            (nt == 128 ? k128 : k256)<<<(unsigned)t.nchunks, (unsigned)nt, smem, st>>>(tab, t.chunks);
             count_launch(ctx);
         }
     }
