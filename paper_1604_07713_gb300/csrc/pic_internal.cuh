@@ -10,6 +10,7 @@
 #include <map>
 #include <unordered_map>
 #include <functional>
+#include <utility>
 #include <vector>
 
 #include "../../include/gbpic.h"
@@ -335,6 +336,30 @@ struct Phase {
 };
 inline void count_launch(pic_ctx *c, int64_t k = 1) { c->launches += k; }
 void check_launch(const char *what);
+
+// Programmatic dependent launch: a kernel of a step's chain lets the next one be scheduled at
+// once and waits, before touching memory that a kernel writes, for the one before it to
+// complete (the waits are no-ops for a kernel launched without the attribute).  Every block of
+// such a kernel calls pdl_chain first, so that completion carries over from kernel to kernel.
+template <typename... KArgs, typename... Args>
+inline void pdl(void (*k)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, Args &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    GB_CUDA(cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...));
+}
+
+__device__ __forceinline__ void pdl_chain() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" :::);
+}
 
 // ------------------------------------------------------------------------------------
 // Device helpers

@@ -89,7 +89,8 @@ __device__ __forceinline__ int32_t leaf_count(const RankEntry &e, int64_t nl, in
 // Blocks (tile, species): the tile's record total; with `fill`, what a step starts from: no
 // entering records, nothing in the overflow store, no moved leaves, the tail not used up, and
 // (electrons with ionization) no spawns counted.
-__global__ void __launch_bounds__(kT) k_lists_sums(RankArgs A) {
+__global__ void __launch_bounds__(kT) k_lists_sums(const __grid_constant__ RankArgs A) {
+    pdl_chain();
     const RankEntry &e = A.e[blockIdx.y];
     int32_t s = 0;
     for (int r = 0; r < A.runs; ++r) {
@@ -125,7 +126,8 @@ __device__ __forceinline__ int32_t tiles_before(const int32_t *__restrict__ part
     return tot;
 }
 // Blocks (tile, species): rank0[L] = records of the leaves before L, rank0[nl] = total.
-__global__ void __launch_bounds__(kT) k_lists_ranks(RankArgs A) {
+__global__ void __launch_bounds__(kT) k_lists_ranks(const __grid_constant__ RankArgs A) {
+    pdl_chain();
     const RankEntry &e = A.e[blockIdx.y];
     int32_t carry = tiles_before(e.part, blockIdx.x);
     for (int r = 0; r < A.runs; ++r) {
@@ -436,6 +438,7 @@ struct RepairArgs {
 
 // Blocks (x, y): y < nsp moves that species' leaves, y == nsp counts the spawns of tile x.
 template <typename R> __global__ void __launch_bounds__(kT) k_step_move(const __grid_constant__ RepairArgs A) {
+    pdl_chain();
     if ((int)blockIdx.y < A.nsp) {
         const ListEntry &e = A.e[blockIdx.y];
         move_to_tail<R>(e.moved, e.nl, e.cap, e.start, e.end, e.lim, e.stay, e.fill, soa_of<R>(e.d), e.key, e.aux,
@@ -452,6 +455,7 @@ template <typename R> __global__ void __launch_bounds__(kT) k_step_move(const __
 }
 // Blocks (x, y): y < nsp places that species' overflow store, y == nsp scans the spawns of tile x.
 template <typename R> __global__ void __launch_bounds__(kT) k_step_place(const __grid_constant__ RepairArgs A) {
+    pdl_chain();
     if ((int)blockIdx.y < A.nsp) {
         const ListEntry &e = A.e[blockIdx.y];
         place_ovf<R>(e.end, e.cap, soa_of<R>(e.o), e.okey, e.oaux, e.odest, e.oslot, soa_of<R>(e.d), e.key, e.aux,
@@ -551,8 +555,8 @@ template <typename R> void step_repairs_impl(pic_ctx *ctx, Instance &in, bool io
         A.spart = in.sp[0].spart + A.tiles;
     }
     const dim3 grid((unsigned)std::max(152, ionize ? A.tiles : 0), (unsigned)(A.nsp + (ionize ? 1 : 0)));
-    k_step_move<R><<<grid, kT, 0, st>>>(A);
-    k_step_place<R><<<grid, kT, 0, st>>>(A);
+    pdl(k_step_move<R>, grid, kT, 0, st, A);
+    pdl(k_step_place<R>, grid, kT, 0, st, A);
     count_launch(ctx, 2);
     if (ctx->capturing) {
         // a captured step of many instances runs them on parallel branches: gated launches
@@ -875,8 +879,8 @@ RankArgs rank_args(Instance &in, int first, int last, bool reset, bool ionize) {
 }
 void launch_ranks(pic_ctx *ctx, const RankArgs &A, int nsp) {
     const dim3 grid((unsigned)leaf_tiles(A.nl), (unsigned)nsp);
-    k_lists_sums<<<grid, kT, 0, ctx->stream>>>(A);
-    k_lists_ranks<<<grid, kT, 0, ctx->stream>>>(A);
+    pdl(k_lists_sums, grid, kT, 0, ctx->stream, A);
+    pdl(k_lists_ranks, grid, kT, 0, ctx->stream, A);
     count_launch(ctx, 2);
     check_launch("list_ranks");
 }

@@ -361,6 +361,7 @@ template <typename T> struct FieldView {
 
 template <typename R>
 __global__ void k_node_e(int64_t n, FieldView<R> F, R *__restrict__ stencil) {
+    pdl_chain();
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= 4 * n) return;
     if (F.wall_dev)
@@ -685,11 +686,11 @@ void node_e(pic_ctx *ctx, Instance &in, const double walls[4]) {
     if (in.cfg.precision == PIC_FP64) {
         FieldView<double> F = field_view<double>(in, walls);
         F.wall_dev = wd;
-        k_node_e<double><<<blocks_for(4 * g.n), kT, 0, ctx->stream>>>(g.n, F, (double *)in.stencil);
+        pdl(k_node_e<double>, blocks_for(4 * g.n), kT, 0, ctx->stream, g.n, F, (double *)in.stencil);
     } else {
         FieldView<float> F = field_view<float>(in, walls);
         F.wall_dev = wd;
-        k_node_e<float><<<blocks_for(4 * g.n), kT, 0, ctx->stream>>>(g.n, F, (float *)in.stencil);
+        pdl(k_node_e<float>, blocks_for(4 * g.n), kT, 0, ctx->stream, g.n, F, (float *)in.stencil);
     }
     count_launch(ctx);
     check_launch("node_e");

@@ -167,6 +167,7 @@ __device__ __forceinline__ void deposit_sums_leaf(const DepositArgs &a, const Le
 }
 template <typename R>
 __global__ void k_deposit_sums(DepositArgs a, LeafSums w0, LeafSums w1) {
+    pdl_chain();
     const int64_t L = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (L < a.nleaf) deposit_sums_leaf<R>(a, w0, w1, L);
 }
@@ -644,6 +645,7 @@ template <typename R> struct PushPair {
 };
 template <typename R, int NT, bool CIC>
 __global__ void __launch_bounds__(NT, 768 / NT) k_push(const __grid_constant__ PushPair<R> P) {
+    pdl_chain();
     extern __shared__ unsigned char push_smem[];
     Queue<R> &q = reinterpret_cast<Queue<R> *>(push_smem)[threadIdx.x >> 5];
     if (blockIdx.x < P.n0) {
@@ -1035,6 +1037,7 @@ template <typename R> struct SortPair {
     const int32_t *spawn_total;
 };
 template <typename R> __global__ void __launch_bounds__(kT) k_sort_entering(const __grid_constant__ SortPair<R> P) {
+    pdl_chain();
     const SortEntry<R> &e = P.e[blockIdx.y];
     if (P.next_id && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
         P.next_id[0] = P.next_id[1] + 2ull * (unsigned long long)(*P.spawn_total);
@@ -1042,12 +1045,14 @@ template <typename R> __global__ void __launch_bounds__(kT) k_sort_entering(cons
                             ((int64_t)gridDim.x * blockDim.x) >> 5);
 }
 template <typename R> __global__ void __launch_bounds__(kT, 3) k_sort_medium(const __grid_constant__ SortPair<R> P) {
+    pdl_chain();
     __shared__ unsigned long long sm_keys[kWarpsPerBlock][kSortSmem];
     const SortEntry<R> &e = P.e[blockIdx.y];
     sort_medium_leaves<R>(e.a, e.d, e.t, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, e.a.nleaf,
                           ((int64_t)gridDim.x * blockDim.x) >> 5, sm_keys[threadIdx.x >> 5]);
 }
 template <typename R> __global__ void __launch_bounds__(512) k_sort_big(const __grid_constant__ SortPair<R> P) {
+    pdl_chain();
     extern __shared__ unsigned long long bk[];
     __shared__ R red_hi[16], red_lo[16];
     const SortEntry<R> &e = P.e[blockIdx.y];
@@ -1239,9 +1244,9 @@ template <typename R> void sort_lists(pic_ctx *ctx, const SortPair<R> &P, int ns
     }
     const unsigned n = (unsigned)nsp;
     const unsigned ge = (unsigned)std::max<int64_t>(1, std::min<int64_t>((nl + 31) / 32, 152 * 16));
-    k_sort_entering<R><<<dim3(ge, n), kT, 0, ctx->stream>>>(P);
-    k_sort_medium<R><<<dim3(std::min<unsigned>(warp_blocks(nl), 152u * 8u), n), kT, 0, ctx->stream>>>(P);
-    k_sort_big<R><<<dim3(152u / n, n), 512, smem, ctx->stream>>>(P);
+    pdl(k_sort_entering<R>, dim3(ge, n), kT, 0, ctx->stream, P);
+    pdl(k_sort_medium<R>, dim3(std::min<unsigned>(warp_blocks(nl), 152u * 8u), n), kT, 0, ctx->stream, P);
+    pdl(k_sort_big<R>, dim3(152u / n, n), 512, smem, ctx->stream, P);
     count_launch(ctx, 3);
 }
 
@@ -1423,11 +1428,11 @@ template <typename R> void step_impl(pic_ctx *ctx, Instance &in, int64_t step, i
         P.n0 = pb;
         const unsigned grid = pb * (unsigned)nsp;
         if (cic) {
-            if (nt == 128) k_push<R, 128, true><<<grid, 128, push_smem, st>>>(P);
-            else k_push<R, 256, true><<<grid, 256, push_smem, st>>>(P);
+            if (nt == 128) pdl(k_push<R, 128, true>, grid, 128, push_smem, st, P);
+            else pdl(k_push<R, 256, true>, grid, 256, push_smem, st, P);
         } else {
-            if (nt == 128) k_push<R, 128, false><<<grid, 128, push_smem, st>>>(P);
-            else k_push<R, 256, false><<<grid, 256, push_smem, st>>>(P);
+            if (nt == 128) pdl(k_push<R, 128, false>, grid, 128, push_smem, st, P);
+            else pdl(k_push<R, 256, false>, grid, 256, push_smem, st, P);
         }
         count_launch(ctx);
     }
@@ -1648,9 +1653,9 @@ void deposit(pic_ctx *ctx, Instance &in, const double walls[4]) {
         const LeafSums w0{in.sp[0].stay_hi, in.sp[0].stay_lo, in.sp[0].ent_hi, in.sp[0].ent_lo};
         const LeafSums w1{s1.stay_hi, s1.stay_lo, s1.ent_hi, s1.ent_lo};
         if (in.cfg.precision == PIC_FP64)
-            k_deposit_sums<double><<<blocks_for(in.nleaf), kT, 0, ctx->stream>>>(a, w0, w1);
+            pdl(k_deposit_sums<double>, blocks_for(in.nleaf), kT, 0, ctx->stream, a, w0, w1);
         else
-            k_deposit_sums<float><<<blocks_for(in.nleaf), kT, 0, ctx->stream>>>(a, w0, w1);
+            pdl(k_deposit_sums<float>, blocks_for(in.nleaf), kT, 0, ctx->stream, a, w0, w1);
     }
     else if (in.cfg.precision == PIC_FP64)
         k_deposit<double><<<warp_blocks(in.nleaf), kT, 0, ctx->stream>>>(a);

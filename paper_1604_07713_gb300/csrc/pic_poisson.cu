@@ -27,30 +27,6 @@ constexpr double kCoarseTol2 = 1e-10;  // coarsest solve (multi-block path): ||r
 constexpr float kSmCoarseTol2 = 1e-6f; // coarsest solve inside a V-cycle in shared memory: 1e-3
 inline unsigned blocks_for(int64_t n, int t = kT) { return (unsigned)std::max<int64_t>(1, (n + t - 1) / t); }
 
-// Launch with programmatic stream serialization (the kernel calls pdl_chain first).
-template <typename... KArgs, typename... Args>
-void pdl(void (*k)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, Args &&...args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    GB_CUDA(cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...));
-}
-
-// Programmatic dependent launch: a kernel of the solve's chain lets the next one be scheduled
-// at once and waits, before touching memory, for the previous one to complete (the waits are
-// no-ops for a kernel launched without the programmatic-serialization attribute).
-__device__ __forceinline__ void pdl_chain() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" :::);
-}
-
 __device__ __forceinline__ double block_sum(double v) {
     __shared__ double sh[32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -985,6 +961,7 @@ __global__ void __launch_bounds__(1024, 1) k_small_solve(const SmallSolve *__res
         for (int k = threadIdx.x; k < D.inv_words; k += 1024) cs[k] = inv[k];
         inv = cs;
     }
+    pdl_chain();  // what came before it reads is constant between mesh changes
     float *lsm = cl.map_shared_rank(sm, 0);  // the leader's levels
     double *lpart = cl.map_shared_rank(part, 0);
     const double *lmean = cl.map_shared_rank(&mean_sh, 0);
@@ -1109,9 +1086,12 @@ cudaLaunchConfig_t small_config(int n_items, int C, size_t smem, cudaLaunchAttri
 
 // One launch of the small solve: n_items clusters of C CTAs.
 void launch_small_solve(const void *items, int n_items, int C, int nbuf, size_t smem, cudaStream_t st) {
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = small_config(n_items, C, smem, attr);
     cfg.stream = st;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
     GB_CUDA(cudaLaunchKernelEx(&cfg, k_small_solve, (const SmallSolve *)items, nbuf));
 }
 
