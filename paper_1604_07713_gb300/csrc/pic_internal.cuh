@@ -79,6 +79,7 @@ struct Level {
     int32_t *child4 = nullptr;             // cell -> up to 4 cells of the next finer level
     int32_t *col = nullptr;                // ELL off-diagonal columns [kEll * n], -1 = empty
     float *val = nullptr;                  // ELL off-diagonal values (FP32)
+    uint16_t *code = nullptr;              // kappa = 1: two bits per ELL slot (0 empty, 1: -1, 2: -2/3, 3: 1/3)
     float *dinv = nullptr;                 // 1 / diagonal (FP32)
     uint8_t *color = nullptr;              // red-black colour of the cell on its own scale
     double *val64 = nullptr, *diag64 = nullptr;  // finest level only (FP64 residual)
@@ -193,7 +194,7 @@ struct Instance {
     uint32_t *root = nullptr;    // per leaf
     uint32_t *morton = nullptr;  // per leaf
     std::vector<Level> lv;       // lv[0] = the leaves
-    double *phi = nullptr, *bvec = nullptr, *res = nullptr, *charge = nullptr;
+    double *phi = nullptr, *bvec = nullptr, *charge = nullptr;
     double *phi_prev = nullptr;  // previous solution: the next solve starts from 2 phi - phi_prev
     int n_solves = 0;            // solves since the mesh was set (extrapolation needs two)
     int32_t *d_n_solves = nullptr;  // the same count on the device, for meshes solved in one launch

@@ -148,7 +148,7 @@ __global__ void k_check_balance(int64_t n, LatView L, int32_t *__restrict__ err)
 __global__ void k_assemble(int64_t n, LatView L, int bcx, int bcy, int32_t *__restrict__ col,
                            float *__restrict__ val, float *__restrict__ dinv, double *__restrict__ val64,
                            double *__restrict__ diag64, double *__restrict__ bcw, uint8_t *__restrict__ color,
-                           int32_t *__restrict__ err, const double *__restrict__ kappa) {
+                           int32_t *__restrict__ err, const double *__restrict__ kappa, uint16_t *__restrict__ code) {
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= n) return;
     {
@@ -210,6 +210,11 @@ __global__ void k_assemble(int64_t n, LatView L, int bcx, int bcy, int32_t *__re
         default:
             atomicExch(err, 5);
         }
+    }
+    if (code) {  // kappa = 1: the values by number
+        uint32_t m = 0;
+        for (int j = 0; j < k; ++j) m |= (vv[j] == -1.0 ? 1u : (vv[j] < 0.0 ? 2u : 3u)) << (2 * j);
+        code[c] = (uint16_t)m;
     }
     for (int j = 0; j < kEll; ++j) {
         const int32_t cj = j < k ? cc[j] : -1;
@@ -407,6 +412,7 @@ void assemble_level(pic_ctx *ctx, Instance &in, Level &g, bool finest, int32_t *
     g.col = dalloc<int32_t>(A, kEll * g.n);
     g.val = dalloc<float>(A, kEll * g.n);
     g.dinv = dalloc<float>(A, g.n);
+    g.code = dalloc<uint16_t>(A, g.n);
     g.color = dalloc<uint8_t>(A, g.n);
     if (finest) {
         g.val64 = dalloc<double>(A, kEll * g.n);
@@ -419,7 +425,7 @@ void assemble_level(pic_ctx *ctx, Instance &in, Level &g, bool finest, int32_t *
     g.kappa = in.cfg.implicit ? dalloc<double>(A, g.n) : nullptr;  // set per step (poisson_kappa)
     k_assemble<<<blocks_for(g.n), kT, 0, ctx->stream>>>(g.n, view_of(in, g), in.cfg.bc_x, in.cfg.bc_y, g.col,
                                                         g.val, g.dinv, g.val64, g.diag64, g.bcw, g.color, d_err,
-                                                        nullptr);
+                                                        nullptr, g.code);
     count_launch(ctx);
 }
 
@@ -668,7 +674,7 @@ void poisson_kappa(pic_ctx *ctx, Instance &in, const double walls[4]) {
     for (size_t g = 0; g < in.lv.size(); ++g) {
         Level &L = in.lv[g];
         k_assemble<<<blocks_for(L.n), kT, 0, st>>>(L.n, view_of(in, L), in.cfg.bc_x, in.cfg.bc_y, L.col, L.val,
-                                                   L.dinv, L.val64, L.diag64, L.bcw, L.color, in.d_err, L.kappa);
+                                                   L.dinv, L.val64, L.diag64, L.bcw, L.color, in.d_err, L.kappa, nullptr);
         count_launch(ctx);
     }
     const Level &F = in.lv[0];

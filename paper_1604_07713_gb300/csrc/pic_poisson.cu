@@ -62,14 +62,19 @@ __device__ __forceinline__ double worst_residual(double a, double b) {
     return (a != a || b != b) ? __longlong_as_double(0x7FF8000000000000ll) : fmax(a, b);
 }
 
+// The off-diagonal value a code stands for (LevelOp).
+template <typename T> __device__ __forceinline__ T op_value(uint32_t k) {
+    return k == 1u ? (T)-1 : (k == 2u ? (T)(-2.0 / 3.0) : (T)(1.0 / 3.0));
+}
+
 // r = b - A phi (FP64) with r^2 and b^2 summed per block (fixed grid), then, in the block that
 // arrives last on the ticket counter (after a fence, so every block's sums are visible), the
 // block sums added as k_finish_sums adds them, the solve's statistics and whether another
 // cycle runs (the condition of the graph's WHILE node; first = 1 before the first cycle),
 // and the counter reset for the next launch.
-__global__ void k_residual_decide(int64_t n, const int32_t *__restrict__ col, const double *__restrict__ val,
-                                  const double *__restrict__ diag, const double *__restrict__ phi,
-                                  const double *__restrict__ b, double *__restrict__ r, float *__restrict__ r32,
+__global__ void k_residual_decide(int64_t n, const int32_t *__restrict__ col, const uint16_t *__restrict__ code,
+                                  const double *__restrict__ val, const double *__restrict__ diag, const double *__restrict__ phi,
+                                  const double *__restrict__ b, float *__restrict__ r32,
                                   double *__restrict__ part, uint32_t *__restrict__ ticket,
                                   cudaGraphConditionalHandle h, double tol, int maxc, double *__restrict__ stats,
                                   int first) {
@@ -78,13 +83,19 @@ __global__ void k_residual_decide(int64_t n, const int32_t *__restrict__ col, co
     double rr = 0.0, bb = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         double ax = diag[i] * phi[i];
+        if (code) {
+            const uint32_t m = code[i];
 #pragma unroll
-        for (int j = 0; j < kEll; ++j) {
-            const int32_t c = col[(int64_t)j * n + i];
-            if (c >= 0) ax += val[(int64_t)j * n + i] * phi[c];
+            for (int j = 0; j < kEll; ++j)
+                if ((m >> (2 * j)) & 3u) ax += op_value<double>((m >> (2 * j)) & 3u) * phi[col[(int64_t)j * n + i]];
+        } else {
+#pragma unroll
+            for (int j = 0; j < kEll; ++j) {
+                const int32_t c = col[(int64_t)j * n + i];
+                if (c >= 0) ax += val[(int64_t)j * n + i] * phi[c];
+            }
         }
         const double ri = b[i] - ax;
-        r[i] = ri;
         r32[i] = (float)ri;
         rr += ri * ri;
         bb += b[i] * b[i];
@@ -165,108 +176,184 @@ __global__ void k_extrapolate(int64_t n, double *__restrict__ phi, double *__res
     prev[i] = p;
 }
 
-__global__ void k_add_correction(int64_t n, const float *__restrict__ e, double *__restrict__ phi) {
-    pdl_chain();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) phi[i] += (double)e[i];
+// The rows of a level swept by many blocks.  An explicit scheme's off-diagonal values are -1
+// (same level), -2/3 (across a level step) and 1/3 (the sibling there): `code` holds two bits
+// per ELL slot (0: empty), so a row is read as 2 bytes and its 4 to 8 columns instead of 64
+// bytes.  The implicit scheme's values come from `val` (code null).
+struct LevelOp {
+    int64_t n;
+    const int32_t *col;
+    const uint16_t *code;
+    const float *val, *dinv;
+    const uint8_t *color;
+};
+struct OpRow {
+    int32_t c[kEll];
+    float v[kEll];
+};
+template <bool CODED> __device__ __forceinline__ void op_row(const LevelOp &A, int64_t i, OpRow &r) {
+    if constexpr (CODED) {
+        const uint32_t m = A.code[i];
+#pragma unroll
+        for (int j = 0; j < kEll; ++j) {
+            const uint32_t k = (m >> (2 * j)) & 3u;
+            r.c[j] = k ? A.col[(int64_t)j * A.n + i] : -1;
+            r.v[j] = op_value<float>(k);
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < kEll; ++j) {
+            r.c[j] = A.col[(int64_t)j * A.n + i];
+            r.v[j] = A.val[(int64_t)j * A.n + i];
+        }
+    }
 }
+
+// Each of the following kernels of a cycle loads what no kernel of the cycle writes (operator,
+// colours, parents) and what was written two or more kernels earlier before it waits for its
+// predecessor, so that after the wait one gather, a few additions and a store are left: the
+// solve is a chain of dozens of such kernels, bound by their latency.  Early streamer (24,500
+// leaves, ~2 cycles): 0.303 -> 0.217 ms per solve; 256 x 256 periodic, 6 cycles: 0.566 -> 0.407 ms.
 
 // One colour of a red-black Gauss-Seidel sweep, written out of place so that the result does
 // not depend on thread order (cells of the same colour can touch on a non-uniform mesh):
-// colour-c cells get D^-1 (b - offdiag x_in), others copy x_in.  zero_in: x_in is zero.
-__global__ void k_rbgs_half(int64_t n, const int32_t *__restrict__ col, const float *__restrict__ val,
-                            const float *__restrict__ dinv, const uint8_t *__restrict__ color, int c,
-                            const float *__restrict__ b, const float *__restrict__ xin, float *__restrict__ xout,
-                            int zero_in) {
-    pdl_chain();
+// colour-c cells get D^-1 (b - offdiag x_in), others copy x_in.  With phi non-null (the
+// finest level's last half sweep of a cycle) the result is also added to the potential.
+template <bool CODED>
+__global__ void __launch_bounds__(kT) k_rbgs_half(const LevelOp A, int c, const float *__restrict__ b,
+                                                  const float *__restrict__ xin, float *__restrict__ xout,
+                                                  double *__restrict__ phi) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (color[i] != c) {
-        xout[i] = zero_in ? 0.0f : xin[i];
-        return;
+    const bool in = i < A.n, mine = in && A.color[i] == c;
+    OpRow r;
+    float bi = 0.0f, di = 0.0f;
+    if (mine) {
+        op_row<CODED>(A, i, r);
+        bi = b[i];
+        di = A.dinv[i];
     }
-    float off = 0.0f;
-    if (!zero_in) {
+    pdl_chain();
+    if (!in) return;
+    float x;
+    if (mine) {
+        float off = 0.0f;
 #pragma unroll
-        for (int j = 0; j < kEll; ++j) {
-            const int32_t cc = col[(int64_t)j * n + i];
-            if (cc >= 0) off = fmaf(val[(int64_t)j * n + i], xin[cc], off);
-        }
+        for (int j = 0; j < kEll; ++j)
+            if (r.c[j] >= 0) off = fmaf(r.v[j], xin[r.c[j]], off);
+        x = di * (bi - off);
+    } else {
+        x = xin[i];
     }
-    xout[i] = dinv[i] * (b[i] - off);
+    xout[i] = x;
+    if (phi) phi[i] += (double)x;
 }
 
 // The first two half sweeps of a pre-smoothing from x = 0 in one kernel: the first (colour 0
 // from zero) leaves t = D^-1 (b - 0) on colour 0 and 0 elsewhere, which the second (colour 1)
 // forms on the fly; the same arithmetic as the two half sweeps, so the same values.
-__global__ void k_rbgs_first(int64_t n, const int32_t *__restrict__ col, const float *__restrict__ val,
-                             const float *__restrict__ dinv, const uint8_t *__restrict__ color,
-                             const float *__restrict__ b, float *__restrict__ xout) {
-    pdl_chain();
+template <bool CODED>
+__global__ void __launch_bounds__(kT) k_rbgs_first(const LevelOp A, const float *__restrict__ b, float *__restrict__ xout) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (color[i] != 1) {
-        xout[i] = dinv[i] * (b[i] - 0.0f);
+    const bool in = i < A.n, mine = in && A.color[i] == 1;
+    OpRow r;
+    float dn[kEll], di = 0.0f;
+    if (in) di = A.dinv[i];
+    if (mine) {
+        op_row<CODED>(A, i, r);
+#pragma unroll
+        for (int j = 0; j < kEll; ++j) {
+            dn[j] = 0.0f;
+            if (r.c[j] >= 0) {
+                if (A.color[r.c[j]] == 0) dn[j] = A.dinv[r.c[j]];
+                else r.c[j] = -2;  // its value is zero: the term is v * 0
+            }
+        }
+    }
+    pdl_chain();
+    if (!in) return;
+    if (!mine) {
+        xout[i] = di * (b[i] - 0.0f);
         return;
     }
     float off = 0.0f;
 #pragma unroll
     for (int j = 0; j < kEll; ++j) {
-        const int32_t cc = col[(int64_t)j * n + i];
-        if (cc >= 0) off = fmaf(val[(int64_t)j * n + i], color[cc] == 0 ? dinv[cc] * (b[cc] - 0.0f) : 0.0f, off);
+        if (r.c[j] >= 0) off = fmaf(r.v[j], dn[j] * (b[r.c[j]] - 0.0f), off);
+        else if (r.c[j] == -2) off = fmaf(r.v[j], 0.0f, off);
     }
-    xout[i] = dinv[i] * (b[i] - off);
+    xout[i] = di * (b[i] - off);
 }
 
 // Injection of the coarse correction (x += xc[parent]) fused into the first half sweep after
-// it: every value the sweep reads gets its correction added on the way, with the same
-// additions as a separate injection pass.
-__global__ void k_rbgs_half_prolong(int64_t n, const int32_t *__restrict__ col, const float *__restrict__ val,
-                                    const float *__restrict__ dinv, const uint8_t *__restrict__ color, int c,
-                                    const float *__restrict__ b, const float *__restrict__ xin,
-                                    const int32_t *__restrict__ parent, const float *__restrict__ xc,
-                                    float *__restrict__ xout) {
-    pdl_chain();
+// it (colour 0): every value the sweep reads gets its correction added on the way, with the
+// same additions as a separate injection pass.
+template <bool CODED>
+__global__ void __launch_bounds__(kT) k_rbgs_half_prolong(const LevelOp A, const float *__restrict__ b,
+                                                          const float *__restrict__ xin,
+                                                          const int32_t *__restrict__ parent,
+                                                          const float *__restrict__ xc, float *__restrict__ xout) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (color[i] != c) {
-        xout[i] = xin[i] + xc[parent[i]];
+    const bool in = i < A.n, mine = in && A.color[i] == 0;
+    OpRow r;
+    float xn[kEll], bi = 0.0f, di = 0.0f, xi = 0.0f;
+    int32_t pi = 0;
+    if (mine) {
+        op_row<CODED>(A, i, r);
+        bi = b[i];
+        di = A.dinv[i];
+#pragma unroll
+        for (int j = 0; j < kEll; ++j) {
+            xn[j] = 0.0f;
+            if (r.c[j] >= 0) {
+                xn[j] = xin[r.c[j]];
+                r.c[j] = parent[r.c[j]];
+            }
+        }
+    } else if (in) {
+        pi = parent[i];
+        xi = xin[i];
+    }
+    pdl_chain();
+    if (!in) return;
+    if (!mine) {
+        xout[i] = xi + xc[pi];
         return;
     }
     float off = 0.0f;
 #pragma unroll
-    for (int j = 0; j < kEll; ++j) {
-        const int32_t cc = col[(int64_t)j * n + i];
-        if (cc >= 0) off = fmaf(val[(int64_t)j * n + i], xin[cc] + xc[parent[cc]], off);
-    }
-    xout[i] = dinv[i] * (b[i] - off);
+    for (int j = 0; j < kEll; ++j)
+        if (r.c[j] >= 0) off = fmaf(r.v[j], xn[j] + xc[r.c[j]], off);
+    xout[i] = di * (bi - off);
 }
 
-// Coarse right-hand side: summed residuals of the children; zero coarse iterate.
-__global__ void k_restrict_residual(int64_t nc, const int32_t *__restrict__ child4, int64_t nf,
-                                    const int32_t *__restrict__ col, const float *__restrict__ val,
-                                    const float *__restrict__ dinv, const float *__restrict__ bf,
-                                    const float *__restrict__ xf, float *__restrict__ bc, float *__restrict__ xc) {
+// Coarse right-hand side: summed residuals of the children (four threads per coarse cell, one
+// child each, added in child order).
+template <bool CODED>
+__global__ void __launch_bounds__(kT) k_restrict_residual(int64_t nc, const int32_t *__restrict__ child4,
+                                                          const LevelOp A, const float *__restrict__ bf,
+                                                          const float *__restrict__ xf, float *__restrict__ bc) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int32_t i = t < 4 * nc ? child4[t] : -1;
+    OpRow r;
+    float bi = 0.0f, di = 1.0f;
+    if (i >= 0) {
+        op_row<CODED>(A, i, r);
+        bi = bf[i];
+        di = A.dinv[i];
+    }
     pdl_chain();
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= nc) return;
-    float s = 0.0f;
+    float res = 0.0f;
+    if (i >= 0) {
+        float ax = xf[i] / di;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int32_t i = child4[4 * p + k];
-        if (i < 0) continue;
-        float ax = xf[i] / dinv[i];
-#pragma unroll
-        for (int j = 0; j < kEll; ++j) {
-            const int32_t c = col[(int64_t)j * nf + i];
-            if (c >= 0) ax = fmaf(val[(int64_t)j * nf + i], xf[c], ax);
-        }
-        s += bf[i] - ax;
+        for (int j = 0; j < kEll; ++j)
+            if (r.c[j] >= 0) ax = fmaf(r.v[j], xf[r.c[j]], ax);
+        res = bi - ax;
     }
-    bc[p] = s;
-    xc[p] = 0.0f;
+    const float r1 = __shfl_down_sync(0xFFFFFFFFu, res, 1, 4), r2 = __shfl_down_sync(0xFFFFFFFFu, res, 2, 4),
+                r3 = __shfl_down_sync(0xFFFFFFFFu, res, 3, 4);
+    if (t < 4 * nc && (t & 3) == 0) bc[t >> 2] = ((res + r1) + r2) + r3;
 }
-
 
 // One-block Jacobi-preconditioned CG on the coarsest level (symmetric: one uniform level).
 __global__ void __launch_bounds__(1024) k_coarse_cg(int64_t n, const int32_t *__restrict__ col,
@@ -1175,6 +1262,8 @@ SmallDesc small_desc(const Instance &in, int g0) {
     return D;
 }
 
+template <bool CODED> void level_cycle(pic_ctx *ctx, Instance &in, size_t g, bool singular);
+
 void vcycle(pic_ctx *ctx, Instance &in, size_t g, bool singular) {
     Level &L = in.lv[g];
     cudaStream_t s = ctx->stream;
@@ -1194,28 +1283,35 @@ void vcycle(pic_ctx *ctx, Instance &in, size_t g, bool singular) {
         count_launch(ctx);
         return;
     }
-    Level &C = in.lv[g + 1];
+    if (in.cfg.implicit) level_cycle<false>(ctx, in, g, singular);
+    else level_cycle<true>(ctx, in, g, singular);
+}
+
+// The sweeps of level g around the coarser levels' cycle.
+template <bool CODED> void level_cycle(pic_ctx *ctx, Instance &in, size_t g, bool singular) {
+    Level &L = in.lv[g], &C = in.lv[g + 1];
+    cudaStream_t s = ctx->stream;
+    const LevelOp A{L.n, L.col, L.code, L.val, L.dinv, L.color};
     const unsigned nb = blocks_for(L.n);
+    double *none = nullptr;
     // pre-smoothing (x starts at zero): the first sweep's two half sweeps in one kernel
-    pdl(k_rbgs_first, nb, kT, 0, s, L.n, L.col, L.val, L.dinv, L.color, L.b, L.x);
+    pdl(k_rbgs_first<CODED>, nb, kT, 0, s, A, L.b, L.x);
     for (int k = 1; k < kNu; ++k)
         for (int c = 0; c < 2; ++c) {
-            pdl(k_rbgs_half, nb, kT, 0, s, L.n, L.col, L.val, L.dinv, L.color, c, L.b, L.x, L.t, 0);
+            pdl(k_rbgs_half<CODED>, nb, kT, 0, s, A, c, L.b, L.x, L.t, none);
             std::swap(L.x, L.t);
         }
-    pdl(k_restrict_residual, blocks_for(C.n), kT, 0, s, C.n, C.child4, L.n, L.col, L.val, L.dinv, L.b, L.x, C.b, C.x);
+    pdl(k_restrict_residual<CODED>, blocks_for(4 * C.n), kT, 0, s, C.n, C.child4, A, L.b, L.x, C.b);
     count_launch(ctx, 2 * kNu);
     vcycle(ctx, in, g + 1, singular);
-    // post-smoothing, the injection of the correction fused into its first half sweep
-    pdl(k_rbgs_half_prolong, nb, kT, 0, s, L.n, L.col, L.val, L.dinv, L.color, 0, L.b, L.x, L.parent, C.x, L.t);
+    // post-smoothing, the injection of the correction fused into its first half sweep; the last
+    // one of the finest level adds its result to the potential
+    pdl(k_rbgs_half_prolong<CODED>, nb, kT, 0, s, A, L.b, L.x, L.parent, C.x, L.t);
     std::swap(L.x, L.t);
-    pdl(k_rbgs_half, nb, kT, 0, s, L.n, L.col, L.val, L.dinv, L.color, 1, L.b, L.x, L.t, 0);
-    std::swap(L.x, L.t);
-    for (int k = 1; k < kNu; ++k)
-        for (int c = 0; c < 2; ++c) {
-            pdl(k_rbgs_half, nb, kT, 0, s, L.n, L.col, L.val, L.dinv, L.color, c, L.b, L.x, L.t, 0);
-            std::swap(L.x, L.t);
-        }
+    for (int h = 1; h < 2 * kNu; ++h) {
+        pdl(k_rbgs_half<CODED>, nb, kT, 0, s, A, h & 1, L.b, L.x, L.t, g == 0 && h == 2 * kNu - 1 ? in.phi : none);
+        std::swap(L.x, L.t);
+    }
     count_launch(ctx, 2 * kNu);
 }
 }  // namespace
@@ -1303,7 +1399,6 @@ void poisson_setup(pic_ctx *ctx, Instance &in) {
     in.n_solves = 0;
     in.d_n_solves = nullptr;
     in.bvec = dalloc<double>(A, n);
-    in.res = dalloc<double>(A, n);
     in.charge = dalloc<double>(A, n);
     in.red = dalloc<double>(A, 2 * kRedBlocks + 8);  // block sums, totals, the residual's ticket
     GB_CUDA(cudaMemsetAsync(in.red, 0, (2 * kRedBlocks + 8) * sizeof(double), ctx->stream));
@@ -1426,21 +1521,13 @@ void poisson_solve(pic_ctx *ctx, Instance &in, const double walls[4]) {
     const int maxc = std::max(1, in.cfg.mg_max_cycles);
     // launches go to ctx->stream, which is the capture stream while the solve is captured
     auto issue_residual = [&](int first, cudaGraphConditionalHandle h) {
-        pdl(k_residual_decide, kRedBlocks, kT, 0, ctx->stream, n, L.col, L.val64, L.diag64, in.phi, in.bvec, in.res, L.b,
-                                                              in.red, (uint32_t *)(in.red + 2 * kRedBlocks + 4), h,
-                                                              in.cfg.mg_rel_tol, maxc, in.mg_stats, first);
+        pdl(k_residual_decide, kRedBlocks, kT, 0, ctx->stream, n, L.col, in.cfg.implicit ? nullptr : L.code, L.val64,
+            L.diag64, in.phi, in.bvec, L.b, in.red, (uint32_t *)(in.red + 2 * kRedBlocks + 4), h, in.cfg.mg_rel_tol, maxc,
+            in.mg_stats, first);
         count_launch(ctx);
     };
     auto issue_cycle = [&](cudaGraphConditionalHandle h) {
-        vcycle(ctx, in, 0, singular);
-        pdl(k_add_correction, blocks_for(n), kT, 0, ctx->stream, n, L.x, in.phi);
-        count_launch(ctx);
-        if (singular) {
-            pdl(k_area_weighted, kRedBlocks, kT, 0, ctx->stream, n, L.lev, L.lmax, in.phi, in.red);
-            pdl(k_finish_sums, 1, 32, 0, ctx->stream, kRedBlocks, in.red, in.red + 2 * kRedBlocks);
-            pdl(k_project, blocks_for(n), kT, 0, ctx->stream, n, L.lev, L.lmax, in.red + 2 * kRedBlocks, in.phi, 1);
-            count_launch(ctx, 3);
-        }
+        vcycle(ctx, in, 0, singular);  // (adds its correction to phi)
         issue_residual(0, h);
     };
     if (!in.mg_cycle) {
@@ -1499,6 +1586,12 @@ void poisson_solve(pic_ctx *ctx, Instance &in, const double walls[4]) {
     }
     GB_CUDA(cudaGraphLaunch(in.mg_cycle, s));
     count_launch(ctx, in.mg_pre_nodes);  // the cycles' launches are counted when the stats are read
+    if (singular) {  // zero area-weighted mean (a constant changes no residual: once, after the cycles)
+        k_area_weighted<<<kRedBlocks, kT, 0, s>>>(n, L.lev, L.lmax, in.phi, in.red);
+        pdl(k_finish_sums, 1, 32, 0, s, kRedBlocks, in.red, in.red + 2 * kRedBlocks);
+        pdl(k_project, blocks_for(n), kT, 0, s, n, L.lev, L.lmax, in.red + 2 * kRedBlocks, in.phi, 1);
+        count_launch(ctx, 3);
+    }
     in.mg_on_device = true;
     in.mg_count_cycles = true;
     check_launch("poisson_solve");
