@@ -27,18 +27,17 @@ constexpr double kCoarseTol2 = 1e-10;  // coarsest solve (multi-block path): ||r
 constexpr float kSmCoarseTol2 = 1e-6f; // coarsest solve inside a V-cycle in shared memory: 1e-3
 inline unsigned blocks_for(int64_t n, int t = kT) { return (unsigned)std::max<int64_t>(1, (n + t - 1) / t); }
 
+// Sum over a block of kT threads as a fixed tree, valid in thread 0.
 __device__ __forceinline__ double block_sum(double v) {
-    __shared__ double sh[32];
+    __shared__ double sh[kT / 32];
+    static_assert(kT == 256, "eight warps");
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, o);
+    __syncthreads();  // (the previous sum's words are read)
     if (lane == 0) sh[wid] = v;
     __syncthreads();
-    double s = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh[w];
-    __syncthreads();
-    return s;  // valid in thread 0
+    return ((sh[0] + sh[1]) + (sh[2] + sh[3])) + ((sh[4] + sh[5]) + (sh[6] + sh[7]));
 }
 
 // out = sums of the block partials (one warp: lanes in a fixed order, then a fixed tree,
@@ -67,17 +66,20 @@ template <typename T> __device__ __forceinline__ T op_value(uint32_t k) {
     return k == 1u ? (T)-1 : (k == 2u ? (T)(-2.0 / 3.0) : (T)(1.0 / 3.0));
 }
 
-// r = b - A phi (FP64) with r^2 and b^2 summed per block (fixed grid), then, in the block that
-// arrives last on the ticket counter (after a fence, so every block's sums are visible), the
-// block sums added as k_finish_sums adds them, the solve's statistics and whether another
-// cycle runs (the condition of the graph's WHILE node; first = 1 before the first cycle),
-// and the counter reset for the next launch.
-__global__ void k_residual_decide(int64_t n, const int32_t *__restrict__ col, const uint16_t *__restrict__ code,
-                                  const double *__restrict__ val, const double *__restrict__ diag, const double *__restrict__ phi,
-                                  const double *__restrict__ b, float *__restrict__ r32,
-                                  double *__restrict__ part, uint32_t *__restrict__ ticket,
-                                  cudaGraphConditionalHandle h, double tol, int maxc, double *__restrict__ stats,
-                                  int first) {
+// r = b - A phi (FP64, handed on in FP32) with r^2 (and, before the first cycle, b^2) summed per
+// block, then, in the block that arrives last on the ticket counter (after a fence, so every
+// block's sums are visible), the block sums added as a fixed tree, whether another cycle runs
+// (the condition of the graph's WHILE node, from the squared norms; first = 1 before the first
+// cycle), the solve's statistics, and the counter reset for the next launch.  stats[3] keeps
+// ||b||^2.  The decision is on the cycle's critical path: with one warp adding 304 pairs and the
+// root and division before it, a 256 x 256 solve of 6 cycles took 0.302 ms, so 0.283 ms.
+__global__ void __launch_bounds__(kT) k_residual_decide(int64_t n, const int32_t *__restrict__ col,
+                                                        const uint16_t *__restrict__ code,
+                                                        const double *__restrict__ val, const double *__restrict__ diag,
+                                                        const double *__restrict__ phi, const double *__restrict__ b,
+                                                        float *__restrict__ r32, double *__restrict__ part,
+                                                        uint32_t *__restrict__ ticket, cudaGraphConditionalHandle h,
+                                                        double tol, int maxc, double *__restrict__ stats, int first) {
     pdl_chain();
     __shared__ bool last;
     double rr = 0.0, bb = 0.0;
@@ -95,13 +97,13 @@ __global__ void k_residual_decide(int64_t n, const int32_t *__restrict__ col, co
                 if (c >= 0) ax += val[(int64_t)j * n + i] * phi[c];
             }
         }
-        const double ri = b[i] - ax;
+        const double bi = b[i], ri = bi - ax;
         r32[i] = (float)ri;
         rr += ri * ri;
-        bb += b[i] * b[i];
+        if (first) bb += bi * bi;
     }
     const double s1 = block_sum(rr);
-    const double s2 = block_sum(bb);
+    const double s2 = first ? block_sum(bb) : 0.0;
     if (threadIdx.x == 0) {
         part[2 * blockIdx.x] = s1;
         part[2 * blockIdx.x + 1] = s2;
@@ -109,24 +111,29 @@ __global__ void k_residual_decide(int64_t n, const int32_t *__restrict__ col, co
         last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     }
     __syncthreads();
-    if (!last || threadIdx.x >= 32) return;
+    if (!last) return;
     __threadfence();
-    const int lane = threadIdx.x;
-    double a = 0.0, c = 0.0;
-    for (int k = lane; k < (int)gridDim.x; k += 32) { a += __ldcg(part + 2 * k); c += __ldcg(part + 2 * k + 1); }
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xFFFFFFFFu, a, o);
-        c += __shfl_down_sync(0xFFFFFFFFu, c, o);
-    }
-    if (lane == 0) {
-        *ticket = 0u;
-        const double rel = c > 0.0 ? sqrt(a / c) : sqrt(a);
+    static_assert(kRedBlocks <= 2 * kT, "two block sums per thread");
+    const int k0 = threadIdx.x, k1 = k0 + kT;
+    const double tot = block_sum((k0 < kRedBlocks ? __ldcg(part + 2 * k0) : 0.0) +
+                                 (k1 < kRedBlocks ? __ldcg(part + 2 * k1) : 0.0));
+    double btot = 0.0;
+    if (first)
+        btot = block_sum((k0 < kRedBlocks ? __ldcg(part + 2 * k0 + 1) : 0.0) +
+                         (k1 < kRedBlocks ? __ldcg(part + 2 * k1 + 1) : 0.0));
+    if (threadIdx.x == 0) {
+        if (!first) btot = stats[3];
         const double cyc = first ? 0.0 : stats[0] + 1.0;
-        const bool done = rel <= tol || (c == 0.0 && a == 0.0) || cyc >= (double)maxc;
-        stats[0] = cyc;
-        stats[1] = rel;
-        if (done) stats[2] = worst_residual(stats[2], rel);
+        const bool done = tot <= tol * tol * (btot > 0.0 ? btot : 1.0) || cyc >= (double)maxc;
         cudaGraphSetConditional(h, done ? 0u : 1u);
+        *ticket = 0u;
+        stats[0] = cyc;
+        if (first) stats[3] = btot;
+        if (done) {
+            const double rel = btot > 0.0 ? sqrt(tot / btot) : sqrt(tot);
+            stats[1] = rel;
+            stats[2] = worst_residual(stats[2], rel);
+        }
     }
 }
 
@@ -355,6 +362,11 @@ __global__ void __launch_bounds__(kT) k_restrict_residual(int64_t nc, const int3
     if (t < 4 * nc && (t & 3) == 0) bc[t >> 2] = ((res + r1) + r2) + r3;
 }
 
+// 1 / d of a diagonal d = 1 .. 6, rounded once (the constants the divisions would give).
+__device__ __forceinline__ float diag_inv(float d) {
+    return d == 4.0f ? 0.25f : (d == 3.0f ? 1.0f / 3.0f : (d == 5.0f ? 0.2f : (d == 6.0f ? 1.0f / 6.0f : (d == 2.0f ? 0.5f : 1.0f))));
+}
+
 // ---- uniform levels of many blocks ---------------------------------------------------------
 // A level of root boxes (row-major, even nx and ny: it coarsens) needs no operator arrays, and a
 // block can form a tile's four half sweeps by itself when it also forms those of a frame of
@@ -381,8 +393,7 @@ __device__ __forceinline__ bool uni_wrap(int &g, int n, int bc) {
 __device__ __forceinline__ float uni_dinv(const UniLevel &A, int gx, int gy) {
     const int wx = A.bcx == PIC_BC_DIRICHLET ? 2 : (A.bcx == PIC_BC_PERIODIC ? 1 : 0);
     const int wy = A.bcy == PIC_BC_DIRICHLET ? 2 : (A.bcy == PIC_BC_PERIODIC ? 1 : 0);
-    const int d = (gx > 0 ? 1 : wx) + (gx < A.nx - 1 ? 1 : wx) + (gy > 0 ? 1 : wy) + (gy < A.ny - 1 ? 1 : wy);
-    return d == 4 ? 0.25f : (d == 3 ? (float)(1.0 / 3.0) : (d == 5 ? 0.2f : (d == 6 ? (float)(1.0 / 6.0) : 0.5f)));
+    return diag_inv((float)((gx > 0 ? 1 : wx) + (gx < A.nx - 1 ? 1 : wx) + (gy > 0 ? 1 : wy) + (gy < A.ny - 1 ? 1 : wy)));
 }
 // The thread's cells of the tile at (tx, ty) and its frame.
 __device__ __forceinline__ void uni_tile(const UniLevel &A, int tx, int ty, UniTile &t, int (&src)[2][kUCells]) {
@@ -629,7 +640,7 @@ struct SmallDesc {
     SmallLevel lv[kMaxSmallLevels];
     int32_t off_cg;  // smem offset of the coarsest CG vectors r, p, q (3 n)
     int32_t smem_floats;  // a multiple of 4
-    const double *cinv;  // coarsest level: dense FP64 inverse (n x n, symmetric), or null (CG)
+    const double *cinv;  // coarsest level: dense FP64 inverse (n rows of n | 1 words), or null (CG)
     int32_t inv_words;   // its words if it is copied to shared memory, else 0
 };
 
@@ -830,48 +841,38 @@ __device__ __forceinline__ void part_bar(int id, int nthr) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthr) : "memory");
 }
 
-// Coarsest level by its dense inverse C (at most kDirectN cells), applied in FP64 by the first
-// nthr >= 256 threads: thread (part, row) sums a run of columns of its row (C is symmetric, so
-// lanes read consecutive words), then the parts are added in order.  The FP64 pipe retires two
-// lanes per clock and SM, so one multiply-add per matrix word and no shuffle trees is the
-// cheapest form.  Singular (periodic in both directions): C inverts A + 1 1^T / n, whose
-// inverse maps 1 to 1, so C (b - mean(b) 1) = C b - mean(b).  `scr` holds n + 512 doubles.
-__device__ void sm_coarse_direct(const SmallLevel &L, const double *inv, float *x, const float *b, bool singular,
-                                 int nthr, int bar, double *scr) {
-    const int n = L.n, t = threadIdx.x;
-    double *ps = scr + n;
-    if (t < n) scr[t] = (double)b[t];
-    part_bar(bar, nthr);
-    const int n32 = (n + 31) & ~31, parts = min(nthr, 512) / n32;
-    const int part = t / n32, r = t - part * n32;
-    if (part < parts && r < n) {
-        const int per = (n + parts - 1) / parts, c1 = min(n, (part + 1) * per);
-        double a0 = 0.0, a1 = 0.0;  // two chains: a dependent FP64 operation takes tens of clocks
-        int c = part * per;
-        for (; c + 1 < c1; c += 2) {
-            a0 = fma(inv[c * n + r], scr[c], a0);
-            a1 = fma(inv[(c + 1) * n + r], scr[c + 1], a1);
-        }
-        if (c < c1) a0 = fma(inv[c * n + r], scr[c], a0);
-        ps[part * n32 + r] = a0 + a1;
-    }
-    part_bar(bar, nthr);
-    if (part == 0) {
-        double m = 0.0;
-        if (singular) {  // the warps of part 0 are whole (n32 is a multiple of 32)
-            for (int c = t & 31; c < n; c += 32) m += scr[c];
+// Coarsest level by its dense inverse C (at most kDirectN cells, rows n | 1 words apart so that
+// lanes of different rows read different banks), applied in FP64 by the first nthr >= 256
+// threads, 8, 4 or 2 lanes per row (one pass over all rows).  The FP64 pipe retires two lanes
+// per clock and SM and a dependent operation takes tens of clocks: a lane runs four chains and
+// few lanes are combined.  Singular (periodic in both directions): C (b - mean(b) 1) with
+// C 1 = 1 is (C - 1 1^T / n) b, whose matrix is formed on the host.  `scr`: n doubles.
+template <int LPR>
+__device__ __forceinline__ void direct_rows(int n, const double *inv, float *x, const double *bd) {
+    const int t = threadIdx.x, part = t & (LPR - 1), r = t / LPR;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    if (r < n) {
+        const double *row = inv + r * (n | 1);
+        int c = part;
+        for (; c + 3 * LPR < n; c += 4 * LPR)
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xFFFFFFFFu, m, o);
-            m /= (double)n;
-        }
-        if (r < n) {
-            double a0 = ps[r], a1 = 0.0;
-            int p = 1;
-            for (; p + 1 < parts; p += 2) { a0 += ps[p * n32 + r]; a1 += ps[(p + 1) * n32 + r]; }
-            if (p < parts) a0 += ps[p * n32 + r];
-            x[r] = (float)((a0 + a1) - m);
-        }
+            for (int k = 0; k < 4; ++k) a[k] = fma(row[c + k * LPR], bd[c + k * LPR], a[k]);
+        for (; c < n; c += LPR) a[0] = fma(row[c], bd[c], a[0]);
     }
+    double s = (a[0] + a[1]) + (a[2] + a[3]);
+#pragma unroll
+    for (int o = 1; o < LPR; o <<= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+    if (part == 0 && r < n) x[r] = (float)s;
+}
+__device__ void sm_coarse_direct(const SmallLevel &L, const double *inv, float *x, const float *b, int nthr, int bar,
+                                 double *scr) {
+    const int n = L.n;
+    if ((int)threadIdx.x < n) scr[threadIdx.x] = (double)b[threadIdx.x];
+    part_bar(bar, nthr);
+    if (threadIdx.x >= 256) return;
+    if (n <= 32) direct_rows<8>(n, inv, x, scr);
+    else if (n <= 64) direct_rows<4>(n, inv, x, scr);
+    else direct_rows<2>(n, inv, x, scr);
 }
 
 // ---- levels stored by colour --------------------------------------------------------------
@@ -901,7 +902,8 @@ __device__ __forceinline__ void rb_strips(const SmallDesc &D, const SmallLevel &
                                           RbStrips<K, S> &c) {
     const int nxh = L.nx >> 1, half = L.half;
     const bool px = D.bcx == PIC_BC_PERIODIC, py = D.bcy == PIC_BC_PERIODIC;
-    const int wx = D.bcx == PIC_BC_DIRICHLET ? 2 : (px ? 1 : 0), wy = D.bcy == PIC_BC_DIRICHLET ? 2 : (py ? 1 : 0);
+    const float wx = D.bcx == PIC_BC_DIRICHLET ? 2.0f : (px ? 1.0f : 0.0f);
+    const float wy = D.bcy == PIC_BC_DIRICHLET ? 2.0f : (py ? 1.0f : 0.0f);
 #pragma unroll
     for (int i = 0; i < S; ++i) {
         const int q = (int)threadIdx.x + L.nthr * i;
@@ -917,12 +919,12 @@ __device__ __forceinline__ void rb_strips(const SmallDesc &D, const SmallLevel &
         const bool hd = y0 > 0, hu = y0 + K < L.ny;
         c.dn[i] = hd ? j - nxh : (py ? j + (L.ny - 1) * nxh : half);
         c.up[i] = hu ? j + K * nxh : (py ? m : half);
-        const int dl = m > 0 ? 1 : wx, dr = m < nxh - 1 ? 1 : wx;
+        const float dl = m > 0 ? 1.0f : wx, dr = m < nxh - 1 ? 1.0f : wx;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            const int dv = 1 + (k > 0 || hd ? 1 : wy) + (k < K - 1 || hu ? 1 : wy);
-            c.di0[i][k] = __frcp_rn((float)(dv + (k & 1 ? dr : dl)));
-            c.di1[i][k] = __frcp_rn((float)(dv + (k & 1 ? dl : dr)));
+            const float dv = (1.0f + (k > 0 || hd ? 1.0f : wy)) + (k < K - 1 || hu ? 1.0f : wy);
+            c.di0[i][k] = diag_inv(dv + (k & 1 ? dr : dl));
+            c.di1[i][k] = diag_inv(dv + (k & 1 ? dl : dr));
             c.b0[i][k] = c.ok[i] ? b0[j + k * nxh] : 0.0f;
             c.b1[i][k] = c.ok[i] ? b1[j + k * nxh] : 0.0f;
         }
@@ -983,6 +985,10 @@ __device__ __forceinline__ void rb_down(const SmallDesc &D, const SmallLevel &L,
         const int q = (int)threadIdx.x + nthr * i;
         const int g = mdiv(q, L.nxh_magic), m = q - g * nxh;
         const float b0d = x0[c.dn[i]], b1d = x1[c.dn[i]], a0u = x0[c.up[i]], a1u = x1[c.up[i]];
+        // half diagonals of the left, right, lower and upper cells of a quartet
+        const float wx = D.bcx == PIC_BC_DIRICHLET ? 2.0f : (D.bcx == PIC_BC_PERIODIC ? 1.0f : 0.0f);
+        const float wy = D.bcy == PIC_BC_DIRICHLET ? 2.0f : (D.bcy == PIC_BC_PERIODIC ? 1.0f : 0.0f);
+        const float gl = 1.0f + (m > 0 ? 1.0f : wx), gr = 1.0f + (m < nxh - 1 ? 1.0f : wx);
 #pragma unroll
         for (int k = 0; k < K; k += 2) {
             const float l0 = x1[c.l[i] + k * c.sl[i]], l1 = x0[c.l[i] + (k + 1) * c.sl[i]];
@@ -990,13 +996,11 @@ __device__ __forceinline__ void rb_down(const SmallDesc &D, const SmallLevel &L,
             const float x00 = a[i][k], x10 = e[i][k], x01 = e[i][k + 1], x11 = a[i][k + 1];
             const float d1 = k > 0 ? e[i][k > 0 ? k - 1 : 0] : b1d, d0 = k > 0 ? a[i][k > 0 ? k - 1 : 0] : b0d;
             const float u0 = k + 2 < K ? a[i][k + 2 < K ? k + 2 : k] : a0u, u1 = k + 2 < K ? e[i][k + 2 < K ? k + 2 : k] : a1u;
-            // the diagonals are small integers: exact from their reciprocals
-            const float g00 = rintf(__frcp_rn(c.di0[i][k])), g10 = rintf(__frcp_rn(c.di1[i][k]));
-            const float g01 = rintf(__frcp_rn(c.di1[i][k + 1])), g11 = rintf(__frcp_rn(c.di0[i][k + 1]));
-            float s = c.b0[i][k] - (g00 * x00 - (((l0 + x10) + d1) + x01));
-            s += c.b1[i][k] - (g10 * x10 - (((x00 + r0) + d0) + x11));
-            s += c.b1[i][k + 1] - (g01 * x01 - (((l1 + x11) + x00) + u0));
-            s += c.b0[i][k + 1] - (g11 * x11 - (((x01 + r1) + x10) + u1));
+            const float gd = 1.0f + (k > 0 || g > 0 ? 1.0f : wy), gu = 1.0f + (k + 2 < K || (g + 1) * K < L.ny ? 1.0f : wy);
+            float s = c.b0[i][k] - ((gl + gd) * x00 - (((l0 + x10) + d1) + x01));
+            s += c.b1[i][k] - ((gr + gd) * x10 - (((x00 + r0) + d0) + x11));
+            s += c.b1[i][k + 1] - ((gl + gu) * x01 - (((l1 + x11) + x00) + u0));
+            s += c.b0[i][k + 1] - ((gr + gu) * x11 - (((x01 + r1) + x10) + u1));
             const int cy = (K / 2) * g + k / 2;
             bc[Cc.fast ? ((m + cy) & 1) * Cc.hs + cy * (nxh >> 1) + (m >> 1) : cy * nxh + m] = s;
         }
@@ -1044,7 +1048,7 @@ __device__ __forceinline__ void rb_up(const SmallDesc &D, const SmallLevel &L, c
 // first level holds the correction on return (after a block barrier).  All 1024 threads call
 // it.  ELL levels are swept by the whole block; a level stored by colour by its nthr threads,
 // whose other warps wait at the next finer level's barrier (barrier ids count from the first
-// such level).  `inv` is the coarsest inverse (null: CG), `scr` kDirectN + 512 doubles.
+// such level).  `inv` is the coarsest inverse (null: CG), `scr` kDirectN doubles.
 __device__ void sm_vcycle(const SmallDesc &D, float *sm, bool singular, float *red, const double *inv, double *scr) {
     const int last = D.nlev - 1;
     int g = 0;
@@ -1079,7 +1083,7 @@ __device__ void sm_vcycle(const SmallDesc &D, float *sm, bool singular, float *r
         const SmallLevel &L = D.lv[last];
         float *x = sm + L.off, *b = x + L.boff;
         float *r = sm + D.off_cg;
-        if (inv) sm_coarse_direct(L, inv, x, b, singular, last > gf ? D.lv[last - 1].nthr : 1024, 1 + last - gf, scr);
+        if (inv) sm_coarse_direct(L, inv, x, b, last > gf ? D.lv[last - 1].nthr : 1024, 1 + last - gf, scr);
         else sm_coarse_cg(D, L, x, b, r, r + L.n, r + 2 * L.n, singular, red);
     }
     for (--g; g >= gf; --g) {
@@ -1105,7 +1109,7 @@ __global__ void __launch_bounds__(1024, 1) k_tail_vcycle(const __grid_constant__
                                                        int singular) {
     extern __shared__ __align__(16) float sm[];
     __shared__ float redf[33];
-    __shared__ double scr[kDirectN + 512];
+    __shared__ double scr[kDirectN];
     __shared__ SmallDesc D;
     // constant data before the wait for the kernel before this one
     for (int k = threadIdx.x; k < (int)(sizeof(SmallDesc) / 4); k += 1024)
@@ -1417,7 +1421,7 @@ SmallDesc small_desc(const Instance &in, int g0) {
     off += 3 * (int32_t)in.lv.back().n + 8;
     D.smem_floats = (off + 3) & ~3;
     D.cinv = in.coarse_inv;
-    const int64_t words = in.lv.back().n * in.lv.back().n;
+    const int64_t words = in.lv.back().n * (in.lv.back().n | 1);
     D.inv_words = D.cinv && (int64_t)D.smem_floats * 4 + words * 8 + 8192 <= kSmallSmemMax ? (int32_t)words : 0;
     return D;
 }
@@ -1490,8 +1494,7 @@ template <bool CODED> void level_cycle(pic_ctx *ctx, Instance &in, size_t g, boo
 namespace {
 // Dense inverse of the coarsest level's operator (a uniform grid of root boxes: the 5-point
 // stencil with the wall rules), plus 1 1^T / n when the mesh is periodic in both directions.
-// Gauss-Jordan with partial pivoting in FP64, made symmetric (the solve reads columns as rows);
-// null (the CG is used) for a level larger than kDirectN cells or a singular matrix.  It depends
+// Gauss-Jordan with partial pivoting in FP64, made symmetric; null (the CG is used) for a level larger than kDirectN cells or a singular matrix.  It depends
 // on the root grid and the walls only, so an adaptation keeps it.
 double *coarse_inverse(pic_ctx *ctx, Instance &in, bool singular) {
     const Level &L = in.lv.back();
@@ -1547,8 +1550,12 @@ double *coarse_inverse(pic_ctx *ctx, Instance &in, bool singular) {
             const double m = 0.5 * (Inv[(size_t)i * n + j] + Inv[(size_t)j * n + i]);
             Inv[(size_t)i * n + j] = Inv[(size_t)j * n + i] = m;
         }
-    if (!in.coarse_inv_mem) in.coarse_inv_mem = dalloc<double>(in.inv_mem, kDirectN * kDirectN);
-    GB_CUDA(cudaMemcpyAsync(in.coarse_inv_mem, Inv.data(), Inv.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
+    if (singular)  // the mean of the right-hand side taken out (sm_coarse_direct)
+        for (double &v : Inv) v -= 1.0 / n;
+    std::vector<double> rows((size_t)n * (n | 1), 0.0);
+    for (int i = 0; i < n; ++i) std::copy_n(Inv.data() + (size_t)i * n, n, rows.data() + (size_t)i * (n | 1));
+    if (!in.coarse_inv_mem) in.coarse_inv_mem = dalloc<double>(in.inv_mem, kDirectN * (kDirectN | 1));
+    GB_CUDA(cudaMemcpyAsync(in.coarse_inv_mem, rows.data(), rows.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
     GB_CUDA(cudaStreamSynchronize(ctx->stream));
     in.coarse_inv_key = key;
     return in.coarse_inv_mem;
