@@ -121,43 +121,143 @@ struct CicDepositArgs {
     double *part;
 };
 
+// A sum of products: FP64 state in FP64; FP32 state as an unevaluated pair of FP32 words (exact
+// products, error-free additions: ~46 bits), since GB300 retires two FP64 lanes per clock and SM
+// against 128 FP32 ones.
+struct Pair { float h, l; };
+__device__ __forceinline__ Pair pair_diff(float x, float y) {  // x - y
+    const float d = x - y, t = d - x;
+    return Pair{d, (x - (d - t)) - (y + t)};
+}
+__device__ __forceinline__ Pair pair_scale(float w, Pair a) {  // w a
+    const float h = w * a.h;
+    return Pair{h, fmaf(w, a.l, fmaf(w, a.h, -h))};
+}
+__device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
+    const float h = a.h * b.h;
+    return Pair{h, fmaf(a.h, b.h, -h) + (a.h * b.l + a.l * b.h)};
+}
+__device__ __forceinline__ void pair_add(Pair &s, Pair p) {
+    const float t = s.h + p.h, u = t - s.h;
+    s.l += ((s.h - (t - u)) + (p.h - u)) + p.l;
+    s.h = t;
+}
+template <typename R> struct CicAcc;
+template <> struct CicAcc<double> {
+    double v = 0.0;
+    __device__ __forceinline__ void add(const CicAcc &o) { v += o.v; }
+    __device__ __forceinline__ double value() const { return v; }
+    __device__ __forceinline__ void store(double *hi, double *) const { *hi = v; }
+    __device__ __forceinline__ void load(const double *hi, const double *) { v = *hi; }
+    __device__ __forceinline__ CicAcc down(int o) const {
+        CicAcc r;
+        r.v = __shfl_down_sync(0xFFFFFFFFu, v, o);
+        return r;
+    }
+    static __device__ __forceinline__ CicAcc of(double w) { CicAcc r; r.v = w; return r; }
+    // (|u - 1/2|, whether u < 1/2)
+    static __device__ __forceinline__ CicAcc half(double u, bool &neg) {
+        const double d = u - 0.5;
+        neg = __double2hiint(d) < 0;
+        return of(fabs(d));
+    }
+    __device__ __forceinline__ CicAcc scaled(double w) const { return of(w * v); }
+    __device__ __forceinline__ CicAcc times(const CicAcc &o) const { return of(v * o.v); }
+};
+template <> struct CicAcc<float> {
+    Pair p{0.0f, 0.0f};
+    __device__ __forceinline__ void add(const CicAcc &o) { pair_add(p, o.p); }
+    __device__ __forceinline__ double value() const { return (double)p.h + (double)p.l; }
+    __device__ __forceinline__ void store(float *hi, float *lo) const { *hi = p.h; *lo = p.l; }
+    __device__ __forceinline__ void load(const float *hi, const float *lo) { p.h = *hi; p.l = *lo; }
+    __device__ __forceinline__ CicAcc down(int o) const {
+        CicAcc r;
+        r.p.h = __shfl_down_sync(0xFFFFFFFFu, p.h, o);
+        r.p.l = __shfl_down_sync(0xFFFFFFFFu, p.l, o);
+        return r;
+    }
+    static __device__ __forceinline__ CicAcc of(float w) { CicAcc r; r.p.h = w; return r; }
+    static __device__ __forceinline__ CicAcc half(float u, bool &neg) {
+        CicAcc r;
+        r.p = pair_diff(u, 0.5f);
+        neg = r.p.h < 0.0f || (r.p.h == 0.0f && r.p.l < 0.0f);
+        if (neg) { r.p.h = -r.p.h; r.p.l = -r.p.l; }
+        return r;
+    }
+    __device__ __forceinline__ CicAcc scaled(float w) const { CicAcc r; r.p = pair_scale(w, p); return r; }
+    __device__ __forceinline__ CicAcc times(const CicAcc &o) const { CicAcc r; r.p = pair_mul(p, o.p); return r; }
+};
+
+// One warp per leaf.  A particle's weights on the three columns around its cell are
+// (a, 1 - a - c, c) with a = max(1/2 - u, 0), c = max(u - 1/2, 0) (one of them zero), and
+// likewise on the rows, so the nine sums 1, a, c, a', c', aa', ca', ac', cc' (times w) give the
+// nine cells: 12 operations per particle instead of the ~55 of nine predicated accumulators per
+// centre; the lanes are combined through shared memory, three lanes per sum.  512 x 16 FP32
+// discharge: the deposit 0.258 ms per step at first, 0.120 with these sums in FP64, 0.055 so.
+constexpr int kCicSums = 9;
 template <typename R>
 __global__ void __launch_bounds__(kT) k_cic_deposit(CicDepositArgs a) {
-    const int lane = threadIdx.x & 31;
+    __shared__ R hi[kT / 32][kCicSums][33], lo[kT / 32][sizeof(R) == 4 ? kCicSums : 1][33];
+    __shared__ double tot[kT / 32][kCicSums];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    auto low = [&](int k, int j) { return &lo[wib][sizeof(R) == 4 ? k : 0][j]; };
+    // cell k of the 3 x 3 block as a combination of the sums: bit j of plus / minus
+    // (sums: 0: 1, 1: a, 2: c, 3: a', 4: c', 5: aa', 6: ca', 7: ac', 8: cc')
+    const uint32_t plus[9] = {1u << 5, 1u << 3, 1u << 6, 1u << 1, 1u | 0xFu << 5, 1u << 2, 1u << 7, 1u << 4, 1u << 8};
+    const uint32_t minus[9] = {0u, 3u << 5, 0u, 5u << 5, 0xFu << 1, 5u << 6, 0u, 3u << 7, 0u};
+    uint32_t mp = 0, mm = 0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k)
+        if (lane == k) { mp = plus[k]; mm = minus[k]; }
+    const int sum = lane / 3, j0 = 11 * (lane - 3 * sum);  // this lane's sum and its lanes from j0 on
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t L = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; L < a.nl; L += nw) {
-        double acc[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+        double q_sum = 0.0;
         for (int s = 0; s < a.nsp; ++s) {
             const R *U = (const R *)a.u[s], *V = (const R *)a.v[s], *Wt = (const R *)a.w[s];
+            CicAcc<R> S[kCicSums];
             for (int32_t p = a.start[s][L] + lane; p < a.end[s][L]; p += 32) {
-                const double u = (double)U[p], v = (double)V[p], qw = a.q[s] * (double)Wt[p];
-                const int qx = u >= 0.5 ? 1 : 0, qy = v >= 0.5 ? 1 : 0;
-                const double fx = u + 0.5 - qx, fy = v + 0.5 - qy;
-                // centres i - 1 + qx + a', j - 1 + qy + b' -> slots (qx + a', qy + b') of the 3 x 3 block
-#pragma unroll
-                for (int bb = 0; bb < 2; ++bb)
-#pragma unroll
-                    for (int aa = 0; aa < 2; ++aa) {
-                        const double wt = (aa ? fx : 1.0 - fx) * (bb ? fy : 1.0 - fy);
-                        const int slot = (qx + aa) + 3 * (qy + bb);
-#pragma unroll
-                        for (int k = 0; k < 9; ++k)
-                            if (k == slot) acc[k] += qw * wt;
-                    }
+                const R w = Wt[p];
+                bool nu, nv;
+                const CicAcc<R> du = CicAcc<R>::half(U[p], nu), dv = CicAcc<R>::half(V[p], nv);
+                const CicAcc<R> x = du.scaled(w), y = dv.scaled(w), xy = x.times(dv);
+                S[0].add(CicAcc<R>::of(w));
+                if (nu) S[1].add(x); else S[2].add(x);
+                if (nv) S[3].add(y); else S[4].add(y);
+                if (nv) { if (nu) S[5].add(xy); else S[6].add(xy); }
+                else { if (nu) S[7].add(xy); else S[8].add(xy); }
             }
-        }
 #pragma unroll
-        for (int k = 0; k < 9; ++k) {
+            for (int k = 0; k < kCicSums; ++k) S[k].store(&hi[wib][k][lane], low(k, lane));
+            __syncwarp();
+            CicAcc<R> t;
+            if (lane < 3 * kCicSums)
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xFFFFFFFFu, acc[k], o);
+                for (int j = 0; j < 11; ++j)
+                    if (j0 + j < 32) {
+                        CicAcc<R> o;
+                        o.load(&hi[wib][sum][j0 + j], low(sum, j0 + j));
+                        t.add(o);
+                    }
+            const CicAcc<R> t1 = t.down(1), t2 = t.down(2);
+            t.add(t1);
+            t.add(t2);
+            q_sum += a.q[s] * t.value();  // (the sum's first lane holds it)
+            __syncwarp();
         }
+        if (lane < 3 * kCicSums && lane == 3 * sum) tot[wib][sum] = q_sum;
+        __syncwarp();
         if (lane < 9) {
             double v = 0.0;
 #pragma unroll
-            for (int k = 0; k < 9; ++k)
-                if (k == lane) v = acc[k];
+            for (int j = 0; j < kCicSums; ++j) {
+                const double w = tot[wib][j];
+                if ((mp >> j) & 1u) v += w;
+                if ((mm >> j) & 1u) v -= w;
+            }
             a.part[9 * L + lane] = v;
         }
+        __syncwarp();
     }
 }
 
