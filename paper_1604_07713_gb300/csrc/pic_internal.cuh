@@ -85,6 +85,7 @@ struct Level {
     double *val64 = nullptr, *diag64 = nullptr;  // finest level only (FP64 residual)
     double *bcw = nullptr;                 // finest level: Dirichlet coefficients [4 * n]
     double *kappa = nullptr;               // implicit scheme: relative permittivity 1 + chi per cell
+    float *face = nullptr;                 // implicit scheme, root-box levels: right [n] and upper [n] conductances
     float *x = nullptr, *b = nullptr, *t = nullptr;  // FP32 work vectors
     int64_t lat_n() const { return ((int64_t)nx0 << lmax) * ((int64_t)ny0 << lmax); }
 };

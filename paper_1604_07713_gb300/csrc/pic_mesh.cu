@@ -148,7 +148,9 @@ __global__ void k_check_balance(int64_t n, LatView L, int32_t *__restrict__ err)
 __global__ void k_assemble(int64_t n, LatView L, int bcx, int bcy, int32_t *__restrict__ col,
                            float *__restrict__ val, float *__restrict__ dinv, double *__restrict__ val64,
                            double *__restrict__ diag64, double *__restrict__ bcw, uint8_t *__restrict__ color,
-                           int32_t *__restrict__ err, const double *__restrict__ kappa, uint16_t *__restrict__ code) {
+                           int32_t *__restrict__ err, const double *__restrict__ kappa, uint16_t *__restrict__ code,
+                           float *__restrict__ face) {
+    pdl_chain();
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= n) return;
     {
@@ -190,10 +192,12 @@ __global__ void k_assemble(int64_t n, LatView L, int bcx, int bcy, int32_t *__re
         switch (f.type) {
         case FB:
             if (bc == PIC_BC_DIRICHLET) { diag += 2.0 * kappa[c]; wall[d] = 2.0 * kappa[c]; }
+            if (face && (d & 1)) face[(d >> 1) * n + c] = 0.0f;
             break;
         case FS:
             kf = 0.5 * (kappa[c] + kappa[f.n1]);
             diag += kf; cc[k] = f.n1; vv[k++] = -kf;
+            if (face && (d & 1)) face[(d >> 1) * n + c] = (float)kf;
             break;
         case FF:
             kf = 0.5 * (kappa[c] + 0.5 * (kappa[f.n1] + kappa[f.n2]));
@@ -423,15 +427,17 @@ void assemble_level(pic_ctx *ctx, Instance &in, Level &g, bool finest, int32_t *
     g.b = dalloc<float>(A, g.n);
     g.t = dalloc<float>(A, g.n);
     g.kappa = in.cfg.implicit ? dalloc<double>(A, g.n) : nullptr;  // set per step (poisson_kappa)
+    g.face = in.cfg.implicit && g.lmax == 0 ? dalloc<float>(A, 2 * g.n) : nullptr;
     k_assemble<<<blocks_for(g.n), kT, 0, ctx->stream>>>(g.n, view_of(in, g), in.cfg.bc_x, in.cfg.bc_y, g.col,
                                                         g.val, g.dinv, g.val64, g.diag64, g.bcw, g.color, d_err,
-                                                        nullptr, g.code);
+                                                        nullptr, g.code, nullptr);
     count_launch(ctx);
 }
 
 // A coarse cell's kappa: the mean over its children.
 __global__ void k_kappa_restrict(int64_t nc, const int32_t *__restrict__ child4, const double *__restrict__ kf,
                                  double *__restrict__ kc) {
+    pdl_chain();
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= nc) return;
     double s = 0.0;
@@ -448,6 +454,7 @@ __global__ void k_kappa_restrict(int64_t nc, const int32_t *__restrict__ child4,
 __global__ void k_rhs(int64_t n, const double *__restrict__ charge, const uint8_t *__restrict__ lev, int lmax,
                       double hf, double rho_bg, double inv_eps0, const double *__restrict__ bcw, double w0, double w1,
                       double w2, double w3, double *__restrict__ b) {
+    pdl_chain();
     const int64_t L = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (L >= n) return;
     const double h = (double)(1 << (lmax - lev[L])) * hf;
@@ -668,19 +675,19 @@ void poisson_kappa(pic_ctx *ctx, Instance &in, const double walls[4]) {
     cudaStream_t st = ctx->stream;
     for (size_t g = 1; g < in.lv.size(); ++g) {
         Level &C = in.lv[g];
-        k_kappa_restrict<<<blocks_for(C.n), kT, 0, st>>>(C.n, C.child4, in.lv[g - 1].kappa, C.kappa);
+        pdl(k_kappa_restrict, blocks_for(C.n), kT, 0, st, C.n, C.child4, in.lv[g - 1].kappa, C.kappa);
         count_launch(ctx);
     }
     for (size_t g = 0; g < in.lv.size(); ++g) {
         Level &L = in.lv[g];
-        k_assemble<<<blocks_for(L.n), kT, 0, st>>>(L.n, view_of(in, L), in.cfg.bc_x, in.cfg.bc_y, L.col, L.val,
-                                                   L.dinv, L.val64, L.diag64, L.bcw, L.color, in.d_err, L.kappa, nullptr);
+        uint16_t *no_code = nullptr;
+        pdl(k_assemble, blocks_for(L.n), kT, 0, st, L.n, view_of(in, L), in.cfg.bc_x, in.cfg.bc_y, L.col, L.val, L.dinv,
+            L.val64, L.diag64, L.bcw, L.color, in.d_err, L.kappa, no_code, L.face);
         count_launch(ctx);
     }
     const Level &F = in.lv[0];
-    k_rhs<<<blocks_for(F.n), kT, 0, st>>>(F.n, in.charge, F.lev, in.lmax, in.h0 / (double)(1 << in.lmax),
-                                          in.cfg.rho_background, 1.0 / in.cfg.eps0, F.bcw, walls[0], walls[1],
-                                          walls[2], walls[3], in.bvec);
+    pdl(k_rhs, blocks_for(F.n), kT, 0, st, F.n, in.charge, F.lev, in.lmax, in.h0 / (double)(1 << in.lmax),
+        in.cfg.rho_background, 1.0 / in.cfg.eps0, F.bcw, walls[0], walls[1], walls[2], walls[3], in.bvec);
     count_launch(ctx);
     check_launch("poisson_kappa");
 }

@@ -623,6 +623,7 @@ struct SmallLevel {
     int32_t n;
     const int32_t *col;
     const float *val, *dinv;
+    const float *face;      // implicit scheme, uniform levels: each cell's right [n] and upper [n] conductance
     const uint8_t *color;
     const int32_t *child4;  // children (in the finer level) of this level's cells
     const int32_t *parent;  // this level's cells -> cells of the next coarser level
@@ -641,7 +642,8 @@ struct SmallDesc {
     int32_t off_cg;  // smem offset of the coarsest CG vectors r, p, q (3 n)
     int32_t smem_floats;  // a multiple of 4
     const double *cinv;  // coarsest level: dense FP64 inverse (n rows of n | 1 words), or null (CG)
-    int32_t inv_words;   // its words if it is copied to shared memory, else 0
+    int32_t build;       // 1: the inverse is formed by each launch (FP32, sm_build_inverse)
+    int32_t inv_words;   // FP64 words of the inverse in shared memory, else 0
 };
 
 // floor(i / d) by a multiply-high reciprocal m = floor((2^32 - 1) / d) + 1; m = 0 stands for
@@ -847,32 +849,80 @@ __device__ __forceinline__ void part_bar(int id, int nthr) {
 // per clock and SM and a dependent operation takes tens of clocks: a lane runs four chains and
 // few lanes are combined.  Singular (periodic in both directions): C (b - mean(b) 1) with
 // C 1 = 1 is (C - 1 1^T / n) b, whose matrix is formed on the host.  `scr`: n doubles.
-template <int LPR>
-__device__ __forceinline__ void direct_rows(int n, const double *inv, float *x, const double *bd) {
+template <int LPR, typename T>
+__device__ __forceinline__ void direct_rows(int n, const T *inv, float *x, const T *bd) {
     const int t = threadIdx.x, part = t & (LPR - 1), r = t / LPR;
-    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    T a[4] = {0, 0, 0, 0};
     if (r < n) {
-        const double *row = inv + r * (n | 1);
+        const T *row = inv + r * (n | 1);
         int c = part;
         for (; c + 3 * LPR < n; c += 4 * LPR)
 #pragma unroll
             for (int k = 0; k < 4; ++k) a[k] = fma(row[c + k * LPR], bd[c + k * LPR], a[k]);
         for (; c < n; c += LPR) a[0] = fma(row[c], bd[c], a[0]);
     }
-    double s = (a[0] + a[1]) + (a[2] + a[3]);
+    T s = (a[0] + a[1]) + (a[2] + a[3]);
 #pragma unroll
     for (int o = 1; o < LPR; o <<= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
     if (part == 0 && r < n) x[r] = (float)s;
+}
+template <typename T> __device__ __forceinline__ void direct_solve(int n, const T *inv, float *x, const T *bd) {
+    if (threadIdx.x >= 256) return;
+    if (n <= 32) direct_rows<8>(n, inv, x, bd);
+    else if (n <= 64) direct_rows<4>(n, inv, x, bd);
+    else direct_rows<2>(n, inv, x, bd);
 }
 __device__ void sm_coarse_direct(const SmallLevel &L, const double *inv, float *x, const float *b, int nthr, int bar,
                                  double *scr) {
     const int n = L.n;
     if ((int)threadIdx.x < n) scr[threadIdx.x] = (double)b[threadIdx.x];
     part_bar(bar, nthr);
-    if (threadIdx.x >= 256) return;
-    if (n <= 32) direct_rows<8>(n, inv, x, scr);
-    else if (n <= 64) direct_rows<4>(n, inv, x, scr);
-    else direct_rows<2>(n, inv, x, scr);
+    direct_solve(n, inv, x, scr);
+}
+
+// The implicit scheme's coarsest operator changes every step: its inverse is formed by the
+// launch that uses it, in FP32 (a coarse-grid correction needs three digits: the CG it replaces
+// stopped at 1e-3), in place by Gauss-Jordan without pivoting (the operator is symmetric and
+// positive definite).  Singular: A + alpha 1 1^T is inverted and the constant's image taken out
+// again, so that the mean of the right-hand side does not matter.  1024 threads; `tmp` 2 n words.
+__device__ void sm_build_inverse(const SmallLevel &L, float *M, bool singular, float *tmp) {
+    const int n = L.n, ld = n | 1, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    float *rowk = tmp, *colk = tmp + n;
+    const float alpha = singular ? __frcp_rn(L.dinv[0]) / (float)n : 0.0f;
+    for (int i = ty; i < n; i += 32)
+        for (int j = tx; j < n; j += 32) M[i * ld + j] = alpha;
+    __syncthreads();
+    if ((int)threadIdx.x < n) {  // a row's columns are distinct except across a wrap of one or two cells
+        const int i = threadIdx.x;
+        M[i * ld + i] += __frcp_rn(L.dinv[i]);
+        for (int j = 0; j < kEll; ++j) {
+            const int32_t c = L.col[(int64_t)j * n + i];
+            if (c >= 0) M[i * ld + c] += L.val[(int64_t)j * n + i];
+        }
+    }
+    __syncthreads();
+    for (int k = 0; k < n; ++k) {
+        if ((int)threadIdx.x < n) {
+            const float p = 1.0f / M[k * ld + k];
+            rowk[threadIdx.x] = (int)threadIdx.x == k ? p : M[k * ld + threadIdx.x] * p;
+            colk[threadIdx.x] = M[threadIdx.x * ld + k];
+        }
+        __syncthreads();
+        for (int i = ty; i < n; i += 32) {
+            const float f = colk[i];
+            for (int j = tx; j < n; j += 32) {
+                const float r = rowk[j];
+                M[i * ld + j] = i == k ? r : (j == k ? -f * r : fmaf(-f, r, M[i * ld + j]));
+            }
+        }
+        __syncthreads();
+    }
+    if (singular) {
+        const float c = 1.0f / (alpha * (float)n * (float)n);
+        for (int i = ty; i < n; i += 32)
+            for (int j = tx; j < n; j += 32) M[i * ld + j] -= c;
+        __syncthreads();
+    }
 }
 
 // ---- levels stored by colour --------------------------------------------------------------
@@ -1044,11 +1094,92 @@ __device__ __forceinline__ void rb_up(const SmallDesc &D, const SmallLevel &L, c
     }
 }
 
+// The same legs on a uniform level whose faces carry the implicit scheme's kappa (face words,
+// reciprocal diagonals from global memory: they stay in L1 over a launch).  Position j of colour
+// c is the cell ix = 2 m + p of row iy, p = (c + iy) & 1.
+struct KapCell { int i, iy, m, p; };
+__device__ __forceinline__ KapCell kap_cell(const SmallLevel &L, int j, int c) {
+    KapCell k;
+    const int nxh = L.nx >> 1;
+    k.iy = mdiv(j, L.nxh_magic);
+    k.m = j - k.iy * nxh;
+    k.p = (c + k.iy) & 1;
+    k.i = k.iy * L.nx + 2 * k.m + k.p;
+    return k;
+}
+// sum over the cell's faces of conductance times neighbour (left, right, below, above); xo: the
+// other colour's values
+__device__ __forceinline__ float kap_row(const SmallDesc &D, const SmallLevel &L, const float *xo, int j, const KapCell &k) {
+    const int nx = L.nx, nxh = nx >> 1, half = L.half, i = k.i;
+    const bool px = D.bcx == PIC_BC_PERIODIC, py = D.bcy == PIC_BC_PERIODIC;
+    const float *fx = L.face, *fy = L.face + L.n;
+    const bool l_in = k.p || k.m > 0, d_in = k.iy > 0, u_in = k.iy < L.ny - 1;
+    const int jl = k.p ? j : (k.m > 0 ? j - 1 : (px ? j + nxh - 1 : half));
+    const int jr = !k.p ? j : (k.m < nxh - 1 ? j + 1 : (px ? j - nxh + 1 : half));
+    const int jd = d_in ? j - nxh : (py ? j + (L.ny - 1) * nxh : half);
+    const int ju = u_in ? j + nxh : (py ? j - (L.ny - 1) * nxh : half);
+    const float gl = __ldg(fx + (l_in ? i - 1 : (px ? i + nx - 1 : i))), gr = __ldg(fx + i);
+    const float gd = __ldg(fy + (d_in ? i - nx : (py ? i + (L.ny - 1) * nx : i))), gu = __ldg(fy + i);
+    return fmaf(gu, xo[ju], fmaf(gd, xo[jd], fmaf(gr, xo[jr], gl * xo[jl])));
+}
+__device__ __forceinline__ void kap_half(const SmallDesc &D, const SmallLevel &L, int c, float *x0, const float *b0) {
+    float *xs = x0 + c * L.hs;
+    const float *xo = x0 + (c ^ 1) * L.hs, *b = b0 + c * L.hs;
+#pragma unroll 2
+    for (int j = threadIdx.x; j < L.half; j += L.nthr) {
+        const KapCell k = kap_cell(L, j, c);
+        xs[j] = (b[j] + kap_row(D, L, xo, j, k)) * __ldg(L.dinv + k.i);
+    }
+}
+__device__ void kap_down(const SmallDesc &D, const SmallLevel &L, const SmallLevel &Cc, float *sm, int bar) {
+    float *x0 = sm + L.off, *x1 = x0 + L.hs;
+    const float *b0 = x0 + L.boff, *b1 = b0 + L.hs;
+    for (int j = threadIdx.x; j < L.half; j += L.nthr) x0[j] = b0[j] * __ldg(L.dinv + kap_cell(L, j, 0).i);
+    if (threadIdx.x == 0) x0[L.half] = x1[L.half] = 0.0f;  // missing neighbours
+    part_bar(bar, L.nthr);
+    for (int h = 1; h < 2 * kNu; ++h) {
+        kap_half(D, L, h & 1, x0, b0);
+        part_bar(bar, L.nthr);
+    }
+    float *bc = sm + Cc.off + Cc.boff;
+    const int nxh = L.nx >> 1;
+    for (int p = threadIdx.x; p < Cc.n; p += L.nthr) {
+        const int qy = mdiv(p, L.nxh_magic), qx = p - qy * nxh;
+        float s = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int iy = 2 * qy + (k >> 1), c = ((k & 1) + iy) & 1, j = iy * nxh + qx;
+            const KapCell kc{iy * L.nx + 2 * qx + (k & 1), iy, qx, k & 1};
+            const float *xo = c ? x0 : x1, *xs = c ? x1 : x0, *b = c ? b1 : b0;
+            const float d = __frcp_rn(__ldg(L.dinv + kc.i));
+            s += b[j] - (d * xs[j] - kap_row(D, L, xo, j, kc));
+        }
+        bc[sm_pos(Cc, p)] = s;
+    }
+    part_bar(bar, L.nthr);
+}
+__device__ void kap_up(const SmallDesc &D, const SmallLevel &L, const SmallLevel &Cc, float *sm, int bar) {
+    float *x0 = sm + L.off, *x1 = x0 + L.hs;
+    const float *b0 = x0 + L.boff, *xc = sm + Cc.off;
+    const int nxh = L.nx >> 1;
+    part_bar(bar, L.nthr);  // the coarser level's correction is complete
+    for (int j = threadIdx.x; j < L.half; j += L.nthr) {
+        const int iy = mdiv(j, L.nxh_magic), m = j - iy * nxh;
+        x1[j] += xc[sm_pos(Cc, (iy >> 1) * nxh + m)];
+    }
+    part_bar(bar, L.nthr);
+    for (int h = 0; h < 2 * kNu; ++h) {
+        kap_half(D, L, h & 1, x0, b0);
+        if (h + 1 < 2 * kNu) part_bar(bar, L.nthr);
+    }
+}
+
 // V-cycle over the shared-memory levels; b of the first level must be in place, x of the
 // first level holds the correction on return (after a block barrier).  All 1024 threads call
 // it.  ELL levels are swept by the whole block; a level stored by colour by its nthr threads,
 // whose other warps wait at the next finer level's barrier (barrier ids count from the first
-// such level).  `inv` is the coarsest inverse (null: CG), `scr` kDirectN doubles.
+// such level).  `inv` is the coarsest inverse (FP32 where the launch built it; null: CG), `scr`
+// kDirectN doubles.
 __device__ void sm_vcycle(const SmallDesc &D, float *sm, bool singular, float *red, const double *inv, double *scr) {
     const int last = D.nlev - 1;
     int g = 0;
@@ -1075,7 +1206,8 @@ __device__ void sm_vcycle(const SmallDesc &D, float *sm, bool singular, float *r
     for (; g < last; ++g) {
         const SmallLevel &L = D.lv[g], &Cc = D.lv[g + 1];
         if ((int)threadIdx.x >= L.nthr) break;
-        if (L.rows == 4) rb_down<4, 1>(D, L, Cc, sm, 1 + g - gf);
+        if (L.face) kap_down(D, L, Cc, sm, 1 + g - gf);
+        else if (L.rows == 4) rb_down<4, 1>(D, L, Cc, sm, 1 + g - gf);
         else if (L.strips == 1) rb_down<2, 1>(D, L, Cc, sm, 1 + g - gf);
         else rb_down<2, 2>(D, L, Cc, sm, 1 + g - gf);
     }
@@ -1083,12 +1215,14 @@ __device__ void sm_vcycle(const SmallDesc &D, float *sm, bool singular, float *r
         const SmallLevel &L = D.lv[last];
         float *x = sm + L.off, *b = x + L.boff;
         float *r = sm + D.off_cg;
-        if (inv) sm_coarse_direct(L, inv, x, b, last > gf ? D.lv[last - 1].nthr : 1024, 1 + last - gf, scr);
+        if (D.build) direct_solve(L.n, reinterpret_cast<const float *>(inv), x, b);
+        else if (inv) sm_coarse_direct(L, inv, x, b, last > gf ? D.lv[last - 1].nthr : 1024, 1 + last - gf, scr);
         else sm_coarse_cg(D, L, x, b, r, r + L.n, r + 2 * L.n, singular, red);
     }
     for (--g; g >= gf; --g) {
         const SmallLevel &L = D.lv[g], &Cc = D.lv[g + 1];
-        if (L.rows == 4) rb_up<4, 1>(D, L, Cc, sm, 1 + g - gf);
+        if (L.face) kap_up(D, L, Cc, sm, 1 + g - gf);
+        else if (L.rows == 4) rb_up<4, 1>(D, L, Cc, sm, 1 + g - gf);
         else if (L.strips == 1) rb_up<2, 1>(D, L, Cc, sm, 1 + g - gf);
         else rb_up<2, 2>(D, L, Cc, sm, 1 + g - gf);
     }
@@ -1116,12 +1250,14 @@ __global__ void __launch_bounds__(1024, 1) k_tail_vcycle(const __grid_constant__
         reinterpret_cast<uint32_t *>(&D)[k] = reinterpret_cast<const uint32_t *>(&Dp)[k];
     __syncthreads();
     const double *inv = D.cinv;
+    double *cs = reinterpret_cast<double *>(sm + D.smem_floats);
     if (D.inv_words) {
-        double *cs = reinterpret_cast<double *>(sm + D.smem_floats);
-        for (int k = threadIdx.x; k < D.inv_words; k += 1024) cs[k] = inv[k];
+        if (inv)
+            for (int k = threadIdx.x; k < D.inv_words; k += 1024) cs[k] = inv[k];
         inv = cs;
     }
     pdl_chain();
+    if (D.build) sm_build_inverse(D.lv[D.nlev - 1], reinterpret_cast<float *>(cs), singular != 0, reinterpret_cast<float *>(scr));
     const SmallLevel &L = D.lv[0];
     for (int i = threadIdx.x; i < L.n; i += blockDim.x) sm[L.off + L.boff + sm_pos(L, i)] = gb[i];
     __syncthreads();
@@ -1209,10 +1345,14 @@ __global__ void __launch_bounds__(1024, 1) k_small_solve(const SmallSolve *__res
     const double *inv = D.cinv;
     if (rank == 0 && D.inv_words) {
         double *cs = vbuf + 1024 * nbuf;
-        for (int k = threadIdx.x; k < D.inv_words; k += 1024) cs[k] = inv[k];
+        if (inv)
+            for (int k = threadIdx.x; k < D.inv_words; k += 1024) cs[k] = inv[k];
         inv = cs;
     }
     pdl_chain();  // what came before it reads is constant between mesh changes
+    if (rank == 0 && D.build)
+        sm_build_inverse(D.lv[D.nlev - 1], reinterpret_cast<float *>(vbuf + 1024 * nbuf), it.singular != 0,
+                         reinterpret_cast<float *>(vbuf));
     float *lsm = cl.map_shared_rank(sm, 0);  // the leader's levels
     double *lpart = cl.map_shared_rank(part, 0);
     const double *lmean = cl.map_shared_rank(&mean_sh, 0);
@@ -1386,6 +1526,11 @@ SmallDesc small_desc(const Instance &in, int g0) {
     D.bcx = in.cfg.bc_x;
     D.bcy = in.cfg.bc_y;
     int32_t off = 0;
+    const int64_t nl = in.lv.back().n, words = nl * (nl | 1);
+    int64_t floats = 3 * nl + 16;
+    for (size_t g = g0; g < in.lv.size(); ++g) floats += 2 * in.lv[g].n + 16;
+    const bool fits = floats * 4 + words * (in.cfg.implicit ? 4 : 8) + 8192 + 16 <= kSmallSmemMax;
+    D.build = in.cfg.implicit && nl <= kDirectN && fits ? 1 : 0;
     for (int k = 0; k < D.nlev; ++k) {
         const Level &L = in.lv[g0 + k];
         SmallLevel &S = D.lv[k];
@@ -1403,7 +1548,8 @@ SmallDesc small_desc(const Instance &in, int g0) {
         for (int64_t i = 0; i < L.n; ++i)
             if (q(i, S.nx_magic) != i / L.nx0 || q(i, S.nxh_magic) != i / (int64_t)nxh)
                 fail(PIC_EINVAL, "index division check failed");
-        S.fast = S.uniform && k + 1 < D.nlev ? 1 : 0;  // (such a level coarsens: nx and ny are even)
+        S.fast = L.lmax == 0 && k + 1 < D.nlev ? 1 : 0;  // (such a level coarsens: nx and ny are even)
+        S.face = L.face;
         S.half = (int32_t)L.n / 2;
         S.hs = S.half + 4;
         S.boff = S.fast ? 2 * S.hs : (int32_t)L.n;
@@ -1414,15 +1560,14 @@ SmallDesc small_desc(const Instance &in, int g0) {
         S.rows = S.ny % 4 == 0 && S.half > 1024 ? 4 : 2;
         const int ns = S.half / S.rows;
         S.strips = ns > 1024 ? 2 : 1;
-        S.nthr = in.coarse_inv ? std::min(1024, std::max(256, (ns + 31) / 32 * 32)) : 1024;
+        S.nthr = in.coarse_inv || D.build ? std::min(1024, std::max(256, (ns + 31) / 32 * 32)) : 1024;
         off += S.fast ? 4 * S.hs : 2 * (int32_t)L.n;
     }
     D.off_cg = off;
     off += 3 * (int32_t)in.lv.back().n + 8;
     D.smem_floats = (off + 3) & ~3;
     D.cinv = in.coarse_inv;
-    const int64_t words = in.lv.back().n * (in.lv.back().n | 1);
-    D.inv_words = D.cinv && (int64_t)D.smem_floats * 4 + words * 8 + 8192 <= kSmallSmemMax ? (int32_t)words : 0;
+    D.inv_words = fits && (D.build || D.cinv) ? (int32_t)(D.build ? (words + 1) / 2 : words) : 0;
     return D;
 }
 

@@ -77,3 +77,31 @@ def test_clusters_of_every_size_give_the_same_bits():
             ctx.step(3)
             for i in range(3):
                 assert np.array_equal(ctx.fields(G.PIC_FIELD_PHI, inst=i), alone[i])
+
+
+# the implicit scheme's operator: a coarsest inverse formed by the launch (up to 128 cells), CG
+# beyond, a mesh two cells wide in a periodic direction, one level only, ragged strips
+@pytest.mark.parametrize("bc", [(D, P), (P, P), (D, N)])
+@pytest.mark.parametrize("nx,ny", [(4, 4), (11, 11), (33, 9), (2, 32), (40, 20), (60, 44), (208, 24), (34, 66), (64, 64)])
+def test_implicit_solve_matches_the_oracle(nx, ny, bc):
+    n = nx * ny * 3
+    rng = np.random.default_rng(nx + 1000 * ny)
+    h, dt = 2.0 ** -6, 3.0
+    cfg = W.base_config(precision=W.FP64, n_species=1, q=[-1.0], m=[1.0], dt=dt, bc_x=bc[0], bc_y=bc[1], implicit=1,
+                        rho_background=1.0, phi_left_dc=0.0 if bc[0] != D else 0.02, mg_rel_tol=1e-11, mg_max_cycles=200)
+    mesh = dict(nx0=nx, ny0=ny, h0=h, lmax=0)
+    z = np.zeros(n)
+    parts = dict(x=rng.random(n) * nx * h, y=rng.random(n) * ny * h, vx=z, vy=z, vz=z, w=np.full(n, h * h / 3))
+    with G.Context(cfg) as ctx:
+        ctx.set_mesh_dict(mesh)
+        ctx.load(0, **parts)
+        ctx.compute_fields()
+        phi = ctx.fields(G.PIC_FIELD_PHI)
+    sim = O.Sim(cfg, O.Mesh(nx, ny, h, 0, bc[0], bc[1]))
+    sim.load(0, **parts)
+    sim.fields()
+    # as above, the eigenvalues scaled by kappa = 1 + dt^2 n: at least 1, at most its largest
+    kmax = 1.0 + dt * dt * sim.counts(0).max() / 3.0
+    lam = 2.0 - 2.0 * np.cos(np.pi / max(nx, ny, 2))
+    bar = (1e-11 * 8.0 + 1e-13) * kmax / lam
+    assert np.linalg.norm(phi - sim.phi) <= bar * np.linalg.norm(sim.phi)
