@@ -58,6 +58,26 @@ template <typename R> __device__ __forceinline__ R below_one();
 template <> __device__ __forceinline__ float below_one<float>() { return 0.99999994f; }
 template <> __device__ __forceinline__ double below_one<double>() { return 0.99999999999999989; }
 
+// The integer part of x, rounded down (one conversion instruction).
+__device__ __forceinline__ int32_t floor_i(float x) { return __float2int_rd(x); }
+__device__ __forceinline__ int32_t floor_i(double x) { return __double2int_rd(x); }
+// x in [0, 1); in FP64 on the high word (an FP64 comparison takes the FP64 pipe)
+__device__ __forceinline__ bool in_unit(float x) { return x >= 0.0f && x < 1.0f; }
+__device__ __forceinline__ bool in_unit(double x) {
+    const uint32_t h = (uint32_t)__double2hiint(x);
+    return h < 0x3FF00000u || (h == 0x80000000u && __double2loint(x) == 0);
+}
+// 2^-k
+template <typename R> __device__ __forceinline__ R pow2_neg(int k);
+template <> __device__ __forceinline__ float pow2_neg<float>(int k) { return __int_as_float((127 - k) << 23); }
+template <> __device__ __forceinline__ double pow2_neg<double>(int k) { return __hiloint2double((1023 - k) << 20, 0); }
+// |x| truncated to FP32 by its bits, FP32's largest at most, (denormal) zero below FP32's range
+__device__ __forceinline__ float abs_f32(double x) {
+    const uint32_t t = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
+    const uint32_t e = min(max(t, 0x38000000u) - 0x38000000u, 0x0FEFFFFFu);
+    return __uint_as_float(__funnelshift_l((uint32_t)__double2loint(x), e, 3));
+}
+
 template <typename R> __device__ __forceinline__ R u24(uint32_t r) { return (R)(r >> 8) * (R)(1.0 / 16777216.0); }
 
 // Compensated accumulation (Kahan) of one lane, and an error-free combination of the lanes'
@@ -259,6 +279,11 @@ template <typename R> struct PushArgs {
     // the bound test of the pass: electrons sigma_el / sc, sigma_iz0 / sc, (n dt sc p_pad)^2 with
     // sc the larger nonzero cross section scale; ions 1 / (n dt sigma_el g_pad p_pad)
     R bnd_el, bnd_iz, bnd_q, bnd_inv;
+    // FP64 state: the same bound in FP32 (f_ok: its constants lie in FP32's range; else every
+    // particle goes on to the exact test): electrons n dt sc, m / (2 qe), the threshold (a little
+    // less), ions n dt sigma_el and the partner bound
+    float f_a, f_hm, f_th, f_g, f_el, f_iz;
+    int f_ok;
     PhiloxKeys keys;    // round keys of the seed
     PhiloxKeys2 keys2;  // the collision test's uniform: Philox2x32-10 keyed by seed and instance
     uint32_t inst_word, step;
@@ -287,18 +312,74 @@ template <typename R> __device__ __forceinline__ void normals3(const U4 &r, R n[
 // time instead of with one or two lanes of a chunk: the location of a particle that left its
 // leaf and its list slot there, and every collision beyond the bound test of the pass (the
 // exact test, the scattering, the ionization with its pair, the ion's partner draw).  A
-// per-warp ring of kQueue entries in shared memory holds them, in list order.
+// per-warp ring of kQueue entries in shared memory holds them, in list order.  FP64 state keeps
+// the collision candidates in a ring of their own: with one ring nearly every batch of 32 ran
+// the collision code (some 250 FP64 operations) for one or two candidates (512 x 16 discharge,
+// push 0.228 -> 0.173 ms per step).  In FP32 that code costs less than the second ring's words
+// and registers (grown streamer, push 1.57 ms with one ring, 1.64 with two).
 constexpr int kQueue = 64;
+template <typename R> constexpr bool two_rings() { return sizeof(R) == 8; }
 
 template <typename R> struct Queue {
+    // (two rings: the collision candidates; one: leavers too)
     R a[kQueue], b[kQueue];  // new offsets in the old leaf (a leaver's lie outside [0, 1))
     R vx[kQueue], vy[kQueue], vz[kQueue], w[kQueue];
-    uint32_t r0[kQueue];    // collision candidates: the test's uniform word
-    uint32_t id[kQueue], key[kQueue], cand[kQueue];
+    uint32_t r0[kQueue];    // the test's uniform word
+    uint32_t id[kQueue], key[kQueue];
+    uint32_t cand[two_rings<R>() ? 1 : kQueue];
     int32_t L[kQueue], dst[kQueue];  // dst: a stayer's slot, -1 for a leaver
+    // two rings: the leavers
+    static constexpr int kLeave = two_rings<R>() ? kQueue : 1;
+    R la[kLeave], lb[kLeave], lvx[kLeave], lvy[kLeave], lvz[kLeave], lw[kLeave];
+    uint32_t lid[kLeave], lkey[kLeave];
+    int32_t lL[kLeave];
 };
 
-// Deferred work of queue entry e; all 32 lanes call it (`valid`: the lane has an entry).
+// The finest-lattice cell (I, J) of offsets (u, v) of leaf L, wrapped or absorbed (false) at the
+// walls; X, Y: the offsets in lattice cells.
+template <typename R>
+__device__ __forceinline__ bool lattice_cell(const PushArgs<R> &a, int32_t L, R u, R v, R &X, R &Y, int32_t &I, int32_t &J) {
+    const int32_t s = 1 << (a.lmax - a.lev[L]);
+    X = u * (R)s; Y = v * (R)s;  // exact: s is a power of two
+    I = a.ix[L] + floor_i(X); J = a.iy[L] + floor_i(Y);
+    // periodic directions wrap modulo the period, however far the particle moved
+    if (I < 0 || I >= a.NX) {
+        if (!a.px) return false;
+        I %= a.NX;
+        if (I < 0) I += a.NX;
+    }
+    if (J < 0 || J >= a.NY) {
+        if (!a.py) return false;
+        J %= a.NY;
+        if (J < 0) J += a.NY;
+    }
+    return true;
+}
+// The leaf of that cell, and the offsets re-expressed in it.
+template <typename R>
+__device__ __forceinline__ int32_t new_leaf(const PushArgs<R> &a, R X, R Y, int32_t I, int32_t J, R &u, R &v) {
+    const int32_t nl = __ldg(a.map + (int64_t)J * a.NX + I);
+    const R inv_s2 = pow2_neg<R>(a.lmax - a.lev[nl]);
+    // I - floor(X) is the old leaf's corner after the periodic wrap
+    R un2 = ((R)(I - floor_i(X) - a.ix[nl]) + X) * inv_s2;
+    R vn2 = ((R)(J - floor_i(Y) - a.iy[nl]) + Y) * inv_s2;
+    un2 = un2 < (R)0 ? (R)0 : (un2 >= (R)1 ? below_one<R>() : un2);
+    vn2 = vn2 < (R)0 ? (R)0 : (vn2 >= (R)1 ? below_one<R>() : vn2);
+    u = un2; v = vn2;
+    return nl;
+}
+
+// Leaver e of the leavers' ring: located, re-expressed in its new leaf, given a slot there (an
+// absorbed particle enters no list).
+template <typename R> __device__ __forceinline__ void run_leaver(const PushArgs<R> &a, const Queue<R> &q, int e) {
+    R X, Y, u, v;
+    int32_t I, J;
+    if (!lattice_cell(a, q.lL[e], q.la[e], q.lb[e], X, Y, I, J)) return;
+    const int32_t nl = new_leaf(a, X, Y, I, J, u, v);
+    list_put(a.self, nl, u, v, q.lvx[e], q.lvy[e], q.lvz[e], q.lw[e], q.lid[e], q.lkey[e], 0u, a.err);
+}
+
+// Deferred work of ring entry e; all 32 lanes call it (`valid`: the lane has an entry).
 // Electrons that spawn are ranked among their leaf's spawning particles in list order: the
 // entries are in list order, and (run_leaf, run_count) carry the count of the last leaf of
 // the previous batch, whose entries may continue in this one.
@@ -306,32 +387,22 @@ template <typename R, int S>
 __device__ __forceinline__ void run_deferred(const PushArgs<R> &a, const Queue<R> &q, int e, bool valid, uint32_t span,
                                              uint32_t ion_span, uint32_t step, int32_t &run_leaf, int32_t &run_count) {
     R vx = 0, vy = 0, vz = 0, w = 0;
-    uint32_t id = 0, cand = 0;
+    uint32_t id = 0;
+    bool cand = false;
     int32_t L = -1, dst = -1;
     if (valid) {
         vx = q.vx[e]; vy = q.vy[e]; vz = q.vz[e]; w = q.w[e];
-        id = q.id[e]; cand = q.cand[e];
+        id = q.id[e];
+        cand = two_rings<R>() || q.cand[two_rings<R>() ? 0 : e];
         L = q.L[e]; dst = q.dst[e];
     }
-    // a leaver: the finest-lattice cell of its new position, wrapped or absorbed at the walls
-    // (an absorbed particle neither collides nor enters a list)
+    // a leaver absorbed at a wall neither collides nor enters a list
     R X = 0, Y = 0;
     int32_t I = 0, J = 0;
     bool alive = true;
     if (valid && dst < 0) {
-        const int32_t s = 1 << (a.lmax - a.lev[L]);
-        X = q.a[e] * (R)s; Y = q.b[e] * (R)s;  // exact: s is a power of two
-        I = a.ix[L] + (int32_t)m_floor(X); J = a.iy[L] + (int32_t)m_floor(Y);
-        // periodic directions wrap modulo the period, however far the particle moved
-        if (I < 0 || I >= a.NX) {
-            if (!a.px) alive = false;
-            else { I %= a.NX; if (I < 0) I += a.NX; }
-        }
-        if (J < 0 || J >= a.NY) {
-            if (!a.py) alive = false;
-            else { J %= a.NY; if (J < 0) J += a.NY; }
-        }
-        if (!alive) cand = 0;
+        alive = lattice_cell(a, L, q.a[e], q.b[e], X, Y, I, J);
+        cand = cand && alive;
     }
     R sv[3] = {0, 0, 0}, si[3] = {0, 0, 0};
     bool spawns = false;
@@ -412,16 +483,8 @@ __device__ __forceinline__ void run_deferred(const PushArgs<R> &a, const Queue<R
         a.d.vx[dst] = vx; a.d.vy[dst] = vy; a.d.vz[dst] = vz;
         nl = L;
         u = q.a[e]; v = q.b[e];
-    } else {         // entering: locate, re-express the offsets in the new leaf, take a slot
-        nl = __ldg(a.map + (int64_t)J * a.NX + I);
-        const int32_t s2 = 1 << (a.lmax - a.lev[nl]);
-        const R inv_s2 = (R)1 / (R)s2;
-        // I - floor(X) is the old leaf's corner after the periodic wrap
-        R un2 = ((R)(I - (int32_t)m_floor(X) - a.ix[nl]) + X) * inv_s2;
-        R vn2 = ((R)(J - (int32_t)m_floor(Y) - a.iy[nl]) + Y) * inv_s2;
-        un2 = un2 < (R)0 ? (R)0 : (un2 >= (R)1 ? below_one<R>() : un2);
-        vn2 = vn2 < (R)0 ? (R)0 : (vn2 >= (R)1 ? below_one<R>() : vn2);
-        u = un2; v = vn2;
+    } else {
+        nl = new_leaf(a, X, Y, I, J, u, v);
         list_put(a.self, nl, u, v, vx, vy, vz, w, id, q.key[e], 0u, a.err);
     }
     if (spawns) {
@@ -439,7 +502,8 @@ __device__ __forceinline__ void run_deferred(const PushArgs<R> &a, const Queue<R
 // chunk lies beyond every slot it writes in this one.  Entering and spawned records only go
 // to free slots past end[], which no warp reads during the pass.
 // NT threads per block (a tuned launch shape); 768 threads per SM either way: 80 registers
-// (a 64-register build for 1024 threads spills and runs slower).
+// (a 64-register build for 1024 threads spills and runs slower); FP64 state 512 threads and 128
+// registers (80 spill 340 bytes, and the FP64 pipe, not the loads, bounds the pass).
 // CIC: the field is gathered from the leaf's per-quarter cloud-in-cell coefficients (32 per
 // leaf, lane k holding coefficient k) instead of the bilinear corner field.
 // The warp walks the leaves first, first + nw, ... below last (all lanes call it).  S: the
@@ -454,7 +518,7 @@ __device__ __forceinline__ void push_leaves(const PushArgs<R> &a, Queue<R> &q, c
     const uint32_t span = (uint32_t)a.rank0[a.nleaf];
     const uint32_t ion_span = a.ion_total ? (uint32_t)*a.ion_total : 0u;
     const uint32_t step = a.step_dev ? (uint32_t)*a.step_dev : a.step;
-    int qhead = 0, qn = 0;  // ring of deferred entries
+    int qhead = 0, qn = 0, lhead = 0, ln = 0;  // rings of deferred entries
     int32_t run_leaf = -1, run_count = 0;  // spawn count of the last leaf seen by the deferred work
     // Persistent warps, software-pipelined: the next chunk's records are loaded while this
     // chunk computes, and during a leaf's last chunk that is the first chunk of the warp's
@@ -534,11 +598,20 @@ __device__ __forceinline__ void push_leaves(const PushArgs<R> &a, Queue<R> &q, c
                 }
                 // leapfrog kick and drift in leaf units (the implicit scheme's predictor has no
                 // kick; its corrector drifts by the kick's increment)
-                const R dvx = a.qm_dt * ex, dvy = a.qm_dt * ey;
-                vx += dvx;
-                vy += dvy;
-                const R un = u + (a.drift_kick ? dvx : vx) * dth, vn = v + (a.drift_kick ? dvy : vy) * dth;
-                if (un >= (R)0 && un < (R)1 && vn >= (R)0 && vn < (R)1) {
+                R sx, sy;  // drift velocities
+                if constexpr (sizeof(R) == 8) {
+                    vx = fma(a.qm_dt, ex, vx);
+                    vy = fma(a.qm_dt, ey, vy);
+                    sx = vx; sy = vy;
+                    if (a.drift_kick) { sx = a.qm_dt * ex; sy = a.qm_dt * ey; }
+                } else {
+                    const R dvx = a.qm_dt * ex, dvy = a.qm_dt * ey;
+                    vx += dvx;
+                    vy += dvy;
+                    sx = a.drift_kick ? dvx : vx; sy = a.drift_kick ? dvy : vy;
+                }
+                const R un = u + sx * dth, vn = v + sy * dth;
+                if (in_unit(un) && in_unit(vn)) {
                     stays = true;
                     u = un; v = vn;
                 } else {
@@ -568,14 +641,28 @@ __device__ __forceinline__ void push_leaves(const PushArgs<R> &a, Queue<R> &q, c
                     }
                 }
                 if (a.mcc) {
-                    const R v2 = vx * vx + vy * vy + vz * vz;
                     // the test's uniform: Philox2x32-10 on the counter (id, step); the deferred
                     // work draws the collision's other uniforms from the 4x32 purpose-0 stream
                     r0x = philox2x32_10_x(id, step, a.keys2);
-                    const R U0 = u24<R>(r0x);
                     // 1 - exp(-x) <= x: a uniform at or above the bound x (with a rounding
                     // margin) means no collision; below it the deferred work makes the exact test
-                    if constexpr (S == 0) {
+                    if constexpr (sizeof(R) == 8) {
+                        // FP64 state: the bound in FP32, whose rounding (1e-6) the margin holds (1e-4;
+                        // the threshold is taken 1e-5 low, since 1 - eps_th / eps cancels), so it
+                        // passes every particle the exact test can collide.  GB300 retires two FP64
+                        // lanes per clock and SM: this test took 19 of the pass's ~38 FP64 operations.
+                        const float fx = abs_f32(vx), fy = abs_f32(vy), fz = abs_f32(vz);
+                        const float v2 = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
+                        float x;
+                        if constexpr (S == 0) {
+                            const float T = a.f_el + a.f_iz * fmaxf(0.0f, 1.0f - __fdividef(a.f_th, a.f_hm * v2));
+                            x = a.f_a * sqrtf(v2) * T;
+                        } else {
+                            x = a.f_a * (sqrtf(v2) + a.f_g);
+                        }
+                        cand = !(u24<float>(r0x) >= x) || r0x < 256u || !a.f_ok;
+                    } else if constexpr (S == 0) {
+                        const R U0 = u24<R>(r0x), v2 = vx * vx + vy * vy + vz * vz;
                         // x = n dt sigma(eps) |v| with eps sigma(eps) = sc T(eps), squared so that
                         // neither a root nor a division is needed: U0 < x pad iff
                         // (U0 eps)^2 < (n dt sc pad)^2 v^2 T^2 (a zero uniform always goes on)
@@ -584,6 +671,7 @@ __device__ __forceinline__ void push_leaves(const PushArgs<R> &a, Queue<R> &q, c
                         const R ue = U0 * eps;
                         cand = ue * ue < a.bnd_q * v2 * (T * T) || r0x < 256u;
                     } else {
+                        const R U0 = u24<R>(r0x), v2 = vx * vx + vy * vy + vz * vz;
                         // the Box-Muller partner speed is at most 8.157 v_t (24-bit uniforms):
                         // U0 < B (|v| + g) iff U0 / B - g < 0 or (U0 / B - g)^2 < v^2
                         const R x = U0 * a.bnd_inv - a.g_partner_max;
@@ -592,7 +680,7 @@ __device__ __forceinline__ void push_leaves(const PushArgs<R> &a, Queue<R> &q, c
                 }
             }
             const uint32_t stay_mask = __ballot_sync(0xFFFFFFFFu, live && stays);
-            const bool defer = live && (!stays || cand);
+            const bool defer = two_rings<R>() ? cand : live && (!stays || cand);
             const uint32_t defer_mask = __ballot_sync(0xFFFFFFFFu, defer);
             int32_t dst = -1;
             if (live && stays) {
@@ -602,12 +690,33 @@ __device__ __forceinline__ void push_leaves(const PushArgs<R> &a, Queue<R> &q, c
                 if (!cand) { a.d.vx[dst] = vx; a.d.vy[dst] = vy; a.d.vz[dst] = vz; }
                 if (dst != p) { a.d.w[dst] = w; a.d.id[dst] = id; }
             }
+            if constexpr (two_rings<R>()) {
+                const bool leaves = live && !stays && !cand;
+                const uint32_t leave_mask = __ballot_sync(0xFFFFFFFFu, leaves);
+                if (leave_mask) {
+                    if (leaves) {
+                        const int e = (lhead + ln + __popc(leave_mask & lanemask_lt())) & (kQueue - 1);
+                        q.la[e] = u; q.lb[e] = v;
+                        q.lvx[e] = vx; q.lvy[e] = vy; q.lvz[e] = vz; q.lw[e] = w;
+                        q.lid[e] = id; q.lkey[e] = key0 + (uint32_t)p;
+                        q.lL[e] = L;
+                    }
+                    ln += __popc(leave_mask);
+                    if (ln >= 32) {
+                        __syncwarp();
+                        run_leaver(a, q, (lhead + lane) & (kQueue - 1));
+                        __syncwarp();
+                        lhead = (lhead + 32) & (kQueue - 1);
+                        ln -= 32;
+                    }
+                }
+            }
             if (defer_mask) {
                 if (defer) {
                     const int e = (qhead + qn + __popc(defer_mask & lanemask_lt())) & (kQueue - 1);
                     q.a[e] = u; q.b[e] = v;
                     q.vx[e] = vx; q.vy[e] = vy; q.vz[e] = vz; q.w[e] = w;
-                    q.cand[e] = cand ? 1u : 0u;
+                    if constexpr (!two_rings<R>()) q.cand[e] = cand ? 1u : 0u;
                     q.r0[e] = r0x;
                     q.id[e] = id; q.key[e] = key0 + (uint32_t)p;
                     q.L[e] = L; q.dst[e] = dst;
@@ -631,6 +740,9 @@ __device__ __forceinline__ void push_leaves(const PushArgs<R> &a, Queue<R> &q, c
         }
     }
     __syncwarp();
+    if constexpr (two_rings<R>())
+        if (lane < ln) run_leaver(a, q, (lhead + lane) & (kQueue - 1));
+    __syncwarp();
     if (qn > 0) run_deferred<R, S>(a, q, (qhead + lane) & (kQueue - 1), lane < qn, span, ion_span, step, run_leaf, run_count);
 }
 
@@ -639,12 +751,13 @@ __device__ __forceinline__ void push_leaves(const PushArgs<R> &a, Queue<R> &q, c
 // launches left the SMs idle while the last warps of the first finished).  The species touch
 // each other's lists only through spawned ions, which take atomic slots past every list's end
 // and are ordered by key afterwards.
+template <typename R> constexpr int push_threads_per_sm() { return sizeof(R) == 8 ? 512 : 768; }
 template <typename R> struct PushPair {
     PushArgs<R> e[2];
     unsigned n0;
 };
 template <typename R, int NT, bool CIC>
-__global__ void __launch_bounds__(NT, 768 / NT) k_push(const __grid_constant__ PushPair<R> P) {
+__global__ void __launch_bounds__(NT, push_threads_per_sm<R>() / NT) k_push(const __grid_constant__ PushPair<R> P) {
     pdl_chain();
     extern __shared__ unsigned char push_smem[];
     Queue<R> &q = reinterpret_cast<Queue<R> *>(push_smem)[threadIdx.x >> 5];
@@ -660,7 +773,7 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_push(const __grid_constant__ P
 // Every instance of an ensemble in one launch: block b takes the leaves [c.y, c.z) of
 // instance c.x (c = chunks[b]), the instance's arguments copied to shared memory.
 template <typename R, int NT, bool CIC, int S>
-__global__ void __launch_bounds__(NT, 768 / NT) k_push_batch(const PushArgs<R> *__restrict__ tab,
+__global__ void __launch_bounds__(NT, push_threads_per_sm<R>() / NT) k_push_batch(const PushArgs<R> *__restrict__ tab,
                                                              const int4 *__restrict__ chunks) {
     extern __shared__ unsigned char push_smem[];
     __shared__ PushArgs<R> sa;
@@ -1333,6 +1446,18 @@ template <typename R> PushArgs<R> push_args(Instance &in, int s, int64_t step) {
         a.bnd_q = (R)(A * A);
         const double B = c.gas_density * c.dt * c.sigma_el * 1.001 * 1.0001;
         a.bnd_inv = B > 0.0 ? (R)(1.0 / B) : (R)INFINITY;
+        auto normal = [](double v) { return v == 0.0 || (v > 1e-30 && v < 1e30); };
+        const double hm = 0.5 * c.m[s] / c.qe, g = 8.2 * std::sqrt(c.gas_temperature_ev * c.qe / c.neutral_mass);
+        a.f_a = (float)(s == 0 ? A * 1.00001 : B);
+        a.f_hm = (float)hm;
+        a.f_th = (float)(c.eps_th_ev * 0.99999);
+        a.f_g = (float)(g * 1.00001);
+        a.f_el = (float)(c.sigma_el / sc);
+        a.f_iz = (float)(c.sigma_iz0 / sc);
+        // a collision frequency factor below FP32's range bounds the probability of any speed FP32
+        // holds by 1e-11, which only the zero uniform is below; one above it makes the bound infinite
+        a.f_ok = hm > 0.0 && normal(hm) && normal(c.eps_th_ev) && c.eps_th_ev >= 0.0 && normal(g) && std::isfinite(A) &&
+                 std::isfinite(B) && c.sigma_el / sc < 1e6 && c.sigma_iz0 / sc < 1e6;
     }
     a.keys = philox_keys(c.seed);
     a.inst_word = (uint32_t)c.instance << 24;
