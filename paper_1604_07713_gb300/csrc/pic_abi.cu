@@ -197,6 +197,12 @@ template <typename F> pic_status guarded(pic_ctx *ctx, F &&f) {
     }
 }
 
+// A read-out's capacity is too small (also how a caller asks for the size: no exception).
+pic_status too_small() {
+    set_error("output capacity too small");
+    return PIC_EINVAL;
+}
+
 void validate(const pic_config &c) {
     if (c.precision != PIC_FP32 && c.precision != PIC_FP64) fail(PIC_EINVAL, "precision must be PIC_FP32 or PIC_FP64");
     if (c.n_species < 1 || c.n_species > 2) fail(PIC_EINVAL, "n_species must be 1 or 2");
@@ -247,7 +253,10 @@ double collect_solver_stats(pic_ctx *ctx, Instance &in) {
 void ensure_species(pic_ctx *ctx, Instance &in) {
     // a species never loaded is an empty population
     for (int s = 0; s < in.cfg.n_species; ++s)
-        if (!in.sp[s].start) species_alloc(ctx, in, s, 1 << 16);
+        if (!in.sp[s].start) {
+            in.counts_exact = false;
+            species_alloc(ctx, in, s, 1 << 16);
+        }
 }
 
 }  // namespace
@@ -256,6 +265,7 @@ void ensure_species(pic_ctx *ctx, Instance &in) {
 // arrays, multigrid levels and the corner-field array built.
 void gbpic::set_mesh_impl(pic_ctx *ctx, Instance &in, int nx0, int ny0, double h0, int64_t n_leaves,
                           const uint32_t *root, const uint32_t *morton, const uint8_t *level) {
+    in.counts_exact = false;
     in.part_mem[0].release_all();
     in.part_mem[1].release_all();
     for (auto &sp : in.sp) sp = Species();
@@ -632,23 +642,23 @@ pic_status pic_read_fields(pic_ctx *ctx, int32_t inst, int32_t field, double *ou
         int64_t need = field == PIC_FIELD_NODE_E ? 8 * nl : nl;
         if (field < PIC_FIELD_PHI || field > PIC_FIELD_AVG_PHI) fail(PIC_EINVAL, "unknown field");
         if (n_out) *n_out = need;
-        if (!out || cap < need) fail(PIC_EINVAL, "output capacity too small");
+        if (!out || cap < need) return too_small();
         cudaStream_t st = ctx->stream;
-        std::vector<uint8_t> lev(nl);
+        DeviceArena tmp(&ctx->cache);
+        // a field formed on the device in FP64, then one copy to the caller
+        auto copy_out = [&](const double *d) {
+            GB_CUDA(cudaMemcpyAsync(out, d, need * 8, cudaMemcpyDeviceToHost, st));
+            GB_CUDA(cudaStreamSynchronize(st));
+            tmp.release_all();
+        };
         switch (field) {
         case PIC_FIELD_PHI:
-            GB_CUDA(cudaMemcpyAsync(out, in.phi, nl * 8, cudaMemcpyDeviceToHost, st));
-            GB_CUDA(cudaStreamSynchronize(st));
+            copy_out(in.phi);
             break;
         case PIC_FIELD_RHO: {
-            GB_CUDA(cudaMemcpyAsync(out, in.charge, nl * 8, cudaMemcpyDeviceToHost, st));
-            GB_CUDA(cudaMemcpyAsync(lev.data(), in.lv[0].lev, nl, cudaMemcpyDeviceToHost, st));
-            GB_CUDA(cudaStreamSynchronize(st));
-            const double hf = in.h0 / (double)(1 << in.lmax);
-            for (int64_t l = 0; l < nl; ++l) {
-                const double h = (double)(1 << (in.lmax - lev[l])) * hf;
-                out[l] = out[l] / (h * h) + in.cfg.rho_background;
-            }
+            double *d = dalloc<double>(tmp, nl);
+            read_rho(ctx, in, d);
+            copy_out(d);
             break;
         }
         case PIC_FIELD_COUNT_E:
@@ -658,42 +668,32 @@ pic_status pic_read_fields(pic_ctx *ctx, int32_t inst, int32_t field, double *ou
                 std::fill(out, out + nl, 0.0);
                 break;
             }
-            std::vector<int32_t> st0(nl), en0(nl);
-            GB_CUDA(cudaMemcpyAsync(st0.data(), in.sp[s].start, nl * 4, cudaMemcpyDeviceToHost, st));
-            GB_CUDA(cudaMemcpyAsync(en0.data(), in.sp[s].end, nl * 4, cudaMemcpyDeviceToHost, st));
-            GB_CUDA(cudaStreamSynchronize(st));
-            for (int64_t l = 0; l < nl; ++l) out[l] = (double)(en0[l] - st0[l]);
+            double *d = dalloc<double>(tmp, nl);
+            read_leaf_counts(ctx, in, s, d);
+            copy_out(d);
             break;
         }
         case PIC_FIELD_NODE_E:
             if (in.cfg.precision == PIC_FP64) {
-                GB_CUDA(cudaMemcpyAsync(out, in.stencil, 8 * nl * 8, cudaMemcpyDeviceToHost, st));
-                GB_CUDA(cudaStreamSynchronize(st));
+                copy_out((const double *)in.stencil);
             } else {
-                std::vector<float> tmp(8 * nl);
-                GB_CUDA(cudaMemcpyAsync(tmp.data(), in.stencil, 8 * nl * 4, cudaMemcpyDeviceToHost, st));
-                GB_CUDA(cudaStreamSynchronize(st));
-                for (int64_t i = 0; i < 8 * nl; ++i) out[i] = tmp[i];
+                double *d = dalloc<double>(tmp, need);
+                read_widened(ctx, (const float *)in.stencil, need, d);
+                copy_out(d);
             }
             break;
         case PIC_FIELD_EMAG: {
-            DeviceArena tmp(&ctx->cache);
             double *d = dalloc<double>(tmp, nl);
             double walls[4];
             walls_at(in, ctx->step, walls);
             cell_emag(ctx, in, walls, d);
-            GB_CUDA(cudaMemcpyAsync(out, d, nl * 8, cudaMemcpyDeviceToHost, st));
-            GB_CUDA(cudaStreamSynchronize(st));
-            tmp.release_all();
+            copy_out(d);
             break;
         }
         default: {  // time averages
-            DeviceArena tmp(&ctx->cache);
             double *d = dalloc<double>(tmp, nl);
             diag_read_field(ctx, in, field, d);
-            GB_CUDA(cudaMemcpyAsync(out, d, nl * 8, cudaMemcpyDeviceToHost, st));
-            GB_CUDA(cudaStreamSynchronize(st));
-            tmp.release_all();
+            copy_out(d);
             break;
         }
         }
@@ -708,7 +708,7 @@ pic_status pic_read_mesh(pic_ctx *ctx, int32_t inst, uint32_t *root, uint32_t *m
         if (!in.has_mesh) fail(PIC_EINVAL, "mesh not set");
         const int64_t nl = in.nleaf;
         if (n_out) *n_out = nl;
-        if (cap < nl) fail(PIC_EINVAL, "output capacity too small");
+        if (cap < nl) return too_small();
         cudaStream_t st = ctx->stream;
         if (root) GB_CUDA(cudaMemcpyAsync(root, in.root, nl * 4, cudaMemcpyDeviceToHost, st));
         if (morton) GB_CUDA(cudaMemcpyAsync(morton, in.morton, nl * 4, cudaMemcpyDeviceToHost, st));
@@ -729,7 +729,7 @@ pic_status pic_read_particles(pic_ctx *ctx, int32_t inst, int32_t species, doubl
         Species &sp = in.sp[species];
         refresh_counts(ctx, in);
         if (n_out) *n_out = sp.n;
-        if (cap < sp.n) fail(PIC_EINVAL, "output capacity too small");
+        if (cap < sp.n) return too_small();
         particles_read(ctx, in, species, x, y, vx, vy, vz, w, id, leaf);
         return PIC_OK;
     });
@@ -856,7 +856,7 @@ pic_status pic_read_eedf(pic_ctx *ctx, int32_t inst, double *f, int64_t cap, int
         Instance &in = get_inst(ctx, inst);
         if (!in.diag.on) fail(PIC_EINVAL, "diagnostics are off (pic_diag_enable)");
         if (n_out) *n_out = in.diag.nbins;
-        if (!f || cap < in.diag.nbins) fail(PIC_EINVAL, "output capacity too small");
+        if (!f || cap < in.diag.nbins) return too_small();
         diag_read_eedf(ctx, in, f, samples);
         return PIC_OK;
     });

@@ -655,6 +655,7 @@ template <typename R> void adapt_particles(pic_ctx *ctx, Instance &in, int64_t n
 }
 
 template <typename R> void split_merge_impl(pic_ctx *ctx, Instance &in) {
+    in.counts_exact = false;
     cudaStream_t st = ctx->stream;
     const int64_t nl = in.nleaf;
     DeviceArena T(&ctx->cache);
@@ -722,6 +723,7 @@ template <typename R> void split_merge_impl(pic_ctx *ctx, Instance &in) {
     GB_CUDA(cudaStreamSynchronize(st));
     in.next_id = (int64_t)next_id;
     T.release_all();
+    in.counts_exact = false;
     refresh_counts(ctx, in);
 }
 

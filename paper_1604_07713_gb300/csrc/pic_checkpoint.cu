@@ -269,6 +269,7 @@ int64_t checkpoint_write(pic_ctx *ctx, Instance &in, void *buf, int64_t cap) {
 }
 
 void checkpoint_read(pic_ctx *ctx, Instance &in, const void *buf, int64_t bytes) {
+    in.counts_exact = false;
     if (!buf || bytes < (int64_t)sizeof(Header)) fail(PIC_EINVAL, "checkpoint: buffer too small");
     Reader r{static_cast<const uint8_t *>(buf), static_cast<const uint8_t *>(buf) + bytes};
     const Header h = r.get<Header>();

@@ -32,16 +32,19 @@ struct ReportTab {
 };
 struct Report {
     int32_t tot[2];
-    int32_t err, pad;
-    double mg[3];  // cycles, relative residual, worst relative residual since the reset
+    int32_t err;
+    uint32_t ticket;  // device copy: blocks that have added their totals
+    double mg[3];     // cycles, relative residual, worst relative residual since the reset
 };
 
-// Blocks (x) over the leaves of instance y: record totals per species (out zeroed before),
-// and from block 0 the consistency flag and the solver statistics.
-__global__ void k_report(const ReportTab *__restrict__ tab, Report *__restrict__ out) {
-    __shared__ int32_t part[kT / 32];
+// Blocks (x) over the leaves of instance y add the record totals per species; the block that
+// arrives last on the instance's ticket writes the totals, the consistency flag and the solver
+// statistics to the host's copy (pinned) and zeroes the accumulators for the next report.
+__global__ void __launch_bounds__(kT) k_report(const ReportTab *__restrict__ tab, Report *__restrict__ acc,
+                                               Report *__restrict__ host) {
+    __shared__ int32_t part[2][kT / 32];
     const ReportTab &t = tab[blockIdx.y];
-    Report &r = out[blockIdx.y];
+    Report &r = acc[blockIdx.y];
     for (int s = 0; s < 2; ++s) {
         int32_t c = 0;
         if (s < t.nsp)
@@ -49,20 +52,23 @@ __global__ void k_report(const ReportTab *__restrict__ tab, Report *__restrict__
                  L += (int64_t)gridDim.x * blockDim.x)
                 c += t.end[s][L] - t.start[s][L];
         for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
-        if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = c;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int32_t tot = 0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += part[w];
-            if (tot) atomicAdd(&r.tot[s], tot);
-        }
-        __syncthreads();
+        if ((threadIdx.x & 31) == 0) part[s][threadIdx.x >> 5] = c;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        r.err = *t.err;
-        r.pad = 0;
-        for (int k = 0; k < 3; ++k) r.mg[k] = t.mg_stats ? t.mg_stats[k] : 0.0;
+    __syncthreads();
+    if (threadIdx.x) return;
+    for (int s = 0; s < 2; ++s) {
+        int32_t tot = 0;
+        for (int w = 0; w < kT / 32; ++w) tot += part[s][w];
+        if (tot) atomicAdd(&r.tot[s], tot);
     }
+    __threadfence();
+    if (atomicAdd(&r.ticket, 1u) != gridDim.x - 1) return;
+    __threadfence();
+    Report &h = host[blockIdx.y];
+    for (int s = 0; s < 2; ++s) h.tot[s] = atomicExch(&r.tot[s], 0);
+    h.err = *t.err;
+    for (int k = 0; k < 3; ++k) h.mg[k] = t.mg_stats ? t.mg_stats[k] : 0.0;
+    r.ticket = 0u;
 }
 
 // The parallel branches of a captured step (their number is a tuned launch shape).
@@ -210,6 +216,7 @@ void graph_prepare(pic_ctx *ctx) {
 }
 
 void one_step(pic_ctx *ctx) {
+    for (Instance &in : ctx->inst) in.counts_exact = false;
     for (Instance &in : ctx->inst) ensure_capacity(ctx, in);
     if (graph_step_possible(ctx)) {
         graph_step(ctx);  // an ensemble in steady state: the whole step as one graph replay
@@ -324,6 +331,7 @@ void report_all(pic_ctx *ctx) {
     const int64_t epoch = ctx->mesh_epoch * 1000003 + ctx->lists_epoch;
     if (!ctx->report_dev) {
         GB_CUDA(cudaMalloc(&ctx->report_dev, n * sizeof(Report)));
+        GB_CUDA(cudaMemsetAsync(ctx->report_dev, 0, n * sizeof(Report), st));
         GB_CUDA(cudaMallocHost(&ctx->report_host, n * sizeof(Report)));
         GB_CUDA(cudaMalloc(&ctx->report_tab, n * sizeof(ReportTab)));
     }
@@ -348,15 +356,14 @@ void report_all(pic_ctx *ctx) {
     int64_t maxl = 0;
     for (Instance &in : ctx->inst) maxl = std::max(maxl, in.nleaf);
     const dim3 grid((unsigned)std::min<int64_t>(std::max<int64_t>(1, (maxl + 8 * kT - 1) / (8 * kT)), 128), n);
-    GB_CUDA(cudaMemsetAsync(ctx->report_dev, 0, n * sizeof(Report), st));
-    k_report<<<grid, kT, 0, st>>>((const ReportTab *)ctx->report_tab, (Report *)ctx->report_dev);
+    k_report<<<grid, kT, 0, st>>>((const ReportTab *)ctx->report_tab, (Report *)ctx->report_dev, (Report *)ctx->report_host);
     count_launch(ctx);
-    GB_CUDA(cudaMemcpyAsync(ctx->report_host, ctx->report_dev, n * sizeof(Report), cudaMemcpyDeviceToHost, st));
     GB_CUDA(cudaStreamSynchronize(st));
     const Report *r = (const Report *)ctx->report_host;
     for (int i = 0; i < n; ++i) {
         Instance &in = ctx->inst[i];
         for (int s = 0; s < in.cfg.n_species; ++s) in.sp[s].n = in.sp[s].n_upper = r[i].tot[s];
+        in.counts_exact = true;
         in.report_err = r[i].err;
         if (in.mg_on_device && in.mg_stats) {
             in.mg_cycles = (int)r[i].mg[0];

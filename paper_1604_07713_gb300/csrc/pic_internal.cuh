@@ -212,6 +212,7 @@ struct Instance {
     int32_t *d_err = nullptr;                // device-side consistency flag (0 = fine)
     double *d_walls = nullptr;               // the context's wall array for this instance (4)
     int32_t report_err = 0;                  // consistency flag read by the last report
+    bool counts_exact = false;               // sp[].n are the record totals (no step or change since they were read)
     double mg_worst = 0;                     // worst relative residual of the solves since the reset
     int mg_cycles = 0;
     double mg_res = 0;
@@ -531,6 +532,10 @@ void lists_from_counts(pic_ctx *ctx, Species &sp, int64_t nl, const int32_t *cnt
 void lists_installed(pic_ctx *ctx, Species &sp, int64_t nl);  // lim, tail after start / end are set
 void list_ranks(pic_ctx *ctx, Instance &in, int s);             // rank0 from start / end
 void count_totals(pic_ctx *ctx, Instance &in);  // flags[1] of every species, device side
+// fields as the read-outs give them, formed on the device (pic_lists.cu, pic_mesh.cu)
+void read_leaf_counts(pic_ctx *ctx, Instance &in, int s, double *out_dev);
+void read_rho(pic_ctx *ctx, Instance &in, double *out_dev);
+void read_widened(pic_ctx *ctx, const float *src_dev, int64_t n, double *out_dev);
 void step_lists_prep(pic_ctx *ctx, Instance &in, bool ionize);  // list ranks of every species, step reset
 void step_repairs(pic_ctx *ctx, Instance &in, bool ionize);     // spawn offsets; tail moves, else re-layout
 BatchTab batch_prepare_lists(pic_ctx *ctx);                // per (instance, species) list arrays

@@ -958,6 +958,17 @@ void step_repairs(pic_ctx *ctx, Instance &in, bool ionize) {
     else step_repairs_impl<float>(ctx, in, ionize);
 }
 
+__global__ void k_read_counts(int64_t nl, const int32_t *__restrict__ start, const int32_t *__restrict__ end,
+                              double *__restrict__ out) {
+    const int64_t L = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (L < nl) out[L] = (double)(end[L] - start[L]);
+}
+void read_leaf_counts(pic_ctx *ctx, Instance &in, int s, double *out_dev) {
+    k_read_counts<<<blocks_for(in.nleaf), kT, 0, ctx->stream>>>(in.nleaf, in.sp[s].start, in.sp[s].end, out_dev);
+    count_launch(ctx);
+    check_launch("read_leaf_counts");
+}
+
 // Lay species s's lists out again in leaf order with fresh free slots (frees the tail).
 void species_compact(pic_ctx *ctx, Instance &in, int s) {
     Species &sp = in.sp[s];

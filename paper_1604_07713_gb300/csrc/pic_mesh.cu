@@ -710,6 +710,30 @@ void node_e(pic_ctx *ctx, Instance &in, const double walls[4]) {
     if (in.cfg.shape != PIC_SHAPE_NGP) cic_patch(ctx, in, walls);  // the push gathers from it
 }
 
+__global__ void k_read_rho(int64_t n, const double *__restrict__ charge, const uint8_t *__restrict__ lev, int lmax,
+                           double hf, double rho_bg, double *__restrict__ out) {
+    const int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (l >= n) return;
+    const double h = (double)(1 << (lmax - lev[l])) * hf;
+    out[l] = __dadd_rn(charge[l] / __dmul_rn(h, h), rho_bg);
+}
+void read_rho(pic_ctx *ctx, Instance &in, double *out_dev) {
+    const Level &g = in.lv[0];
+    k_read_rho<<<blocks_for(g.n), kT, 0, ctx->stream>>>(g.n, in.charge, g.lev, in.lmax,
+                                                        in.h0 / (double)(1 << in.lmax), in.cfg.rho_background, out_dev);
+    count_launch(ctx);
+    check_launch("read_rho");
+}
+__global__ void k_widen(int64_t n, const float *__restrict__ src, double *__restrict__ out) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) out[i] = (double)src[i];
+}
+void read_widened(pic_ctx *ctx, const float *src_dev, int64_t n, double *out_dev) {
+    k_widen<<<blocks_for(n), kT, 0, ctx->stream>>>(n, src_dev, out_dev);
+    count_launch(ctx);
+    check_launch("read_widened");
+}
+
 void cell_emag(pic_ctx *ctx, Instance &in, const double walls[4], double *out_dev) {
     Level &g = in.lv[0];
     k_cell_emag<<<blocks_for(g.n), kT, 0, ctx->stream>>>(g.n, field_view<double>(in, walls), out_dev);

@@ -1635,6 +1635,7 @@ void particles_load(pic_ctx *ctx, Instance &in, int s, int64_t n, const double *
     cudaStream_t st = ctx->stream;
     Species &sp = in.sp[s];
     const int64_t nl = in.nleaf;
+    in.counts_exact = false;
     unsigned long long next_id = 0;
     GB_CUDA(cudaMemcpyAsync(&next_id, in.d_next_id, 8, cudaMemcpyDeviceToHost, st));
     GB_CUDA(cudaStreamSynchronize(st));
@@ -1848,6 +1849,7 @@ void particle_bookkeeping(Instance &in) {
 
 // Exact record totals into sp.n (one sync).
 void refresh_counts(pic_ctx *ctx, Instance &in) {
+    if (in.counts_exact) return;
     count_totals(ctx, in);
     for (int s = 0; s < in.cfg.n_species; ++s)
         if (in.sp[s].start)
@@ -1855,6 +1857,7 @@ void refresh_counts(pic_ctx *ctx, Instance &in) {
     GB_CUDA(cudaStreamSynchronize(ctx->stream));
     for (int s = 0; s < in.cfg.n_species; ++s)
         if (in.sp[s].start) in.sp[s].n = in.sp[s].n_upper = in.cnt_host[s];
+    in.counts_exact = true;
 }
 
 void particles_read(pic_ctx *ctx, Instance &in, int s, double *x, double *y, double *vx, double *vy,
