@@ -122,31 +122,46 @@ struct DepositArgs {
     double chi[2];           // dt^2 q_s^2 / (m_s eps0)
 };
 
+// From the records (after a load, an adaptation or split/merge): a warp sums `per` consecutive
+// leaves one after another, and lane i then forms leaf i's charge and right-hand side.  With
+// one leaf a warp, every warp issued the ~25 FP64 instructions of a leaf for itself (an SM's
+// FP64 pipe takes two lanes a clock).  Streamer of 8.8e7 records on 9e5 leaves, ten steps of
+// which the first deposits this way: 0.14 -> 0.061 ms per step.
 template <typename R>
-__global__ void __launch_bounds__(kT) k_deposit(DepositArgs a) {
+__global__ void __launch_bounds__(kT) k_deposit(DepositArgs a, int per) {
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t L = warp; L < a.nleaf; L += nw) {
+    for (int64_t L0 = warp * per; L0 < a.nleaf; L0 += nw * per) {
+        const int m = (int)min((int64_t)per, a.nleaf - L0);
+        const int64_t L = L0 + lane;
         double total = 0.0, chi = 0.0;
         for (int s = 0; s < a.nsp; ++s) {
-            const int32_t p0 = a.start[s][L], p1 = a.end[s][L];
+            const int32_t f = lane < m ? a.start[s][L] : 0, e = lane < m ? a.end[s][L] : 0;
             const R *w = (const R *)a.w[s];
-            R sum = 0, c = 0;
-            for (int32_t p = p0 + lane; p < p1; p += 128) {
-                R x4[4];
+            R my_hi = 0, my_lo = 0;
+            for (int i = 0; i < m; ++i) {
+                const int32_t p0 = __shfl_sync(0xFFFFFFFFu, f, i), p1 = __shfl_sync(0xFFFFFFFFu, e, i);
+                R sum = 0, c = 0;
+                for (int32_t p = p0 + lane; p < p1; p += 128) {
+                    R x4[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) x4[k] = p + 32 * k < p1 ? w[p + 32 * k] : (R)0;
+                    for (int k = 0; k < 4; ++k) x4[k] = p + 32 * k < p1 ? w[p + 32 * k] : (R)0;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) kahan_add(sum, c, x4[k]);
+                    for (int k = 0; k < 4; ++k) kahan_add(sum, c, x4[k]);
+                }
+                R hi = sum, lo = -c;
+                warp_two_sum(hi, lo);
+                if (lane == i) {
+                    my_hi = hi;
+                    my_lo = lo;
+                }
             }
-            R hi = sum, lo = -c;
-            warp_two_sum(hi, lo);
-            const double Ws = (double)hi + (double)lo;
+            const double Ws = (double)my_hi + (double)my_lo;
             total += a.q[s] * Ws;
             chi += a.chi[s] * Ws;
         }
-        if (lane == 0) {
+        if (lane < m) {
             const double h = (double)(1 << (a.lmax - a.lev[L])) * a.hf;
             if (a.kappa) a.kappa[L] = 1.0 + chi / (h * h);
             a.charge[L] = total;
@@ -1783,10 +1798,13 @@ void deposit(pic_ctx *ctx, Instance &in, const double walls[4]) {
         else
             pdl(k_deposit_sums<float>, blocks_for(in.nleaf), kT, 0, ctx->stream, a, w0, w1);
     }
-    else if (in.cfg.precision == PIC_FP64)
-        k_deposit<double><<<warp_blocks(in.nleaf), kT, 0, ctx->stream>>>(a);
-    else
-        k_deposit<float><<<warp_blocks(in.nleaf), kT, 0, ctx->stream>>>(a);
+    else {
+        // leaves per warp: as many as still leave 48 warps per SM
+        const int per = (int)std::max<int64_t>(1, std::min<int64_t>(32, in.nleaf / (152 * 48)));
+        const unsigned nb = warp_blocks((in.nleaf + per - 1) / per);
+        if (in.cfg.precision == PIC_FP64) k_deposit<double><<<nb, kT, 0, ctx->stream>>>(a, per);
+        else k_deposit<float><<<nb, kT, 0, ctx->stream>>>(a, per);
+    }
     count_launch(ctx);
     check_launch("deposit");
     if (in.cfg.implicit) poisson_kappa(ctx, in, walls);  // the operator with this step's susceptibility
