@@ -376,15 +376,17 @@ pic_status pic_create(const pic_config *cfg, int32_t n_instances, pic_ctx **out)
             in.part_mem[0].cache = &ctx->cache;
             in.part_mem[1].cache = &ctx->cache;
             GB_CUDA(cudaMallocHost(&in.red_host, 64));
-            GB_CUDA(cudaMallocHost(&in.cnt_host, 64));
+            GB_CUDA(cudaMallocHost(&in.cnt_host, 128));
+            std::memset(in.cnt_host, 0, 128);
+            in.pub = reinterpret_cast<unsigned long long *>(in.cnt_host + 16);
             GB_CUDA(cudaMalloc(&in.d_next_id, 16));
             GB_CUDA(cudaMemset(in.d_next_id, 0, 16));
             GB_CUDA(cudaMalloc(&in.d_err, 4));
             GB_CUDA(cudaMemset(in.d_err, 0, 4));
         }
         // device step counter and wall potentials (read by captured ensemble steps)
-        GB_CUDA(cudaMalloc(&ctx->d_step, 8));
-        GB_CUDA(cudaMemset(ctx->d_step, 0, 8));
+        GB_CUDA(cudaMalloc(&ctx->d_step, 16));
+        GB_CUDA(cudaMemset(ctx->d_step, 0, 16));
         GB_CUDA(cudaMalloc(&ctx->d_walls, 4 * 8 * (size_t)n_instances));
         for (int i = 0; i < n_instances; ++i) ctx->inst[i].d_walls = ctx->d_walls + 4 * i;
         ctx->precision = cfg[0].precision;
@@ -516,6 +518,7 @@ pic_status pic_step(pic_ctx *ctx, int32_t n_steps) {
             if (!in.has_mesh) fail(PIC_EINVAL, "mesh not set");
             ensure_species(ctx, in);
             reset_solver_stats(ctx, in);
+            in.pub_tag = 0;
         }
         for (int32_t k = 0; k < n_steps; ++k) one_step(ctx);
         return end_of_steps(ctx);
@@ -532,6 +535,7 @@ pic_status pic_autotune(pic_ctx *ctx, int32_t max_steps, int32_t *steps_used) {
             if (!in.has_mesh) fail(PIC_EINVAL, "mesh not set");
             ensure_species(ctx, in);
             reset_solver_stats(ctx, in);
+            in.pub_tag = 0;
         }
         int32_t used = 0;
         // an ensemble reaches the state in which its steps replay as one graph after a step

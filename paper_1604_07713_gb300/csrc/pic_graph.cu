@@ -218,6 +218,7 @@ void graph_prepare(pic_ctx *ctx) {
 void one_step(pic_ctx *ctx) {
     for (Instance &in : ctx->inst) in.counts_exact = false;
     for (Instance &in : ctx->inst) ensure_capacity(ctx, in);
+    if (++ctx->step_tag == 0) ++ctx->step_tag;
     if (graph_step_possible(ctx)) {
         graph_step(ctx);  // an ensemble in steady state: the whole step as one graph replay
     } else {
@@ -230,6 +231,7 @@ void one_step(pic_ctx *ctx) {
             particle_step(ctx, in, ctx->step, true, in.cfg.implicit ? PUSH_CORRECT : PUSH_LEAPFROG);
         }
     }
+    for (Instance &in : ctx->inst) in.pub_tag = in.cfg.mcc && in.cfg.sigma_iz0 > 0.0 ? ctx->step_tag : 0;
     ++ctx->step;
 }
 
@@ -252,9 +254,9 @@ void graph_step(pic_ctx *ctx) {
     const int n = (int)ctx->inst.size();
     std::vector<double> walls(4 * (size_t)n);
     for (int i = 0; i < n; ++i) walls_at(ctx->inst[i], ctx->step, walls.data() + 4 * i);
-    const int64_t step = ctx->step;
+    const int64_t step[2] = {ctx->step, (int64_t)ctx->step_tag};
     GB_CUDA(cudaMemcpyAsync(ctx->d_walls, walls.data(), walls.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
-    GB_CUDA(cudaMemcpyAsync(ctx->d_step, &step, 8, cudaMemcpyHostToDevice, ctx->stream));
+    GB_CUDA(cudaMemcpyAsync(ctx->d_step, step, 16, cudaMemcpyHostToDevice, ctx->stream));
     {
         Phase ph(ctx, PIC_PHASE_GRAPH);
         GB_CUDA(cudaGraphLaunch(ctx->step_graph, ctx->stream));
@@ -364,6 +366,7 @@ void report_all(pic_ctx *ctx) {
         Instance &in = ctx->inst[i];
         for (int s = 0; s < in.cfg.n_species; ++s) in.sp[s].n = in.sp[s].n_upper = r[i].tot[s];
         in.counts_exact = true;
+        in.pub_tag = 0;
         in.report_err = r[i].err;
         if (in.mg_on_device && in.mg_stats) {
             in.mg_cycles = (int)r[i].mg[0];

@@ -203,6 +203,8 @@ struct Instance {
     double *red = nullptr;       // reduction scratch
     double *red_host = nullptr;  // pinned
     int32_t *cnt_host = nullptr; // pinned
+    unsigned long long *pub = nullptr;  // pinned, per species: (step tag << 32) | the step's upper count
+    uint32_t pub_tag = 0;        // the tag of the last step issued in this call (0: none)
     void *stencil = nullptr;     // node E per leaf corner: 8 x R per leaf
     void *patch = nullptr;       // cloud-in-cell shapes: per leaf 4 quarters x 2 components x 4 R
     double *cic_part = nullptr;  // cloud-in-cell deposit: per leaf its charge on the 3 x 3 cells around it
@@ -301,7 +303,8 @@ struct pic_ctx {
     gbpic::BlockCache cache;  // device blocks released by this context, for reuse
     // captured multi-instance step (pic_graph.cu)
     bool capturing = false;          // launches are being captured: read step and walls on the device
-    int64_t *d_step = nullptr;       // device copy of the step number
+    int64_t *d_step = nullptr;       // device copy of the step number and of step_tag
+    uint32_t step_tag = 0;           // counts the steps issued; tags what a step publishes to the host
     double *d_walls = nullptr;       // per instance: the 4 wall potentials of the current step
     int64_t lists_epoch = 0;         // bumped whenever list buffers or per-leaf arrays are re-allocated
     cudaGraphExec_t step_graph = nullptr;
