@@ -376,8 +376,9 @@ pic_status pic_create(const pic_config *cfg, int32_t n_instances, pic_ctx **out)
             in.part_mem[0].cache = &ctx->cache;
             in.part_mem[1].cache = &ctx->cache;
             GB_CUDA(cudaMallocHost(&in.red_host, 64));
-            GB_CUDA(cudaMallocHost(&in.cnt_host, 128));
-            std::memset(in.cnt_host, 0, 128);
+            GB_CUDA(cudaMallocHost(&in.cnt_host, 256));
+            std::memset(in.cnt_host, 0, 256);
+            in.dec_host = in.cnt_host + 32;
             in.pub = reinterpret_cast<unsigned long long *>(in.cnt_host + 16);
             GB_CUDA(cudaMalloc(&in.d_next_id, 16));
             GB_CUDA(cudaMemset(in.d_next_id, 0, 16));

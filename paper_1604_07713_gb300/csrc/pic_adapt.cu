@@ -588,11 +588,12 @@ __global__ void k_compact_flags(int64_t n, const int32_t *__restrict__ flag, con
     if (l < n && flag[l]) list[pos[l]] = (int32_t)l;
 }
 
-int32_t read_i32(pic_ctx *ctx, const int32_t *d) {
-    int32_t h = 0;
-    GB_CUDA(cudaMemcpyAsync(&h, d, 4, cudaMemcpyDeviceToHost, ctx->stream));
-    GB_CUDA(cudaStreamSynchronize(ctx->stream));
-    return h;
+// Device words the host decides on: copied to pinned memory (word w of the instance's), read
+// after one synchronisation for all of them.  An adaptation waited for each word and species in
+// turn, ~30 copies to pageable memory (streamer of 2e5 particles: mesh 0.94 -> 0.80 ms,
+// particles 0.37 -> 0.26 ms).
+void fetch_words(pic_ctx *ctx, Instance &in, int w, const void *d, int n = 1) {
+    GB_CUDA(cudaMemcpyAsync(in.dec_host + w, d, 4 * (size_t)n, cudaMemcpyDeviceToHost, ctx->stream));
 }
 
 // Re-allocate one species' per-leaf arrays for a new leaf count; the records stay.  With
@@ -610,14 +611,12 @@ void species_relist(pic_ctx *ctx, Instance &in, int s, int64_t nl, const int32_t
     } else {
         lists_installed(ctx, sp, nl);
     }
-    GB_CUDA(cudaStreamSynchronize(ctx->stream));
 }
 
-// Lists whose tail has used up more than a quarter of the buffer are laid out again first,
-// so that repairs and adaptation do not keep growing the buffers.
-void compact_if_crowded(pic_ctx *ctx, Instance &in, int s) {
+// Lists whose tail (fetched) has used up more than a quarter of the buffer are laid out again
+// first, so that repairs and adaptation do not keep growing the buffers.
+void compact_if_crowded(pic_ctx *ctx, Instance &in, int s, int32_t tail) {
     Species &sp = in.sp[s];
-    const int32_t tail = read_i32(ctx, sp.flags + 4);
     if ((int64_t)tail > sp.cap - sp.cap / 4) species_compact(ctx, in, s);
 }
 
@@ -625,11 +624,12 @@ template <typename R> void adapt_particles(pic_ctx *ctx, Instance &in, int64_t n
                                            const int32_t *kind, const int32_t *group, const int32_t *new_of,
                                            const uint32_t *morton_old, DeviceArena &T) {
     cudaStream_t st = ctx->stream;
+    int32_t *ncnt2[2], *need2[2];
+    for (int s = 0; s < in.cfg.n_species; ++s) compact_if_crowded(ctx, in, s, in.dec_host[s]);
     for (int s = 0; s < in.cfg.n_species; ++s) {
         Species &sp = in.sp[s];
-        compact_if_crowded(ctx, in, s);
-        int32_t *ncnt = dalloc<int32_t>(T, n_new + 1);
-        int32_t *need = dalloc<int32_t>(T, n_old + 1);
+        int32_t *ncnt = ncnt2[s] = dalloc<int32_t>(T, n_new + 1);
+        int32_t *need = need2[s] = dalloc<int32_t>(T, n_old + 1);
         int32_t *scr = dalloc<int32_t>(T, scan_scratch_elems(std::max(n_old, n_new)));
         GB_CUDA(cudaMemsetAsync(ncnt, 0, (n_new + 1) * 4, st));
         k_adapt_count<R><<<warp_blocks(n_old), kT, 0, st>>>(n_old, sp.start, sp.end, kind, group, new_of,
@@ -637,11 +637,15 @@ template <typename R> void adapt_particles(pic_ctx *ctx, Instance &in, int64_t n
         k_adapt_tail_need<<<blocks_for(n_old), kT, 0, st>>>(n_old, sp.start, sp.end, kind, group, need);
         count_launch(ctx, 2);
         exclusive_scan_i32(ctx, need, need, n_old, scr);
+        fetch_words(ctx, in, 2 * s, sp.flags + 4);
+        fetch_words(ctx, in, 2 * s + 1, need + n_old);
+    }
+    GB_CUDA(cudaStreamSynchronize(st));
+    for (int s = 0; s < in.cfg.n_species; ++s) {
+        Species &sp = in.sp[s];
+        const int32_t *ncnt = ncnt2[s], *need = need2[s];
+        const int32_t h[2] = {in.dec_host[2 * s], in.dec_host[2 * s + 1]};
         // the coarsened quartets' lists go to the tail: make room for them first
-        int32_t h[2] = {0, 0};
-        GB_CUDA(cudaMemcpyAsync(&h[0], sp.flags + 4, 4, cudaMemcpyDeviceToHost, st));
-        GB_CUDA(cudaMemcpyAsync(&h[1], need + n_old, 4, cudaMemcpyDeviceToHost, st));
-        GB_CUDA(cudaStreamSynchronize(st));
         ensure_slots(ctx, in, s, (int64_t)h[0] + h[1]);
         int32_t *nstart = dalloc<int32_t>(T, n_new + 1), *nend = dalloc<int32_t>(T, n_new + 1);
         int32_t *nlim = dalloc<int32_t>(T, n_new + 1);
@@ -659,14 +663,19 @@ template <typename R> void split_merge_impl(pic_ctx *ctx, Instance &in) {
     cudaStream_t st = ctx->stream;
     const int64_t nl = in.nleaf;
     DeviceArena T(&ctx->cache);
-    unsigned long long next_id = 0;
-    GB_CUDA(cudaMemcpyAsync(&next_id, in.d_next_id, 8, cudaMemcpyDeviceToHost, st));
-    GB_CUDA(cudaStreamSynchronize(st));
     int32_t *err = dalloc<int32_t>(T, 1);
     GB_CUDA(cudaMemsetAsync(err, 0, 4, st));
+    for (int s = 0; s < in.cfg.n_species; ++s) fetch_words(ctx, in, s, in.sp[s].flags + 4);
+    fetch_words(ctx, in, 2, in.d_next_id, 2);
+    GB_CUDA(cudaStreamSynchronize(st));
+    unsigned long long next_id = 0;
+    std::memcpy(&next_id, in.dec_host + 2, 8);
+    struct Plan {
+        int32_t *tneed, *toff, *idb, *mflag, *mpos, *mlist, *sflag, *spos, *slist;
+    } plan[2];
+    for (int s = 0; s < in.cfg.n_species; ++s) compact_if_crowded(ctx, in, s, in.dec_host[s]);
     for (int s = 0; s < in.cfg.n_species; ++s) {
         Species &sp = in.sp[s];
-        compact_if_crowded(ctx, in, s);
         int32_t *ncnt = dalloc<int32_t>(T, nl + 1), *nids = dalloc<int32_t>(T, nl + 1);
         int32_t *mflag = dalloc<int32_t>(T, nl + 1), *sflag = dalloc<int32_t>(T, nl + 1);
         int32_t *tneed = dalloc<int32_t>(T, nl + 1), *toff = dalloc<int32_t>(T, nl + 1);
@@ -683,13 +692,20 @@ template <typename R> void split_merge_impl(pic_ctx *ctx, Instance &in) {
         exclusive_scan_i32(ctx, mflag, mpos, nl, scr);
         exclusive_scan_i32(ctx, sflag, spos, nl, scr);
         exclusive_scan_i32(ctx, tneed, toff, nl, scr);
-        int32_t tot[5];
-        GB_CUDA(cudaMemcpyAsync(&tot[0], toff + nl, 4, cudaMemcpyDeviceToHost, st));
-        GB_CUDA(cudaMemcpyAsync(&tot[1], idb + nl, 4, cudaMemcpyDeviceToHost, st));
-        GB_CUDA(cudaMemcpyAsync(&tot[2], mpos + nl, 4, cudaMemcpyDeviceToHost, st));
-        GB_CUDA(cudaMemcpyAsync(&tot[3], spos + nl, 4, cudaMemcpyDeviceToHost, st));
-        GB_CUDA(cudaMemcpyAsync(&tot[4], sp.flags + 4, 4, cudaMemcpyDeviceToHost, st));
-        GB_CUDA(cudaStreamSynchronize(st));
+        fetch_words(ctx, in, 5 * s, toff + nl);
+        fetch_words(ctx, in, 5 * s + 1, idb + nl);
+        fetch_words(ctx, in, 5 * s + 2, mpos + nl);
+        fetch_words(ctx, in, 5 * s + 3, spos + nl);
+        fetch_words(ctx, in, 5 * s + 4, sp.flags + 4);
+        plan[s] = Plan{tneed, toff, idb, mflag, mpos, mlist, sflag, spos, slist};
+    }
+    GB_CUDA(cudaStreamSynchronize(st));
+    int32_t totals[2][5];
+    std::memcpy(totals, in.dec_host, sizeof totals);
+    for (int s = 0; s < in.cfg.n_species; ++s) {
+        Species &sp = in.sp[s];
+        const int32_t *tot = totals[s];
+        const auto [tneed, toff, idb, mflag, mpos, mlist, sflag, spos, slist] = plan[s];
         if (in.cfg.particle_capacity > 0 && sp.n_upper + tot[1] > in.cfg.particle_capacity)
             fail(PIC_ECAPACITY, "split would exceed the particle capacity");
         // split leaves whose segment is too small go to the tail: make room first (may move
@@ -715,7 +731,9 @@ template <typename R> void split_merge_impl(pic_ctx *ctx, Instance &in) {
         check_launch("split_merge");
         const int32_t tail = tot[4] + tot[0];  // the split leaves moved to the tail took up to here
         GB_CUDA(cudaMemcpyAsync(sp.flags + 4, &tail, 4, cudaMemcpyHostToDevice, st));
-        if (read_i32(ctx, err)) fail(PIC_EINVAL, "a leaf holds more particles than one merge block sorts (12288)");
+        fetch_words(ctx, in, 0, err);
+        GB_CUDA(cudaStreamSynchronize(st));
+        if (in.dec_host[0]) fail(PIC_EINVAL, "a leaf holds more particles than one merge block sorts (12288)");
         next_id += (unsigned long long)tot[1];
         sp.sums_valid = false;
     }
@@ -759,21 +777,27 @@ void adapt_mesh(pic_ctx *ctx, Instance &in) {
                                                       in.cfg.bc_x == PIC_BC_PERIODIC, in.cfg.bc_y == PIC_BC_PERIODIC,
                                                       g.ix, g.iy, g.lev, refine, group, gactive, changed);
         count_launch(ctx);
-        if (!read_i32(ctx, changed)) break;
+        fetch_words(ctx, in, 0, changed);
+        GB_CUDA(cudaStreamSynchronize(st));
+        if (!in.dec_host[0]) break;
         if (it == max_sweeps - 1)
             fail(PIC_ETIMEOUT, "2:1 balance closure did not settle in " + std::to_string(max_sweeps) + " sweeps");
     }
-    int32_t *cnt = dalloc<int32_t>(T, n + 1), *pos = dalloc<int32_t>(T, n + 1);
+    int32_t *cnt = dalloc<int32_t>(T, n + 1), *pos = dalloc<int32_t>(T, n + 2);
     int32_t *scr = dalloc<int32_t>(T, scan_scratch_elems(n));
     k_adapt_emit_count<<<blocks_for(n), kT, 0, st>>>(n, refine, group, gactive, cnt);
     count_launch(ctx);
     exclusive_scan_i32(ctx, cnt, pos, n, scr);
-    int32_t *grid_changed = dalloc<int32_t>(T, 1);
+    int32_t *grid_changed = pos + n + 1;
     GB_CUDA(cudaMemsetAsync(grid_changed, 0, 4, st));
     k_adapt_changed<<<blocks_for(n), kT, 0, st>>>(n, cnt, grid_changed);
     count_launch(ctx);
-    const bool grid_did_change = read_i32(ctx, grid_changed) != 0;
-    const int64_t n_new = read_i32(ctx, pos + n);
+    // (and the lists' tails, for adapt_particles)
+    for (int s = 0; s < in.cfg.n_species; ++s) fetch_words(ctx, in, s, in.sp[s].flags + 4);
+    fetch_words(ctx, in, 2, pos + n, 2);
+    GB_CUDA(cudaStreamSynchronize(st));
+    const bool grid_did_change = in.dec_host[3] != 0;
+    const int64_t n_new = in.dec_host[2];
     uint32_t *nroot = dalloc<uint32_t>(T, n_new), *nmort = dalloc<uint32_t>(T, n_new);
     uint8_t *nlev = dalloc<uint8_t>(T, n_new);
     double *nphi = dalloc<double>(T, n_new);

@@ -203,6 +203,7 @@ struct Instance {
     double *red = nullptr;       // reduction scratch
     double *red_host = nullptr;  // pinned
     int32_t *cnt_host = nullptr; // pinned
+    int32_t *dec_host = nullptr;        // pinned: the words an adaptation decides on
     unsigned long long *pub = nullptr;  // pinned, per species: (step tag << 32) | the step's upper count
     uint32_t pub_tag = 0;        // the tag of the last step issued in this call (0: none)
     void *stencil = nullptr;     // node E per leaf corner: 8 x R per leaf

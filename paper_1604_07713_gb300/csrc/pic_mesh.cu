@@ -396,11 +396,22 @@ __global__ void k_cell_emag(int64_t n, FieldView<double> F, double *__restrict__
     out[l] = sqrt(ex * ex + ey * ey);
 }
 
-int32_t read_err(pic_ctx *ctx, int32_t *d_err) {
-    int32_t h = 0;
-    GB_CUDA(cudaMemcpyAsync(&h, d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
+int32_t read_err(pic_ctx *ctx, Instance &in, int32_t *d_err) {
+    GB_CUDA(cudaMemcpyAsync(in.dec_host, d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
     GB_CUDA(cudaStreamSynchronize(ctx->stream));
-    return h;
+    return in.dec_host[0];
+}
+
+// cnt[c] += cells of the tree level of depth c: a cell holds exactly one leaf at its lower left
+// corner, so a leaf counts at every depth whose lattice its corner lies on.
+__global__ void k_level_counts(int64_t n, const int32_t *__restrict__ ix, const int32_t *__restrict__ iy, int lmax,
+                               int32_t *__restrict__ cnt) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int32_t at = i < n ? ix[i] | iy[i] : -1;
+    for (int c = 0; c < lmax; ++c) {
+        const int m = __syncthreads_count(i < n && (at & ((1 << (lmax - c)) - 1)) == 0);
+        if (threadIdx.x == 0 && m) atomicAdd(cnt + c, m);
+    }
 }
 
 LatView view_of(const Instance &in, const Level &g) {
@@ -509,8 +520,8 @@ void mesh_build_device(pic_ctx *ctx, Instance &in, int64_t n) {
     const uint64_t nkeys64 = (uint64_t)nx0 * ny0 << (2 * lmax);
     if (nkeys64 >= (1ull << 31)) fail(PIC_EINVAL, "lattice too large (nx0*ny0*4^max_level >= 2^31)");
     const uint32_t nkeys = (uint32_t)nkeys64;
-    int32_t *d_err = dalloc<int32_t>(A, 1);
-    GB_CUDA(cudaMemsetAsync(d_err, 0, 4, ctx->stream));
+    int32_t *d_err = dalloc<int32_t>(A, 1 + kMaxLevel);  // the flag, then the tree levels' cell counts
+    GB_CUDA(cudaMemsetAsync(d_err, 0, (1 + kMaxLevel) * 4, ctx->stream));
     uint32_t *raw_key = dalloc<uint32_t>(A, n);
     const uint32_t *raw_root = in.root, *raw_mort = in.morton;
     const uint8_t *raw_lev = in.lv[0].lev;
@@ -532,7 +543,7 @@ void mesh_build_device(pic_ctx *ctx, Instance &in, int64_t n) {
                                                                lmax, in.key, root, mort, g.lev, g.ix, g.iy);
     k_check_tiling<<<blocks_for(n), kT, 0, ctx->stream>>>(n, in.key, g.lev, lmax, nkeys64, d_err);
     count_launch(ctx, 2);
-    int32_t e = read_err(ctx, d_err);
+    int32_t e = read_err(ctx, in, d_err);
     if (e) fail(PIC_EINVAL, "leaf set is not a tiling of the root boxes (code " + std::to_string(e) + ")");
     A.release(raw_key);
     A.release(slot);
@@ -543,8 +554,13 @@ void mesh_build_device(pic_ctx *ctx, Instance &in, int64_t n) {
     in.lv.clear();
     in.lv.push_back(g);
     k_check_balance<<<blocks_for(n), kT, 0, ctx->stream>>>(n, view_of(in, in.lv[0]), d_err);
-    count_launch(ctx);
-    e = read_err(ctx, d_err);
+    k_level_counts<<<blocks_for(n), kT, 0, ctx->stream>>>(n, g.ix, g.iy, lmax, d_err + 1);
+    count_launch(ctx, 2);
+    GB_CUDA(cudaMemcpyAsync(in.dec_host, d_err, (1 + kMaxLevel) * 4, cudaMemcpyDeviceToHost, ctx->stream));
+    GB_CUDA(cudaStreamSynchronize(ctx->stream));
+    e = in.dec_host[0];
+    int32_t level_cells[kMaxLevel];
+    std::copy_n(in.dec_host + 1, kMaxLevel, level_cells);
     if (e) fail(PIC_EINVAL, "leaf set is not 2:1 balanced across faces");
     assemble_level(ctx, in, in.lv[0], true, d_err);
     // coarser levels
@@ -557,9 +573,7 @@ void mesh_build_device(pic_ctx *ctx, Instance &in, int64_t n) {
             k_clamp_flags<<<blocks_for(f.n), kT, 0, ctx->stream>>>(f.n, f.ix, f.iy, f.lev, f.lmax, keep);
             count_launch(ctx);
             exclusive_scan_i32(ctx, keep, keep, f.n, sc);
-            int32_t nc = 0;
-            GB_CUDA(cudaMemcpyAsync(&nc, keep + f.n, 4, cudaMemcpyDeviceToHost, ctx->stream));
-            GB_CUDA(cudaStreamSynchronize(ctx->stream));
+            const int32_t nc = level_cells[f.lmax - 1];
             c.nx0 = f.nx0; c.ny0 = f.ny0; c.lmax = f.lmax - 1; c.h0 = f.h0; c.n = nc;
             c.ix = dalloc<int32_t>(A, nc); c.iy = dalloc<int32_t>(A, nc); c.lev = dalloc<uint8_t>(A, nc);
             f.parent = dalloc<int32_t>(A, f.n);
@@ -585,7 +599,7 @@ void mesh_build_device(pic_ctx *ctx, Instance &in, int64_t n) {
         fill_map(ctx, in, cc);
         assemble_level(ctx, in, cc, false, d_err);
     }
-    e = read_err(ctx, d_err);
+    e = read_err(ctx, in, d_err);
     if (e) fail(PIC_EINVAL, "multigrid level construction failed (code " + std::to_string(e) + ")");
     check_launch("mesh_build");
     in.has_mesh = true;
