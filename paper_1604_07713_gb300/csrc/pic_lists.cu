@@ -169,11 +169,36 @@ __device__ __forceinline__ void copy_record(SoA<R> t, int64_t q, SoA<R> d, int64
     t.w[q] = d.w[p]; t.id[q] = d.id[p];
 }
 
-// Repair 1 (one warp per leaf that ran out of free slots): a segment at the tail with room
-// for its staying and entering records and free slots, the staying records and the entering
-// records already in free slots copied there.  A leaf that does not fit any more marks the
-// tail as used up (flags[5]) and keeps its segment; the re-layout then takes over.
-// The warp takes the moved leaves warp, warp + nw, ...
+// Repair 1: each leaf that ran out of free slots gets a segment at the tail with room for its
+// staying and entering records and free slots, the staying records and the entering records
+// already in free slots copied there.  A leaf that does not fit any more marks the tail as used
+// up (flags[5]) and keeps its segment; the re-layout then takes over.
+// The leaf's words, and its copies by `nt` threads of which this is `t`.
+struct TailMove {
+    int32_t L, ns, need, base, s0, e0, room;
+    __device__ __forceinline__ TailMove(int32_t leaf, const int32_t *start, const int32_t *end, const int32_t *lim,
+                                        const int32_t *stay, const int32_t *fill)
+        : L(leaf), ns(stay[leaf]), base(0), s0(start[leaf]), e0(end[leaf]), room(lim[leaf] - end[leaf]) {
+        const int32_t f = fill[leaf], c = ns + f;
+        need = c + list_slack(c) + f;
+    }
+    template <typename R>
+    __device__ __forceinline__ void copy(SoA<R> d, uint32_t *__restrict__ key, uint32_t *__restrict__ aux, int t, int nt) const {
+        for (int32_t j = t; j < ns; j += nt) copy_record(d, base + j, d, s0 + j);
+        for (int32_t j = t; j < room; j += nt) {
+            copy_record(d, base + ns + j, d, e0 + j);
+            key[base + ns + j] = key[e0 + j];
+            aux[base + ns + j] = aux[e0 + j];
+        }
+    }
+    __device__ __forceinline__ void install(int32_t *__restrict__ start, int32_t *__restrict__ end,
+                                            int32_t *__restrict__ lim) const {
+        start[L] = base;
+        end[L] = base + ns;
+        lim[L] = base + need;
+    }
+};
+// A warp per leaf: the moved leaves warp, warp + nw, ...
 template <typename R>
 __device__ __forceinline__ void move_to_tail(const int32_t *__restrict__ moved, int64_t nl, int64_t cap,
                                              int32_t *__restrict__ start, int32_t *__restrict__ end,
@@ -185,29 +210,16 @@ __device__ __forceinline__ void move_to_tail(const int32_t *__restrict__ moved, 
     const int lane = threadIdx.x & 31;
     const int32_t nm = moved[nl];
     for (int64_t i = warp; i < nm; i += nw) {
-        const int32_t L = moved[i];
-        const int32_t ns = stay[L], f = fill[L], c = ns + f;
-        const int32_t need = c + list_slack(c) + f;
-        int32_t base = 0;
-        if (lane == 0) base = atomicAdd(flags + 4, need);
-        base = __shfl_sync(0xFFFFFFFFu, base, 0);
-        if ((int64_t)base + need > cap) {
+        TailMove m(moved[i], start, end, lim, stay, fill);
+        if (lane == 0) m.base = atomicAdd(flags + 4, m.need);
+        m.base = __shfl_sync(0xFFFFFFFFu, m.base, 0);
+        if ((int64_t)m.base + m.need > cap) {
             if (lane == 0) flags[5] = 1;
             continue;
         }
-        const int32_t s0 = start[L], e0 = end[L], room = lim[L] - e0;
-        for (int32_t j = lane; j < ns; j += 32) copy_record(d, base + j, d, s0 + j);
-        for (int32_t j = lane; j < room; j += 32) {
-            copy_record(d, base + ns + j, d, e0 + j);
-            key[base + ns + j] = key[e0 + j];
-            aux[base + ns + j] = aux[e0 + j];
-        }
+        m.copy(d, key, aux, lane, 32);
         __syncwarp();
-        if (lane == 0) {
-            start[L] = base;
-            end[L] = base + ns;
-            lim[L] = base + need;
-        }
+        if (lane == 0) m.install(start, end, lim);
     }
 }
 
@@ -421,11 +433,37 @@ ListEntry list_entry(Instance &in, int s) {
     return e;
 }
 
+// Repair 1 by the grid's x blocks.  Few leaves (the usual step): a block for each, so that its
+// copies are one round of loads and not one per 32 records (512 x 16 discharge, some 20 leaves a
+// step: repairs and spawn scan 0.0255 -> 0.0188 ms, FP64 0.0331 -> 0.0229); more leaves than
+// blocks: a warp for each.
+template <typename R> __device__ __forceinline__ void tail_moves(const ListEntry &e) {
+    if (e.flags[0] == 0) return;
+    const int32_t nm = e.moved[e.nl];
+    if (nm > (int32_t)gridDim.x) {
+        move_to_tail<R>(e.moved, e.nl, e.cap, e.start, e.end, e.lim, e.stay, e.fill, soa_of<R>(e.d), e.key, e.aux,
+                        e.flags, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                        ((int64_t)gridDim.x * blockDim.x) >> 5);
+    } else if ((int32_t)blockIdx.x < nm) {
+        __shared__ int32_t at;
+        TailMove m(e.moved[blockIdx.x], e.start, e.end, e.lim, e.stay, e.fill);
+        if (threadIdx.x == 0) at = atomicAdd(e.flags + 4, m.need);
+        __syncthreads();  // (every thread has read the leaf's words)
+        m.base = at;
+        if ((int64_t)m.base + m.need > e.cap) {
+            if (threadIdx.x == 0) e.flags[5] = 1;
+            return;
+        }
+        m.copy(soa_of<R>(e.d), e.key, e.aux, threadIdx.x, kT);
+        if (threadIdx.x == 0) m.install(e.start, e.end, e.lim);
+    }
+}
+
 // After a push, the spawn offsets and the repairs of both species in three launches (they were
 // three scan launches and, per species, a graph of two conditional nodes, ~25 us each): the
 // spawn scan's tile totals beside the tail moves, the scan itself beside the placement of the
 // overflow store, and the re-layout, whose blocks return at once unless a tail was used up.
-// 512 x 16 discharge: 0.076 -> 0.027 ms per step.
+// 512 x 16 discharge: 0.076 -> 0.019 ms per step.
 struct RepairArgs {
     ListEntry e[2];
     int nsp;
@@ -440,10 +478,7 @@ struct RepairArgs {
 template <typename R> __global__ void __launch_bounds__(kT) k_step_move(const __grid_constant__ RepairArgs A) {
     pdl_chain();
     if ((int)blockIdx.y < A.nsp) {
-        const ListEntry &e = A.e[blockIdx.y];
-        move_to_tail<R>(e.moved, e.nl, e.cap, e.start, e.end, e.lim, e.stay, e.fill, soa_of<R>(e.d), e.key, e.aux,
-                        e.flags, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5,
-                        ((int64_t)gridDim.x * blockDim.x) >> 5);
+        tail_moves<R>(A.e[blockIdx.y]);
         return;
     }
     if ((int)blockIdx.x >= A.tiles) return;
@@ -602,7 +637,7 @@ __global__ void k_compact_done(int32_t *__restrict__ flags) {
 }
 
 // ---- the batched ensemble step: one entry per (instance, species) ------------------------
-// Before the pushes, per entry: what k_step_reset clears, and the record counts whose scan
+// Before the pushes, per entry: what k_lists_sums clears, and the record counts whose scan
 // gives the list ranks (block = leaves [c.y, c.z) of entry c.x).
 __global__ void k_lists_prep_batch(const ListEntry *__restrict__ tab, const int4 *__restrict__ chunks) {
     const int4 c = chunks[blockIdx.x];
@@ -629,11 +664,8 @@ __global__ void k_any_flag(const ListEntry *__restrict__ tab, int n, int word, i
 }
 
 // Repair 1 of every entry (blocks (x, entry)); entries without overflow return at once.
-template <typename R> __global__ void k_move_to_tail_batch(const ListEntry *__restrict__ tab) {
-    const ListEntry &e = tab[blockIdx.y];
-    move_to_tail<R>(e.moved, e.nl, e.cap, e.start, e.end, e.lim, e.stay, e.fill, soa_of<R>(e.d), e.key, e.aux,
-                    e.flags, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5,
-                    ((int64_t)gridDim.x * blockDim.x) >> 5);
+template <typename R> __global__ void __launch_bounds__(kT) k_move_to_tail_batch(const ListEntry *__restrict__ tab) {
+    tail_moves<R>(tab[blockIdx.y]);
 }
 template <typename R> __global__ void k_place_ovf_batch(const ListEntry *__restrict__ tab) {
     const ListEntry &e = tab[blockIdx.y];
@@ -701,7 +733,7 @@ template <typename R> void repairs_batch_impl(pic_ctx *ctx) {
     k_any_flag<<<1, kT, 0, ctx->stream>>>(tab, t.n, 0, flag);
     count_launch(ctx);
     capture_if(ctx, ctx->stream, flag, [&]() {
-        k_move_to_tail_batch<R><<<dim3(8, (unsigned)t.n), kT, 0, ctx->stream>>>(tab);
+        k_move_to_tail_batch<R><<<dim3(32, (unsigned)t.n), kT, 0, ctx->stream>>>(tab);
         k_place_ovf_batch<R><<<dim3(8, (unsigned)t.n), kT, 0, ctx->stream>>>(tab);
         // a tail used up: those species' lists are laid out again
         k_any_flag<<<1, kT, 0, ctx->stream>>>(tab, t.n, 5, flag + 1);
@@ -890,7 +922,7 @@ void launch_ranks(pic_ctx *ctx, const RankArgs &A, int nsp) {
 void list_ranks(pic_ctx *ctx, Instance &in, int s) { launch_ranks(ctx, rank_args(in, s, s + 1, false, false), 1); }
 
 // Before a push: every species' list ranks and the step's counters cleared, in two launches
-// (they were five per species: 512 x 16 discharge 0.043 -> 0.011 ms per step).
+// (they were five per species: 512 x 16 discharge 0.043 -> 0.010 ms per step).
 void step_lists_prep(pic_ctx *ctx, Instance &in, bool ionize) {
     launch_ranks(ctx, rank_args(in, 0, in.cfg.n_species, true, ionize), in.cfg.n_species);
 }
