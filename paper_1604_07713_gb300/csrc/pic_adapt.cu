@@ -196,67 +196,6 @@ __global__ void k_adapt_count(int64_t n, const int32_t *__restrict__ start, cons
     }
 }
 
-// Move the records to the new lists; offsets re-expressed exactly in the new leaf.  A
-// coarsened quartet's list is its children's lists one after another in Morton order.
-template <typename R>
-__global__ void k_adapt_move(int64_t n, const int32_t *__restrict__ start, const int32_t *__restrict__ end,
-                             const int32_t *__restrict__ kind, const int32_t *__restrict__ group,
-                             const int32_t *__restrict__ new_of, const uint32_t *__restrict__ morton,
-                             const int32_t *__restrict__ nstart, SoA<R> s, SoA<R> d) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t l = warp; l < n; l += nw) {
-        const int k = kind[l];
-        const int32_t p0 = start[l], p1 = end[l];
-        int32_t q0 = 0;  // first slot of this leaf's records in the new list
-        if (k == 0) {
-            q0 = nstart[new_of[l]];
-        } else if (k == 2) {
-            const int32_t g = group[l];
-            q0 = nstart[new_of[l]];
-            for (int32_t i = g; i < (int32_t)l; ++i) q0 += end[i] - start[i];
-        }
-        int32_t run[4] = {0, 0, 0, 0};
-        for (int32_t c0 = p0; c0 < p1; c0 += 32) {
-            const int32_t p = c0 + lane;
-            const bool live = p < p1;
-            R u = 0, v = 0;
-            int32_t dst = -1;
-            int ch = -1;
-            if (live) {
-                u = s.u[p];
-                v = s.v[p];
-            }
-            if (k == 0) {
-                dst = q0 + (p - p0);
-            } else if (k == 2) {
-                const R cx = (R)(morton[l] & 1u), cy = (R)((morton[l] >> 1) & 1u);
-                dst = q0 + (p - p0);
-                u = (cx + u) * (R)0.5;
-                v = (cy + v) * (R)0.5;
-            } else {
-                ch = live ? (u >= (R)0.5 ? 1 : 0) + (v >= (R)0.5 ? 2 : 0) : -1;
-                int32_t rank = 0;
-                for (int c = 0; c < 4; ++c) {
-                    const uint32_t m = __ballot_sync(0xFFFFFFFFu, ch == c);
-                    if (ch == c) rank = run[c] + __popc(m & lanemask_lt());
-                    run[c] += __popc(m);
-                }
-                if (live) {
-                    dst = nstart[new_of[l] + ch] + rank;
-                    u = (R)2 * u - (R)(ch & 1);
-                    v = (R)2 * v - (R)(ch >> 1);
-                }
-            }
-            if (live) {
-                d.u[dst] = u; d.v[dst] = v;
-                d.vx[dst] = s.vx[p]; d.vy[dst] = s.vy[p]; d.vz[dst] = s.vz[p]; d.w[dst] = s.w[p]; d.id[dst] = s.id[p];
-            }
-        }
-    }
-}
-
 // Slots a coarsened quartet's list takes at the tail (its first sibling only; 0 elsewhere).
 __global__ void k_adapt_tail_need(int64_t n, const int32_t *__restrict__ start, const int32_t *__restrict__ end,
                                   const int32_t *__restrict__ kind, const int32_t *__restrict__ group,
