@@ -937,7 +937,8 @@ __device__ void sm_build_inverse(const SmallLevel &L, float *M, bool singular, f
 // What bounds the solve is this serial chain of half sweeps; with four cells per thread the
 // finest level's is bound by shared-memory words.  512 x 16 cells, 4 cycles: 0.283 ms when each
 // cell's index division and wall tests were done in every half sweep and two barriers ended it,
-// 0.118 ms with the neighbour offsets formed once per leg (4 K loads), 0.105 ms so.
+// 0.118 ms with the neighbour offsets formed once per leg (4 K loads), 0.105 ms so, and 0.100 ms
+// with the decision and the coarsest solve as they are now.
 template <int K, int S> struct RbStrips {
     int j[S];            // position of the first row
     int l[S], sl[S];     // word left of it and the step to the next row's (0: missing)
@@ -1639,8 +1640,9 @@ template <bool CODED> void level_cycle(pic_ctx *ctx, Instance &in, size_t g, boo
 namespace {
 // Dense inverse of the coarsest level's operator (a uniform grid of root boxes: the 5-point
 // stencil with the wall rules), plus 1 1^T / n when the mesh is periodic in both directions.
-// Gauss-Jordan with partial pivoting in FP64, made symmetric; null (the CG is used) for a level larger than kDirectN cells or a singular matrix.  It depends
-// on the root grid and the walls only, so an adaptation keeps it.
+// Gauss-Jordan with partial pivoting in FP64, made symmetric; null (the CG is used) for a level
+// larger than kDirectN cells or a singular matrix.  It depends on the root grid and the walls
+// only, so an adaptation keeps it.
 double *coarse_inverse(pic_ctx *ctx, Instance &in, bool singular) {
     const Level &L = in.lv.back();
     const int n = (int)L.n;
