@@ -526,12 +526,15 @@ __global__ void __launch_bounds__(kT) k_uni_up(UniLevel A, const float *__restri
     }
 }
 
-// One-block Jacobi-preconditioned CG on the coarsest level (symmetric: one uniform level).
+// One-block Jacobi-preconditioned CG on the coarsest level (symmetric: one uniform level).  With
+// phi non-null (a mesh that does not coarsen: the coarsest level is the finest) the result is also
+// added to the potential.
 __global__ void __launch_bounds__(1024) k_coarse_cg(int64_t n, const int32_t *__restrict__ col,
                                                     const float *__restrict__ val, const float *__restrict__ dinv,
                                                     const float *__restrict__ b, float *__restrict__ x,
                                                     float *__restrict__ r, float *__restrict__ p,
-                                                    float *__restrict__ q, int singular, int maxit) {
+                                                    float *__restrict__ q, int singular, int maxit,
+                                                    double *__restrict__ phi) {
     pdl_chain();
     __shared__ double red[32];
     __shared__ double bcast;
@@ -605,6 +608,8 @@ __global__ void __launch_bounds__(1024) k_coarse_cg(int64_t n, const int32_t *__
         mx = bsum(mx) / (double)n;
         for (int64_t i = threadIdx.x; i < n; i += blockDim.x) x[i] -= (float)mx;
     }
+    if (phi)
+        for (int64_t i = threadIdx.x; i < n; i += blockDim.x) phi[i] += (double)x[i];
 }
 
 // ---- levels held in shared memory by one block (n <= kSmallN cells each) ----------------
@@ -1588,8 +1593,9 @@ void vcycle(pic_ctx *ctx, Instance &in, size_t g, bool singular) {
     if (g + 1 == in.lv.size()) {
         const int maxit = (int)std::min<int64_t>(2 * L.n + 10, 500);
         // r, p, q: three slices of the coarsest level's work buffer (allocated 3n)
-        pdl(k_coarse_cg, 1, 1024, 0, s, L.n, L.col, L.val, L.dinv, L.b, L.x, L.t, L.t + L.n, L.t + 2 * L.n,
-                                       singular, maxit);
+        double *phi = g == 0 ? in.phi : nullptr;
+        pdl(k_coarse_cg, 1, 1024, 0, s, L.n, L.col, L.val, L.dinv, L.b, L.x, L.t, L.t + L.n, L.t + 2 * L.n, singular,
+            maxit, phi);
         count_launch(ctx);
         return;
     }
