@@ -1536,7 +1536,11 @@ SmallDesc small_desc(const Instance &in, int g0) {
     int64_t floats = 3 * nl + 16;
     for (size_t g = g0; g < in.lv.size(); ++g) floats += 2 * in.lv[g].n + 16;
     const bool fits = floats * 4 + words * (in.cfg.implicit ? 4 : 8) + 8192 + 16 <= kSmallSmemMax;
-    D.build = in.cfg.implicit && nl <= kDirectN && fits ? 1 : 0;
+    // (an inverse needs a Dirichlet wall, or the periodic case's constant mode taken out; between
+    // Neumann walls alone the operator is singular and the CG solves what the charge allows)
+    const bool wall = in.cfg.bc_x == PIC_BC_DIRICHLET || in.cfg.bc_y == PIC_BC_DIRICHLET;
+    const bool periodic = in.cfg.bc_x == PIC_BC_PERIODIC && in.cfg.bc_y == PIC_BC_PERIODIC;
+    D.build = in.cfg.implicit && nl <= kDirectN && fits && (wall || periodic) ? 1 : 0;
     for (int k = 0; k < D.nlev; ++k) {
         const Level &L = in.lv[g0 + k];
         SmallLevel &S = D.lv[k];
