@@ -121,86 +121,34 @@ struct CicDepositArgs {
     double *part;
 };
 
-// A sum of products: FP64 state in FP64; FP32 state as an unevaluated pair of FP32 words (exact
-// products, error-free additions: ~46 bits), since GB300 retires two FP64 lanes per clock and SM
-// against 128 FP32 ones.
-struct Pair { float h, l; };
-__device__ __forceinline__ Pair pair_diff(float x, float y) {  // x - y
-    const float d = x - y, t = d - x;
-    return Pair{d, (x - (d - t)) - (y + t)};
+// x in FP64, exactly.  GB300 retires two FP64-pipe lanes per clock and SM, and a conversion from
+// FP32 is one of them: a normal number's bits are moved instead.
+__device__ __forceinline__ double widened(double x) { return x; }
+__device__ __forceinline__ double widened(float x) {
+    const uint32_t b = __float_as_uint(x), m = b & 0x7FFFFFFFu;
+    if (m - 0x00800000u >= 0x7F000000u) return (double)x;  // zero, denormal, infinite or not a number
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
 }
-__device__ __forceinline__ Pair pair_scale(float w, Pair a) {  // w a
-    const float h = w * a.h;
-    return Pair{h, fmaf(w, a.l, fmaf(w, a.h, -h))};
+// x added to a if `first`, else to b (one FP64 addition; two predicated ones take the pipe twice)
+__device__ __forceinline__ void add_either(bool first, double &a, double &b, double x) {
+    const double s = (first ? a : b) + x;
+    a = first ? s : a;
+    b = first ? b : s;
 }
-__device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
-    const float h = a.h * b.h;
-    return Pair{h, fmaf(a.h, b.h, -h) + (a.h * b.l + a.l * b.h)};
-}
-__device__ __forceinline__ void pair_add(Pair &s, Pair p) {
-    const float t = s.h + p.h, u = t - s.h;
-    s.l += ((s.h - (t - u)) + (p.h - u)) + p.l;
-    s.h = t;
-}
-template <typename R> struct CicAcc;
-template <> struct CicAcc<double> {
-    double v = 0.0;
-    __device__ __forceinline__ void add(const CicAcc &o) { v += o.v; }
-    __device__ __forceinline__ double value() const { return v; }
-    __device__ __forceinline__ void store(double *hi, double *) const { *hi = v; }
-    __device__ __forceinline__ void load(const double *hi, const double *) { v = *hi; }
-    __device__ __forceinline__ CicAcc down(int o) const {
-        CicAcc r;
-        r.v = __shfl_down_sync(0xFFFFFFFFu, v, o);
-        return r;
-    }
-    static __device__ __forceinline__ CicAcc of(double w) { CicAcc r; r.v = w; return r; }
-    // (|u - 1/2|, whether u < 1/2)
-    static __device__ __forceinline__ CicAcc half(double u, bool &neg) {
-        const double d = u - 0.5;
-        neg = __double2hiint(d) < 0;
-        return of(fabs(d));
-    }
-    __device__ __forceinline__ CicAcc scaled(double w) const { return of(w * v); }
-    __device__ __forceinline__ CicAcc times(const CicAcc &o) const { return of(v * o.v); }
-};
-template <> struct CicAcc<float> {
-    Pair p{0.0f, 0.0f};
-    __device__ __forceinline__ void add(const CicAcc &o) { pair_add(p, o.p); }
-    __device__ __forceinline__ double value() const { return (double)p.h + (double)p.l; }
-    __device__ __forceinline__ void store(float *hi, float *lo) const { *hi = p.h; *lo = p.l; }
-    __device__ __forceinline__ void load(const float *hi, const float *lo) { p.h = *hi; p.l = *lo; }
-    __device__ __forceinline__ CicAcc down(int o) const {
-        CicAcc r;
-        r.p.h = __shfl_down_sync(0xFFFFFFFFu, p.h, o);
-        r.p.l = __shfl_down_sync(0xFFFFFFFFu, p.l, o);
-        return r;
-    }
-    static __device__ __forceinline__ CicAcc of(float w) { CicAcc r; r.p.h = w; return r; }
-    static __device__ __forceinline__ CicAcc half(float u, bool &neg) {
-        CicAcc r;
-        r.p = pair_diff(u, 0.5f);
-        neg = r.p.h < 0.0f || (r.p.h == 0.0f && r.p.l < 0.0f);
-        if (neg) { r.p.h = -r.p.h; r.p.l = -r.p.l; }
-        return r;
-    }
-    __device__ __forceinline__ CicAcc scaled(float w) const { CicAcc r; r.p = pair_scale(w, p); return r; }
-    __device__ __forceinline__ CicAcc times(const CicAcc &o) const { CicAcc r; r.p = pair_mul(p, o.p); return r; }
-};
 
 // One warp per leaf.  A particle's weights on the three columns around its cell are
 // (a, 1 - a - c, c) with a = max(1/2 - u, 0), c = max(u - 1/2, 0) (one of them zero), and
-// likewise on the rows, so the nine sums 1, a, c, a', c', aa', ca', ac', cc' (times w) give the
-// nine cells: 12 operations per particle instead of the ~55 of nine predicated accumulators per
-// centre; the lanes are combined through shared memory, three lanes per sum.  512 x 16 FP32
-// discharge: the deposit 0.258 ms per step at first, 0.120 with these sums in FP64, 0.055 so.
+// likewise on the rows, so the nine sums 1, a, c, a', c', aa', ca', ac', cc' (times q w) give the
+// nine cells: 10 FP64 operations per particle instead of the ~55 of nine predicated accumulators
+// per centre; the lanes are combined through shared memory, three lanes per sum.  The FP64 pipe
+// bounds it.  512 x 16 FP32 discharge: the deposit 0.258 ms per step with nine predicated accumulators,
+// 0.119 with the nine sums, 0.089 with one addition for either sum and the conversions off the
+// pipe, 0.084 with the next chunk's loads under way.
 constexpr int kCicSums = 9;
 template <typename R>
-__global__ void __launch_bounds__(kT) k_cic_deposit(CicDepositArgs a) {
-    __shared__ R hi[kT / 32][kCicSums][33], lo[kT / 32][sizeof(R) == 4 ? kCicSums : 1][33];
-    __shared__ double tot[kT / 32][kCicSums];
+__global__ void __launch_bounds__(kT) k_cic_deposit(const __grid_constant__ CicDepositArgs a) {
+    __shared__ double lanes[kT / 32][kCicSums][33], tot[kT / 32][kCicSums];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    auto low = [&](int k, int j) { return &lo[wib][sizeof(R) == 4 ? k : 0][j]; };
     // cell k of the 3 x 3 block as a combination of the sums: bit j of plus / minus
     // (sums: 0: 1, 1: a, 2: c, 3: a', 4: c', 5: aa', 6: ca', 7: ac', 8: cc')
     const uint32_t plus[9] = {1u << 5, 1u << 3, 1u << 6, 1u << 1, 1u | 0xFu << 5, 1u << 2, 1u << 7, 1u << 4, 1u << 8};
@@ -212,48 +160,50 @@ __global__ void __launch_bounds__(kT) k_cic_deposit(CicDepositArgs a) {
     const int sum = lane / 3, j0 = 11 * (lane - 3 * sum);  // this lane's sum and its lanes from j0 on
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t L = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; L < a.nl; L += nw) {
-        double q_sum = 0.0;
+        double S[kCicSums] = {};
         for (int s = 0; s < a.nsp; ++s) {
             const R *U = (const R *)a.u[s], *V = (const R *)a.v[s], *Wt = (const R *)a.w[s];
-            CicAcc<R> S[kCicSums];
-            for (int32_t p = a.start[s][L] + lane; p < a.end[s][L]; p += 32) {
-                const R w = Wt[p];
-                bool nu, nv;
-                const CicAcc<R> du = CicAcc<R>::half(U[p], nu), dv = CicAcc<R>::half(V[p], nv);
-                const CicAcc<R> x = du.scaled(w), y = dv.scaled(w), xy = x.times(dv);
-                S[0].add(CicAcc<R>::of(w));
-                if (nu) S[1].add(x); else S[2].add(x);
-                if (nv) S[3].add(y); else S[4].add(y);
-                if (nv) { if (nu) S[5].add(xy); else S[6].add(xy); }
-                else { if (nu) S[7].add(xy); else S[8].add(xy); }
+            const double q = a.q[s];
+            int32_t p = a.start[s][L] + lane;
+            const int32_t p1 = a.end[s][L];
+            R fu = 0, fv = 0, fw = 0;  // the next chunk's words, loaded before this chunk's arithmetic
+            if (p < p1) { fu = U[p]; fv = V[p]; fw = Wt[p]; }
+            while (p < p1) {
+                const R cu = fu, cv = fv, cw = fw;
+                p += 32;
+                if (p < p1) { fu = U[p]; fv = V[p]; fw = Wt[p]; }
+                const double w = q * widened(cw);
+                const double du = widened(cu) - 0.5, dv = widened(cv) - 0.5;
+                const bool nu = __double2hiint(du) < 0, nv = __double2hiint(dv) < 0;
+                const double x = w * fabs(du), y = w * fabs(dv), xy = x * fabs(dv);
+                S[0] += w;
+                add_either(nu, S[1], S[2], x);
+                add_either(nv, S[3], S[4], y);
+                const double c = (nv ? (nu ? S[5] : S[6]) : (nu ? S[7] : S[8])) + xy;
+                S[5] = nu && nv ? c : S[5];
+                S[6] = !nu && nv ? c : S[6];
+                S[7] = nu && !nv ? c : S[7];
+                S[8] = !nu && !nv ? c : S[8];
             }
-#pragma unroll
-            for (int k = 0; k < kCicSums; ++k) S[k].store(&hi[wib][k][lane], low(k, lane));
-            __syncwarp();
-            CicAcc<R> t;
-            if (lane < 3 * kCicSums)
-#pragma unroll
-                for (int j = 0; j < 11; ++j)
-                    if (j0 + j < 32) {
-                        CicAcc<R> o;
-                        o.load(&hi[wib][sum][j0 + j], low(sum, j0 + j));
-                        t.add(o);
-                    }
-            const CicAcc<R> t1 = t.down(1), t2 = t.down(2);
-            t.add(t1);
-            t.add(t2);
-            q_sum += a.q[s] * t.value();  // (the sum's first lane holds it)
-            __syncwarp();
         }
-        if (lane < 3 * kCicSums && lane == 3 * sum) tot[wib][sum] = q_sum;
+#pragma unroll
+        for (int k = 0; k < kCicSums; ++k) lanes[wib][k][lane] = S[k];
+        __syncwarp();
+        double t = 0.0;
+        if (lane < 3 * kCicSums)
+#pragma unroll
+            for (int j = 0; j < 11; ++j)
+                if (j0 + j < 32) t += lanes[wib][sum][j0 + j];
+        const double t1 = __shfl_down_sync(0xFFFFFFFFu, t, 1), t2 = __shfl_down_sync(0xFFFFFFFFu, t, 2);
+        if (lane < 3 * kCicSums && lane == 3 * sum) tot[wib][sum] = (t + t1) + t2;
         __syncwarp();
         if (lane < 9) {
             double v = 0.0;
 #pragma unroll
             for (int j = 0; j < kCicSums; ++j) {
                 const double w = tot[wib][j];
-                if ((mp >> j) & 1u) v += w;
-                if ((mm >> j) & 1u) v -= w;
+                const double t = (mm >> j) & 1u ? -w : w;
+                if (((mp | mm) >> j) & 1u) v += t;
             }
             a.part[9 * L + lane] = v;
         }
