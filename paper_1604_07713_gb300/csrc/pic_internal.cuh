@@ -148,7 +148,7 @@ struct Species {
     void *stay_hi = nullptr, *stay_lo = nullptr;               // R [nleaf]
     void *ent_hi = nullptr, *ent_lo = nullptr;                 // R [nleaf]
     bool sums_valid = false;
-    int32_t *part = nullptr;  // [kPartWords] block totals of the re-layout's scan
+    int32_t *part = nullptr;  // [2 kPartWords] run totals of the re-layout's scan, with and without inflow room
 };
 
 template <typename R> struct SoA {

@@ -7,7 +7,7 @@
 // Entering records that find no free slot left go to the overflow store, and their leaf
 // moves to a fresh segment at the tail of the buffer (past every segment in use) with room
 // for them.  Only when the tail is used up are all lists of the species laid out again, in
-// leaf order with fresh free slots.  The device decides: a step without overflow runs three
+// leaf order with fresh free slots.  The device decides: a step without overflow runs five
 // launches whose blocks return at once, and the host never waits; the order of records inside a
 // list never depends on where its segment lies (order keys are list ranks, not slot numbers).
 //
@@ -15,8 +15,6 @@
 // per-leaf counts, list ranks and record totals, and the two repairs.
 #include <algorithm>
 #include <cstring>
-
-#include <cooperative_groups.h>
 
 #include "pic_internal.cuh"
 
@@ -247,6 +245,24 @@ __device__ __forceinline__ void place_ovf(const int32_t *__restrict__ end, int64
     }
 }
 
+// One leaf of the re-layout's step 1, by a warp.
+template <typename R>
+__device__ __forceinline__ void relayout_leaf(int64_t L, const int32_t *__restrict__ start, const int32_t *__restrict__ end,
+                                              const int32_t *__restrict__ lim, const int32_t *__restrict__ stay,
+                                              const int32_t *__restrict__ fill, const int32_t *start_new, SoA<R> d,
+                                              const uint32_t *__restrict__ key, const uint32_t *__restrict__ aux,
+                                              SoA<R> t, uint32_t *__restrict__ tkey, uint32_t *__restrict__ taux) {
+    const int lane = threadIdx.x & 31;
+    const int32_t s0 = start[L], q0 = start_new[L], ns = stay[L];
+    for (int32_t j = lane; j < ns; j += 32) copy_record(t, q0 + j, d, s0 + j);
+    const int32_t e0 = end[L], room = lim[L] - e0;
+    const int32_t k = fill[L] < room ? fill[L] : room;
+    for (int32_t j = lane; j < k; j += 32) {
+        const int32_t p = e0 + j, q = q0 + ns + j;
+        copy_record(t, q, d, p);
+        tkey[q] = key[p]; taux[q] = aux[p];
+    }
+}
 // Re-layout, step 1 (one warp per leaf): the staying records and the entering records that
 // found a free slot go to the scratch buffer at the new segment starts; staying records
 // first, entering records at their slot after them.
@@ -264,18 +280,7 @@ __device__ __forceinline__ void relayout_move(int64_t nl, const int32_t *__restr
         if (first) atomicExch(err, 1);
         return;
     }
-    const int lane = threadIdx.x & 31;
-    for (int64_t L = warp; L < nl; L += nw) {
-        const int32_t s0 = start[L], q0 = start_new[L], ns = stay[L];
-        for (int32_t j = lane; j < ns; j += 32) copy_record(t, q0 + j, d, s0 + j);
-        const int32_t e0 = end[L], room = lim[L] - e0;
-        const int32_t k = fill[L] < room ? fill[L] : room;
-        for (int32_t j = lane; j < k; j += 32) {
-            const int32_t p = e0 + j, q = q0 + ns + j;
-            copy_record(t, q, d, p);
-            tkey[q] = key[p]; taux[q] = aux[p];
-        }
-    }
+    for (int64_t L = warp; L < nl; L += nw) relayout_leaf<R>(L, start, end, lim, stay, fill, start_new, d, key, aux, t, tkey, taux);
 }
 template <typename R>
 __global__ void k_relayout_move(int64_t nl, const int32_t *__restrict__ start, const int32_t *__restrict__ end,
@@ -459,10 +464,12 @@ template <typename R> __device__ __forceinline__ void tail_moves(const ListEntry
     }
 }
 
-// After a push, the spawn offsets and the repairs of both species in three launches (they were
+// After a push, the spawn offsets and the repairs of both species in five launches (they were
 // three scan launches and, per species, a graph of two conditional nodes, ~25 us each): the
 // spawn scan's tile totals beside the tail moves, the scan itself beside the placement of the
-// overflow store, and the re-layout, whose blocks return at once unless a tail was used up.
+// overflow store, and the re-layout in three, whose blocks return at once unless a tail was used
+// up.  No block waits for another one, so the step runs on any share of the GPU's SMs (a
+// cooperative launch in their place is refused where its blocks do not all fit).
 // 512 x 16 discharge: 0.076 -> 0.019 ms per step.
 struct RepairArgs {
     ListEntry e[2];
@@ -471,8 +478,15 @@ struct RepairArgs {
     int32_t *spawn_base, *spart;
     int64_t nl;
     int tiles, runs;
-    int32_t *part[2];      // re-layout: block totals
+    int nb;                // the re-layout's runs of leaves, at most kPartWords
+    int32_t *part[2];      // re-layout: slots of each run with room for inflow, then without
 };
+// Slots of leaf L after a re-layout: free slots, and with `room` one more step of this step's inflow.
+__device__ __forceinline__ int32_t relayout_slots(const ListEntry &e, int64_t L, bool room) {
+    const int32_t f = e.fill[L], c = e.stay[L] + f;
+    return c + list_slack(c) + (room ? f : 0);
+}
+__device__ __forceinline__ int64_t run_leaves(const RepairArgs &A) { return (A.nl + A.nb - 1) / A.nb; }
 
 // Blocks (x, y): y < nsp moves that species' leaves, y == nsp counts the spawns of tile x.
 template <typename R> __global__ void __launch_bounds__(kT) k_step_move(const __grid_constant__ RepairArgs A) {
@@ -498,6 +512,20 @@ template <typename R> __global__ void __launch_bounds__(kT) k_step_place(const _
                      (int64_t)gridDim.x * blockDim.x, blockIdx.x == 0 && threadIdx.x == 0);
         // (after its count is read) the array holds the sort's medium regions next
         if (blockIdx.x == 0 && threadIdx.x == 0) e.moved[e.nl] = 0;
+        if (e.flags[5]) {  // the re-layout's totals
+            const int64_t per = run_leaves(A);
+            for (int r = blockIdx.x; r < A.nb; r += gridDim.x) {
+                int32_t with = 0, without = 0, tot;
+                for (int64_t L = per * r + threadIdx.x; L < min(e.nl, per * (r + 1)); L += kT) {
+                    with += relayout_slots(e, L, true);
+                    without += relayout_slots(e, L, false);
+                }
+                block_exclusive_scan(with, &tot);
+                if (threadIdx.x == 0) A.part[blockIdx.y][r] = tot;
+                block_exclusive_scan(without, &tot);
+                if (threadIdx.x == 0) A.part[blockIdx.y][kPartWords + r] = tot;
+            }
+        }
         return;
     }
     if ((int)blockIdx.x >= A.tiles) return;
@@ -518,59 +546,51 @@ template <typename R> __global__ void __launch_bounds__(kT) k_step_place(const _
     if ((int)blockIdx.x == A.tiles - 1 && threadIdx.x == 0) A.spawn_base[A.nl] = carry;
 }
 
-// The re-layout of the species whose tail was used up (flags[5]), as one cooperative launch of at
-// most kPartWords blocks: block b sums and scans the new segment sizes of its run of leaves
-// (with room for one more step of this step's inflow, or without when that does not fit), then
-// the records move through the scratch buffer as in relayout_lists.
+// The re-layout of the species whose tail was used up (flags[5]), blocks (x, species): block x
+// scans the new segment sizes of run x of the leaves (with room for one more step of this step's
+// inflow, or without when that does not fit) and moves their records to the scratch buffer, then
+// the records go on as in relayout_lists.
 template <typename R> __global__ void __launch_bounds__(kT) k_step_relayout(const __grid_constant__ RepairArgs A) {
-    namespace cg = cooperative_groups;
-    cg::grid_group grid = cg::this_grid();
-    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
-    for (int s = 0; s < A.nsp; ++s) {
-        const ListEntry &e = A.e[s];
-        if (e.flags[5] == 0) continue;  // the same on every block: the flag holds still from here on
-        const int64_t per = (e.nl + gridDim.x - 1) / gridDim.x;
-        const int64_t La = min(e.nl, per * blockIdx.x), Lb = min(e.nl, La + per);
-        for (int room = 1; room >= 0; --room) {
-            auto size = [&](int64_t L) -> int32_t {
-                if (L >= Lb) return 0;
-                const int32_t f = e.fill[L], c = e.stay[L] + f;
-                return c + list_slack(c) + (room ? f : 0);
-            };
-            int32_t sum = 0, tot;
-            for (int64_t L = La + threadIdx.x; L < Lb; L += kT) sum += size(L);
-            block_exclusive_scan(sum, &tot);
-            if (threadIdx.x == 0) A.part[s][blockIdx.x] = tot;
-            grid.sync();
-            const int32_t all = tiles_before(A.part[s], gridDim.x);
-            if (room && (int64_t)all > e.cap) {
-                grid.sync();  // every block has read the totals
-                continue;
-            }
-            int32_t carry = tiles_before(A.part[s], blockIdx.x);
-            for (int64_t L0 = La; L0 < Lb; L0 += kT) {
-                const int64_t L = L0 + threadIdx.x;
-                const int32_t v = size(L);
-                const int32_t at = block_exclusive_scan(v, &tot) + carry;
-                if (L < Lb) e.start_new[L] = at;
-                carry += tot;
-            }
-            if (i0 == 0) e.start_new[e.nl] = all;
-            break;
-        }
-        grid.sync();
-        relayout_move<R>(e.nl, e.start, e.end, e.lim, e.stay, e.fill, e.start_new, e.cap, soa_of<R>(e.d), e.key,
-                         e.aux, soa_of<R>(e.t), e.tkey, e.taux, e.flags, e.err, i0 >> 5, stride >> 5, i0 == 0);
-        // a leaf that still found its room at the tail this step was copied with the (empty) slots
-        // of its overflow records: they land there only now
-        grid.sync();
-        relayout_ovf<R>(e.stay, e.start_new, e.nl, e.cap, soa_of<R>(e.o), e.okey, e.oaux, e.odest, e.oslot,
-                        soa_of<R>(e.t), e.tkey, e.taux, e.flags, i0, stride);
-        grid.sync();
-        relayout_back<R>(e.nl, e.start_new, e.stay, e.cap, soa_of<R>(e.t), e.tkey, e.taux, soa_of<R>(e.d), e.key,
-                         e.aux, e.start, e.end, e.lim, e.flags, i0, stride, i0 == 0);
-        grid.sync();  // before the next species' totals
+    pdl_chain();
+    const ListEntry &e = A.e[blockIdx.y];
+    if (e.flags[5] == 0) return;
+    const int32_t *part = A.part[blockIdx.y];
+    const bool room = (int64_t)tiles_before(part, A.nb) <= e.cap;
+    if (!room) part += kPartWords;
+    const int32_t all = tiles_before(part, A.nb);
+    const int64_t per = run_leaves(A), La = min(e.nl, per * blockIdx.x), Lb = min(e.nl, La + per);
+    int32_t carry = tiles_before(part, blockIdx.x);
+    for (int64_t L0 = La; L0 < Lb; L0 += kT) {
+        const int64_t L = L0 + threadIdx.x;
+        int32_t tot;
+        const int32_t at = block_exclusive_scan(L < Lb ? relayout_slots(e, L, room) : 0, &tot) + carry;
+        if (L < Lb) e.start_new[L] = at;
+        carry += tot;
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        e.start_new[e.nl] = all;
+        if ((int64_t)all > e.cap) atomicExch(e.err, 1);
+    }
+    if ((int64_t)all > e.cap) return;
+    __syncthreads();  // the run's new starts
+    for (int64_t L = La + (threadIdx.x >> 5); L < Lb; L += kT / 32)
+        relayout_leaf<R>(L, e.start, e.end, e.lim, e.stay, e.fill, e.start_new, soa_of<R>(e.d), e.key, e.aux, soa_of<R>(e.t),
+                         e.tkey, e.taux);
+}
+// (a leaf that still found its room at the tail this step was copied with the (empty) slots of its
+// overflow records: they land there only now)
+template <typename R> __global__ void __launch_bounds__(kT) k_step_relayout_ovf(const __grid_constant__ RepairArgs A) {
+    pdl_chain();
+    const ListEntry &e = A.e[blockIdx.y];
+    relayout_ovf<R>(e.stay, e.start_new, e.nl, e.cap, soa_of<R>(e.o), e.okey, e.oaux, e.odest, e.oslot, soa_of<R>(e.t),
+                    e.tkey, e.taux, e.flags, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+}
+template <typename R> __global__ void __launch_bounds__(kT) k_step_relayout_back(const __grid_constant__ RepairArgs A) {
+    pdl_chain();
+    const ListEntry &e = A.e[blockIdx.y];
+    relayout_back<R>(e.nl, e.start_new, e.stay, e.cap, soa_of<R>(e.t), e.tkey, e.taux, soa_of<R>(e.d), e.key, e.aux,
+                     e.start, e.end, e.lim, e.flags, (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
+                     (int64_t)gridDim.x * blockDim.x, blockIdx.x == 0 && threadIdx.x == 0);
 }
 
 template <typename R> void step_repairs_impl(pic_ctx *ctx, Instance &in, bool ionize) {
@@ -589,33 +609,16 @@ template <typename R> void step_repairs_impl(pic_ctx *ctx, Instance &in, bool io
         A.spawn_base = in.sp[0].spawn_base;
         A.spart = in.sp[0].spart + A.tiles;
     }
+    // at most one run per 8 leaves: a small mesh's launches return sooner
+    A.nb = (int)std::max<int64_t>(1, std::min<int64_t>(152 * 4, (A.nl + 7) / 8));
     const dim3 grid((unsigned)std::max(152, ionize ? A.tiles : 0), (unsigned)(A.nsp + (ionize ? 1 : 0)));
     pdl(k_step_move<R>, grid, kT, 0, st, A);
     pdl(k_step_place<R>, grid, kT, 0, st, A);
-    count_launch(ctx, 2);
-    if (ctx->capturing) {
-        // a captured step of many instances runs them on parallel branches: gated launches
-        // behind IF nodes, so that no two cooperative launches can meet
-        for (int s = 0; s < A.nsp; ++s) {
-            capture_if(ctx, st, in.sp[s].flags + 5, [&]() { relayout_lists<R>(ctx, in, s); });
-            count_launch(ctx);
-        }
-        return;
-    }
-    static int blocks = 0;  // per process (one device model)
-    if (!blocks) {
-        int dev = 0, sms = 0, per = 0;
-        GB_CUDA(cudaGetDevice(&dev));
-        GB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        GB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_step_relayout<R>, kT, 0));
-        if (per < 1) fail(PIC_ECUDA, "re-layout kernel does not fit on an SM");
-        blocks = std::min(kPartWords, sms * std::min(per, 4));
-    }
-    void *args[] = {&A};
-    // at most one block per 8 leaves: a small mesh's launch returns sooner
-    const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(blocks, (A.nl + 7) / 8));
-    GB_CUDA(cudaLaunchCooperativeKernel((const void *)k_step_relayout<R>, dim3(nb), dim3(kT), args, 0, st));
-    count_launch(ctx);
+    const dim3 runs((unsigned)A.nb, (unsigned)A.nsp);
+    pdl(k_step_relayout<R>, runs, kT, 0, st, A);
+    pdl(k_step_relayout_ovf<R>, dim3(152, (unsigned)A.nsp), kT, 0, st, A);
+    pdl(k_step_relayout_back<R>, runs, kT, 0, st, A);
+    count_launch(ctx, 5);
     check_launch("step_repairs");
 }
 
@@ -863,7 +866,7 @@ void species_alloc(pic_ctx *ctx, Instance &in, int s, int64_t cap) {
     sp.key = dalloc<uint32_t>(A, 2 * cap);
     sp.aux = dalloc<uint32_t>(A, 2 * cap);
     sp.flags = dalloc<int32_t>(A, 8);
-    sp.part = dalloc<int32_t>(A, kPartWords);
+    sp.part = dalloc<int32_t>(A, 2 * kPartWords);
     GB_CUDA(cudaMemsetAsync(sp.flags, 0, 8 * 4, ctx->stream));
     species_leaf_arrays(ctx, in, s, in.nleaf);
     sp.cur = 0;
