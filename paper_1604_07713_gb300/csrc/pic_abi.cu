@@ -650,7 +650,19 @@ pic_status pic_read_fields(pic_ctx *ctx, int32_t inst, int32_t field, double *ou
         if (!out || cap < need) return too_small();
         cudaStream_t st = ctx->stream;
         DeviceArena tmp(&ctx->cache);
-        // a field formed on the device in FP64, then one copy to the caller
+        // a field formed on the device in FP64, then one copy to the caller; counts, charge density
+        // and FP32 corner fields are formed on the host when the device has no room for that
+        auto spare = [&](int64_t n) -> double * {
+            try {
+                return dalloc<double>(tmp, n);
+            } catch (const Failure &e) {
+                if (e.code != PIC_ENOMEM) throw;
+                return nullptr;
+            }
+        };
+        auto fetch = [&](void *dst, const void *src, size_t bytes) {
+            GB_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, st));
+        };
         auto copy_out = [&](const double *d) {
             GB_CUDA(cudaMemcpyAsync(out, d, need * 8, cudaMemcpyDeviceToHost, st));
             GB_CUDA(cudaStreamSynchronize(st));
@@ -661,9 +673,20 @@ pic_status pic_read_fields(pic_ctx *ctx, int32_t inst, int32_t field, double *ou
             copy_out(in.phi);
             break;
         case PIC_FIELD_RHO: {
-            double *d = dalloc<double>(tmp, nl);
-            read_rho(ctx, in, d);
-            copy_out(d);
+            if (double *d = spare(nl)) {
+                read_rho(ctx, in, d);
+                copy_out(d);
+                break;
+            }
+            std::vector<uint8_t> lev(nl);
+            fetch(out, in.charge, nl * 8);
+            fetch(lev.data(), in.lv[0].lev, nl);
+            GB_CUDA(cudaStreamSynchronize(st));
+            const double hf = in.h0 / (double)(1 << in.lmax);
+            for (int64_t l = 0; l < nl; ++l) {
+                const double h = (double)(1 << (in.lmax - lev[l])) * hf;
+                out[l] = out[l] / (h * h) + in.cfg.rho_background;
+            }
             break;
         }
         case PIC_FIELD_COUNT_E:
@@ -673,18 +696,29 @@ pic_status pic_read_fields(pic_ctx *ctx, int32_t inst, int32_t field, double *ou
                 std::fill(out, out + nl, 0.0);
                 break;
             }
-            double *d = dalloc<double>(tmp, nl);
-            read_leaf_counts(ctx, in, s, d);
-            copy_out(d);
+            if (double *d = spare(nl)) {
+                read_leaf_counts(ctx, in, s, d);
+                copy_out(d);
+                break;
+            }
+            std::vector<int32_t> first(nl), last(nl);
+            fetch(first.data(), in.sp[s].start, nl * 4);
+            fetch(last.data(), in.sp[s].end, nl * 4);
+            GB_CUDA(cudaStreamSynchronize(st));
+            for (int64_t l = 0; l < nl; ++l) out[l] = (double)(last[l] - first[l]);
             break;
         }
         case PIC_FIELD_NODE_E:
             if (in.cfg.precision == PIC_FP64) {
                 copy_out((const double *)in.stencil);
-            } else {
-                double *d = dalloc<double>(tmp, need);
+            } else if (double *d = spare(need)) {
                 read_widened(ctx, (const float *)in.stencil, need, d);
                 copy_out(d);
+            } else {
+                std::vector<float> e(need);
+                fetch(e.data(), in.stencil, need * 4);
+                GB_CUDA(cudaStreamSynchronize(st));
+                std::copy(e.begin(), e.end(), out);
             }
             break;
         case PIC_FIELD_EMAG: {
