@@ -435,21 +435,26 @@ static vec2 node_e(const or_mesh *m, const double *phi, const double *walls, int
     int64_t LL = or_leaf_at(m, I - 1, J - 1), LR = or_leaf_at(m, I, J - 1);
     int64_t UL = or_leaf_at(m, I - 1, J), UR = or_leaf_at(m, I, J);
     /* hanging: the node lies strictly inside an edge of one leaf */
+    /* (off: the node's distance along the edge; 0 where a leaf as wide as a periodic
+     * domain meets itself across the wrap and the node is its corner) */
     int64_t q = -1;
     int horizontal = 0;
-    if (UL >= 0 && UL == UR) { q = UL; horizontal = 1; }      /* bottom edge of q */
-    else if (LL >= 0 && LL == LR) { q = LL; horizontal = 1; } /* top edge of q */
-    else if (LL >= 0 && LL == UL) { q = LL; horizontal = 0; } /* right edge of q */
-    else if (LR >= 0 && LR == UR) { q = LR; horizontal = 0; } /* left edge of q */
+    int32_t off = 0;
+#define INSIDE_X(c) ((off = ((I - m->ix[c]) % lat_nx(m) + lat_nx(m)) % lat_nx(m)) != 0)
+#define INSIDE_Y(c) ((off = ((J - m->iy[c]) % lat_ny(m) + lat_ny(m)) % lat_ny(m)) != 0)
+    if (UL >= 0 && UL == UR && INSIDE_X(UL)) { q = UL; horizontal = 1; }      /* bottom edge of q */
+    else if (LL >= 0 && LL == LR && INSIDE_X(LL)) { q = LL; horizontal = 1; } /* top edge of q */
+    else if (LL >= 0 && LL == UL && INSIDE_Y(LL)) { q = LL; horizontal = 0; } /* right edge of q */
+    else if (LR >= 0 && LR == UR && INSIDE_Y(LR)) { q = LR; horizontal = 0; } /* left edge of q */
+#undef INSIDE_X
+#undef INSIDE_Y
     if (q >= 0) {
         int32_t s = m->s[q];
         int32_t I0, J0, I1, J1;
         if (horizontal) {
             /* the edge's x-range is [ix, ix+s] in the periodic-unwrapped frame of the node */
-            int32_t off = ((I - m->ix[q]) % lat_nx(m) + lat_nx(m)) % lat_nx(m);
             I0 = I - off; I1 = I0 + s; J0 = J1 = J;
         } else {
-            int32_t off = ((J - m->iy[q]) % lat_ny(m) + lat_ny(m)) % lat_ny(m);
             J0 = J - off; J1 = J0 + s; I0 = I1 = I;
         }
         vec2 a = node_e(m, phi, walls, I0, J0), b = node_e(m, phi, walls, I1, J1);

@@ -337,20 +337,28 @@ template <typename T> struct FieldView {
             const int32_t i = sI[top], j = sJ[top];
             const T wt = sw[top];
             const int32_t LL = L.at(i - 1, j - 1), LR = L.at(i, j - 1), UL = L.at(i - 1, j), UR = L.at(i, j);
-            int32_t q = -1;
+            // the node's distance along that edge; 0 where a leaf as wide as a periodic domain meets
+            // itself across the wrap: the node is then the leaf's corner, not inside its edge
+            int32_t q = -1, off = 0;
             bool horiz = false;
-            if (UL >= 0 && UL == UR) { q = UL; horiz = true; }
-            else if (LL >= 0 && LL == LR) { q = LL; horiz = true; }
-            else if (LL >= 0 && LL == UL) { q = LL; horiz = false; }
-            else if (LR >= 0 && LR == UR) { q = LR; horiz = false; }
+            auto inside_x = [&](int32_t c) {
+                off = (((i - L.ix[c]) % L.NX) + L.NX) % L.NX;
+                return off != 0;
+            };
+            auto inside_y = [&](int32_t c) {
+                off = (((j - L.iy[c]) % L.NY) + L.NY) % L.NY;
+                return off != 0;
+            };
+            if (UL >= 0 && UL == UR && inside_x(UL)) { q = UL; horiz = true; }
+            else if (LL >= 0 && LL == LR && inside_x(LL)) { q = LL; horiz = true; }
+            else if (LL >= 0 && LL == UL && inside_y(LL)) { q = LL; horiz = false; }
+            else if (LR >= 0 && LR == UR && inside_y(LR)) { q = LR; horiz = false; }
             if (q >= 0 && top + 2 <= 24) {
                 const int32_t s = L.side(q);
                 if (horiz) {
-                    const int32_t off = (((i - L.ix[q]) % L.NX) + L.NX) % L.NX;
                     sI[top] = i - off; sJ[top] = j; sw[top] = (T)0.5 * wt; ++top;
                     sI[top] = i - off + s; sJ[top] = j; sw[top] = (T)0.5 * wt; ++top;
                 } else {
-                    const int32_t off = (((j - L.iy[q]) % L.NY) + L.NY) % L.NY;
                     sI[top] = i; sJ[top] = j - off; sw[top] = (T)0.5 * wt; ++top;
                     sI[top] = i; sJ[top] = j - off + s; sw[top] = (T)0.5 * wt; ++top;
                 }
