@@ -1493,9 +1493,10 @@ template <typename R> PushArgs<R> push_args(Instance &in, int s, int64_t step) {
         a.f_el = (float)(c.sigma_el / sc);
         a.f_iz = (float)(c.sigma_iz0 / sc);
         // a collision frequency factor below FP32's range bounds the probability of any speed FP32
-        // holds by 1e-11, which only the zero uniform is below; one above it makes the bound infinite
-        a.f_ok = hm > 0.0 && normal(hm) && normal(c.eps_th_ev) && c.eps_th_ev >= 0.0 && normal(g) && std::isfinite(A) &&
-                 std::isfinite(B) && c.sigma_el / sc < 1e6 && c.sigma_iz0 / sc < 1e6;
+        // holds by 1e-11, which only the zero uniform is below; with one above 1e12 speeds whose squares
+        // FP32 does not hold (below 4e-21) could collide
+        a.f_ok = hm > 0.0 && normal(hm) && normal(c.eps_th_ev) && c.eps_th_ev >= 0.0 && normal(g) && B < 1e12 &&
+                 A * std::max(c.sigma_el, c.sigma_iz0) / sc < 1e12 && c.sigma_el / sc < 1e6 && c.sigma_iz0 / sc < 1e6;
     }
     a.keys = philox_keys(c.seed);
     a.inst_word = (uint32_t)c.instance << 24;
