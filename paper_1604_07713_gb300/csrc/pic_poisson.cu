@@ -685,7 +685,8 @@ __device__ __forceinline__ T uni_row(int nx, int ny, uint32_t magic, int bcx, in
     return ((l + r) + dn) + up;
 }
 
-__device__ __forceinline__ float sm_row(const SmallDesc &D, const SmallLevel &L, const float *x, int i, float &d,
+template <typename Desc>
+__device__ __forceinline__ float sm_row(const Desc &D, const SmallLevel &L, const float *x, int i, float &d,
                                         float &dinv) {
     if (L.uniform) {
         int dd;
@@ -704,7 +705,8 @@ __device__ __forceinline__ float sm_row(const SmallDesc &D, const SmallLevel &L,
     d = __frcp_rn(dinv);
     return -off;
 }
-__device__ __forceinline__ float sm_row(const SmallDesc &D, const SmallLevel &L, const float *x, int i, float &d) {
+template <typename Desc>
+__device__ __forceinline__ float sm_row(const Desc &D, const SmallLevel &L, const float *x, int i, float &d) {
     float dinv;
     return sm_row(D, L, x, i, d, dinv);
 }
@@ -714,7 +716,7 @@ __device__ __forceinline__ float sm_row(const SmallDesc &D, const SmallLevel &L,
 // non-uniform mesh, and the result must not depend on thread order).  The block has 1024
 // threads; thread t owns cells t + 1024 k, k < 8, so the new values stay in registers.
 constexpr int kPerThread = kSmallN / 1024;
-__device__ void sm_smooth(const SmallDesc &D, const SmallLevel &L, float *x, const float *b, bool first) {
+__device__ __noinline__ void sm_smooth(const SmallDesc &D, const SmallLevel &L, float *x, const float *b, bool first) {
     if (first) {
         for (int i = threadIdx.x; i < L.n; i += blockDim.x) x[i] = 0.0f;
         __syncthreads();
@@ -765,8 +767,11 @@ __device__ float sm_block_sumf(float v, float *red) {
 // Coarsest level: Jacobi-preconditioned CG in shared memory (one uniform level: symmetric),
 // all in FP32 (GB300's FP64 rate is a small fraction of FP32), to 1e-3 relative residual,
 // which is all a coarse-grid correction needs.  Up to 256 cells it runs on the first warp.
-__device__ void sm_coarse_cg(const SmallDesc &D, const SmallLevel &L, float *x, const float *b, float *r, float *p,
+struct SmallWalls { int bcx, bcy; };
+__device__ void sm_coarse_cg(const SmallDesc &Ds, const SmallLevel &level, float *x, const float *b, float *r, float *p,
                              float *q, bool singular, float *red) {
+    const SmallWalls D{Ds.bcx, Ds.bcy};
+    const SmallLevel L = level;  // in registers: the vectors' stores could alias the shared copy
     const int n = L.n;
     const int maxit = min(2 * n + 10, 500);
     const bool warp_only = n <= 256;
@@ -890,7 +895,7 @@ __device__ void sm_coarse_direct(const SmallLevel &L, const double *inv, float *
 // stopped at 1e-3), in place by Gauss-Jordan without pivoting (the operator is symmetric and
 // positive definite).  Singular: A + alpha 1 1^T is inverted and the constant's image taken out
 // again, so that the mean of the right-hand side does not matter.  1024 threads; `tmp` 2 n words.
-__device__ void sm_build_inverse(const SmallLevel &L, float *M, bool singular, float *tmp) {
+__device__ __noinline__ void sm_build_inverse(const SmallLevel &L, float *M, bool singular, float *tmp) {
     const int n = L.n, ld = n | 1, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     float *rowk = tmp, *colk = tmp + n;
     const float alpha = singular ? __frcp_rn(L.dinv[0]) / (float)n : 0.0f;
@@ -1137,7 +1142,7 @@ __device__ __forceinline__ void kap_half(const SmallDesc &D, const SmallLevel &L
         xs[j] = (b[j] + kap_row(D, L, xo, j, k)) * __ldg(L.dinv + k.i);
     }
 }
-__device__ void kap_down(const SmallDesc &D, const SmallLevel &L, const SmallLevel &Cc, float *sm, int bar) {
+__device__ __noinline__ void kap_down(const SmallDesc &D, const SmallLevel &L, const SmallLevel &Cc, float *sm, int bar) {
     float *x0 = sm + L.off, *x1 = x0 + L.hs;
     const float *b0 = x0 + L.boff, *b1 = b0 + L.hs;
     for (int j = threadIdx.x; j < L.half; j += L.nthr) x0[j] = b0[j] * __ldg(L.dinv + kap_cell(L, j, 0).i);
@@ -1164,7 +1169,7 @@ __device__ void kap_down(const SmallDesc &D, const SmallLevel &L, const SmallLev
     }
     part_bar(bar, L.nthr);
 }
-__device__ void kap_up(const SmallDesc &D, const SmallLevel &L, const SmallLevel &Cc, float *sm, int bar) {
+__device__ __noinline__ void kap_up(const SmallDesc &D, const SmallLevel &L, const SmallLevel &Cc, float *sm, int bar) {
     float *x0 = sm + L.off, *x1 = x0 + L.hs;
     const float *b0 = x0 + L.boff, *xc = sm + Cc.off;
     const int nxh = L.nx >> 1;
