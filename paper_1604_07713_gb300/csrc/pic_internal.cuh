@@ -223,6 +223,7 @@ struct Instance {
     bool mg_on_device = false;     // last solve ran its loop on the device (stats below)
     double *mg_stats = nullptr;    // device: [cycles, rel. residual, max rel. since reset]
     double *coarse_inv = nullptr;        // coarsest multigrid level: dense FP64 inverse (small levels)
+    double *coarse_build = nullptr;      // implicit multi-block solves: the inverse of this step's operator (FP32)
     double *coarse_inv_mem = nullptr;    // its memory, kept over mesh rebuilds, and the root grid
     std::array<int, 4> coarse_inv_key = {0, 0, 0, 0};  // (nx, ny, walls) it was formed for
     DeviceArena inv_mem;

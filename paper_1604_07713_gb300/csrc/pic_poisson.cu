@@ -647,7 +647,7 @@ struct SmallDesc {
     int32_t off_cg;  // smem offset of the coarsest CG vectors r, p, q (3 n)
     int32_t smem_floats;  // a multiple of 4
     const double *cinv;  // coarsest level: dense FP64 inverse (n rows of n | 1 words), or null (CG)
-    int32_t build;       // 1: the inverse is formed by each launch (FP32, sm_build_inverse)
+    int32_t build;       // FP32 inverse (sm_build_inverse): 1: formed by each launch, 2: in cinv, formed once per solve
     int32_t inv_words;   // FP64 words of the inverse in shared memory, else 0
 };
 
@@ -891,7 +891,7 @@ __device__ void sm_coarse_direct(const SmallLevel &L, const double *inv, float *
 }
 
 // The implicit scheme's coarsest operator changes every step: its inverse is formed by the
-// launch that uses it, in FP32 (a coarse-grid correction needs three digits: the CG it replaces
+// launch that uses it (by one before the cycles of a multi-block solve), in FP32 (a coarse-grid correction needs three digits: the CG it replaces
 // stopped at 1e-3), in place by Gauss-Jordan without pivoting (the operator is symmetric and
 // positive definite).  Singular: A + alpha 1 1^T is inverted and the constant's image taken out
 // again, so that the mean of the right-hand side does not matter.  1024 threads; `tmp` 2 n words.
@@ -1248,6 +1248,16 @@ __device__ void sm_vcycle(const SmallDesc &D, float *sm, bool singular, float *r
     }
 }
 
+// The coarsest inverse of a multi-block solve of the implicit scheme, formed once before its cycles
+// (formed in every cycle's tail, 208 x 144 cells with 117 coarsest: 1.40 ms per solve of 5 cycles; so 0.59).
+__global__ void __launch_bounds__(1024, 1) k_coarse_inverse(const __grid_constant__ SmallLevel L, int singular,
+                                                            float *__restrict__ out) {
+    extern __shared__ __align__(16) float sm[];
+    __shared__ float tmp[2 * kDirectN];
+    sm_build_inverse(L, sm, singular != 0, tmp);
+    for (int k = threadIdx.x; k < L.n * (L.n | 1); k += 1024) out[k] = sm[k];
+}
+
 // Tail of a V-cycle started by the multi-block levels: b from global, x back to global.
 __global__ void __launch_bounds__(1024, 1) k_tail_vcycle(const __grid_constant__ SmallDesc Dp,
                                                        const float *__restrict__ gb, float *__restrict__ gx,
@@ -1268,7 +1278,6 @@ __global__ void __launch_bounds__(1024, 1) k_tail_vcycle(const __grid_constant__
         inv = cs;
     }
     pdl_chain();
-    if (D.build) sm_build_inverse(D.lv[D.nlev - 1], reinterpret_cast<float *>(cs), singular != 0, reinterpret_cast<float *>(scr));
     const SmallLevel &L = D.lv[0];
     for (int i = threadIdx.x; i < L.n; i += blockDim.x) sm[L.off + L.boff + sm_pos(L, i)] = gb[i];
     __syncthreads();
@@ -1361,7 +1370,7 @@ __global__ void __launch_bounds__(1024, 1) k_small_solve(const SmallSolve *__res
         inv = cs;
     }
     pdl_chain();  // what came before it reads is constant between mesh changes
-    if (rank == 0 && D.build)
+    if (rank == 0 && D.build == 1)
         sm_build_inverse(D.lv[D.nlev - 1], reinterpret_cast<float *>(vbuf + 1024 * nbuf), it.singular != 0,
                          reinterpret_cast<float *>(vbuf));
     float *lsm = cl.map_shared_rank(sm, 0);  // the leader's levels
@@ -1545,7 +1554,7 @@ SmallDesc small_desc(const Instance &in, int g0) {
     // Neumann walls alone the operator is singular and the CG solves what the charge allows)
     const bool wall = in.cfg.bc_x == PIC_BC_DIRICHLET || in.cfg.bc_y == PIC_BC_DIRICHLET;
     const bool periodic = in.cfg.bc_x == PIC_BC_PERIODIC && in.cfg.bc_y == PIC_BC_PERIODIC;
-    D.build = in.cfg.implicit && nl <= kDirectN && fits && (wall || periodic) ? 1 : 0;
+    D.build = in.cfg.implicit && nl <= kDirectN && fits && (wall || periodic) ? (in.coarse_build ? 2 : 1) : 0;
     for (int k = 0; k < D.nlev; ++k) {
         const Level &L = in.lv[g0 + k];
         SmallLevel &S = D.lv[k];
@@ -1581,7 +1590,7 @@ SmallDesc small_desc(const Instance &in, int g0) {
     D.off_cg = off;
     off += 3 * (int32_t)in.lv.back().n + 8;
     D.smem_floats = (off + 3) & ~3;
-    D.cinv = in.coarse_inv;
+    D.cinv = D.build == 2 ? in.coarse_build : in.coarse_inv;
     D.inv_words = fits && (D.build || D.cinv) ? (int32_t)(D.build ? (words + 1) / 2 : words) : 0;
     return D;
 }
@@ -1732,6 +1741,7 @@ void poisson_setup(pic_ctx *ctx, Instance &in) {
     // (the tail has no sums' buffers, and more static shared memory)
     GB_CUDA(cudaFuncSetAttribute(k_tail_vcycle, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmemMax - 8192));
     GB_CUDA(cudaFuncSetAttribute(k_small_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmemMax));
+    GB_CUDA(cudaFuncSetAttribute(k_coarse_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, kDirectN * (kDirectN | 1) * 4));
     DeviceArena &A = in.mesh_mem;
     const int64_t n = in.lv[0].n;
     in.phi = dalloc<double>(A, n);
@@ -1750,7 +1760,10 @@ void poisson_setup(pic_ctx *ctx, Instance &in) {
     // coarsest-level CG needs three extra vectors: give it its own buffers
     Level &c = in.lv.back();
     c.t = dalloc<float>(A, 3 * c.n + 16);
-    // (the implicit scheme's coarsest operator changes every step: the CG solves it)
+    // (the implicit scheme's coarsest operator changes every step: sm_build_inverse, or the CG)
+    in.coarse_build = in.cfg.implicit && small_from(in) > 0 && c.n <= kDirectN
+                          ? dalloc<double>(A, (kDirectN * (kDirectN | 1) + 1) / 2)
+                          : nullptr;
     in.coarse_inv = in.cfg.implicit ? nullptr
                                     : coarse_inverse(ctx, in, in.cfg.bc_x == PIC_BC_PERIODIC && in.cfg.bc_y == PIC_BC_PERIODIC);
     // meshes whose every level fits one block: the whole solve is one block's work item
@@ -1889,6 +1902,14 @@ void poisson_solve(pic_ctx *ctx, Instance &in, const double walls[4]) {
                                                                 cudaStreamCaptureModeThreadLocal);
         cudaGraphNodeParams np = {};
         if (e == cudaSuccess) {
+            if (in.coarse_build) {
+                const SmallDesc D = small_desc(in, small_from(in));
+                const SmallLevel &C = D.lv[D.nlev - 1];
+                if (D.build) {
+                    k_coarse_inverse<<<1, 1024, (size_t)C.n * (C.n | 1) * 4, cs>>>(C, singular, (float *)in.coarse_build);
+                    count_launch(ctx);
+                }
+            }
             issue_residual(1, h);
             cudaStreamCaptureStatus status;
             const cudaGraphNode_t *deps = nullptr;
