@@ -229,6 +229,7 @@ struct Instance {
     DeviceArena inv_mem;
     void *small_item = nullptr;          // meshes that fit one block: the solve's work item
     size_t small_smem = 0;               // and the shared memory of its levels
+    bool small_cg = false;               // its coarsest level is solved by the CG
     int small_cluster = 1;               // CTAs of its cluster when solved alone
     cudaGraphExec_t mg_cycle = nullptr;  // multi-block meshes: one captured cycle (V-cycle,
     int64_t mg_cycle_nodes = 0;          // correction, residual, norm read-back) and its launches

@@ -1190,8 +1190,8 @@ __device__ __noinline__ void kap_up(const SmallDesc &D, const SmallLevel &L, con
 // it.  ELL levels are swept by the whole block; a level stored by colour by its nthr threads,
 // whose other warps wait at the next finer level's barrier (barrier ids count from the first
 // such level).  `inv` is the coarsest inverse (FP32 where the launch built it; null: CG), `scr`
-// kDirectN doubles.
-__device__ void sm_vcycle(const SmallDesc &D, float *sm, bool singular, float *red, const double *inv, double *scr) {
+// kDirectN doubles.  CG: the coarsest level is solved by the CG.
+template <bool CG> __device__ void sm_vcycle(const SmallDesc &D, float *sm, bool singular, float *red, const double *inv, double *scr) {
     const int last = D.nlev - 1;
     int g = 0;
     for (; g < last && !D.lv[g].fast; ++g) {
@@ -1226,8 +1226,8 @@ __device__ void sm_vcycle(const SmallDesc &D, float *sm, bool singular, float *r
         const SmallLevel &L = D.lv[last];
         float *x = sm + L.off, *b = x + L.boff;
         float *r = sm + D.off_cg;
-        if (D.build) direct_solve(L.n, reinterpret_cast<const float *>(inv), x, b);
-        else if (inv) sm_coarse_direct(L, inv, x, b, last > gf ? D.lv[last - 1].nthr : 1024, 1 + last - gf, scr);
+        if (!CG && D.build) direct_solve(L.n, reinterpret_cast<const float *>(inv), x, b);
+        else if (!CG && inv) sm_coarse_direct(L, inv, x, b, last > gf ? D.lv[last - 1].nthr : 1024, 1 + last - gf, scr);
         else sm_coarse_cg(D, L, x, b, r, r + L.n, r + 2 * L.n, singular, red);
     }
     for (--g; g >= gf; --g) {
@@ -1281,7 +1281,7 @@ __global__ void __launch_bounds__(1024, 1) k_tail_vcycle(const __grid_constant__
     const SmallLevel &L = D.lv[0];
     for (int i = threadIdx.x; i < L.n; i += blockDim.x) sm[L.off + L.boff + sm_pos(L, i)] = gb[i];
     __syncthreads();
-    sm_vcycle(D, sm, singular != 0, redf, inv, scr);
+    sm_vcycle<false>(D, sm, singular != 0, redf, inv, scr);
     __syncthreads();
     for (int i = threadIdx.x; i < L.n; i += blockDim.x) gx[i] = sm[L.off + sm_pos(L, i)];
 }
@@ -1347,7 +1347,10 @@ struct SmallSolve {
     double tol;
 };
 
-// `nbuf`: chunk buffers of the sums that fit behind every item's levels.
+// `nbuf`: chunk buffers of the sums that fit behind every item's levels.  CG: a mesh solved alone
+// whose coarsest level goes to the CG, without the code of the direct solves (their registers cost
+// the CG's loops 2 %).
+template <bool CG>
 __global__ void __launch_bounds__(1024, 1) k_small_solve(const SmallSolve *__restrict__ items, int nbuf) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
@@ -1370,7 +1373,7 @@ __global__ void __launch_bounds__(1024, 1) k_small_solve(const SmallSolve *__res
         inv = cs;
     }
     pdl_chain();  // what came before it reads is constant between mesh changes
-    if (rank == 0 && D.build == 1)
+    if (!CG && rank == 0 && D.build == 1)
         sm_build_inverse(D.lv[D.nlev - 1], reinterpret_cast<float *>(vbuf + 1024 * nbuf), it.singular != 0,
                          reinterpret_cast<float *>(vbuf));
     float *lsm = cl.map_shared_rank(sm, 0);  // the leader's levels
@@ -1459,7 +1462,7 @@ __global__ void __launch_bounds__(1024, 1) k_small_solve(const SmallSolve *__res
                 }
             }
             __syncthreads();
-            if (!stop_sh) sm_vcycle(D, sm, singular != 0, redf, inv, vbuf);
+            if (!stop_sh) sm_vcycle<CG>(D, sm, singular != 0, redf, inv, vbuf);
         }
         cl.sync();  // the correction is in the leader's x
         if (*lstop) break;
@@ -1496,14 +1499,14 @@ cudaLaunchConfig_t small_config(int n_items, int C, size_t smem, cudaLaunchAttri
 }
 
 // One launch of the small solve: n_items clusters of C CTAs.
-void launch_small_solve(const void *items, int n_items, int C, int nbuf, size_t smem, cudaStream_t st) {
+void launch_small_solve(const void *items, int n_items, int C, int nbuf, size_t smem, bool cg, cudaStream_t st) {
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = small_config(n_items, C, smem, attr);
     cfg.stream = st;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = 2;
-    GB_CUDA(cudaLaunchKernelEx(&cfg, k_small_solve, (const SmallSolve *)items, nbuf));
+    GB_CUDA(cudaLaunchKernelEx(&cfg, cg ? k_small_solve<true> : k_small_solve<false>, (const SmallSolve *)items, nbuf));
 }
 
 // The cluster size for n_items instances solved in one launch: one CTA per 1024-cell chunk of
@@ -1520,7 +1523,7 @@ int small_cluster(int n, int n_items, size_t lv_bytes) {
         cudaLaunchAttribute attr[1];
         cudaLaunchConfig_t cfg = small_config(n_items, C, lv_bytes + (size_t)small_bufs(n, C, lv_bytes) * 8192, attr);
         int nc = 0;
-        if (cudaOccupancyMaxActiveClusters(&nc, k_small_solve, &cfg) == cudaSuccess && nc >= n_items) break;
+        if (cudaOccupancyMaxActiveClusters(&nc, k_small_solve<false>, &cfg) == cudaSuccess && nc >= n_items) break;
         cudaGetLastError();
     }
     return C;
@@ -1740,7 +1743,8 @@ void poisson_setup(pic_ctx *ctx, Instance &in) {
     }
     // (the tail has no sums' buffers, and more static shared memory)
     GB_CUDA(cudaFuncSetAttribute(k_tail_vcycle, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmemMax - 8192));
-    GB_CUDA(cudaFuncSetAttribute(k_small_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmemMax));
+    GB_CUDA(cudaFuncSetAttribute(k_small_solve<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmemMax));
+    GB_CUDA(cudaFuncSetAttribute(k_small_solve<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmemMax));
     GB_CUDA(cudaFuncSetAttribute(k_coarse_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, kDirectN * (kDirectN | 1) * 4));
     DeviceArena &A = in.mesh_mem;
     const int64_t n = in.lv[0].n;
@@ -1787,6 +1791,7 @@ void poisson_setup(pic_ctx *ctx, Instance &in) {
         GB_CUDA(cudaStreamSynchronize(ctx->stream));
         in.small_item = d;
         in.small_smem = (size_t)it.D.smem_floats * 4 + (size_t)it.D.inv_words * 8;
+        in.small_cg = !it.D.build && !it.D.cinv;
         in.small_cluster = small_cluster((int)L.n, 1, in.small_smem);
     }
     ++ctx->mesh_epoch;
@@ -1839,7 +1844,7 @@ void poisson_solve_batch(pic_ctx *ctx, const std::vector<Instance *> &list, cons
     }
     const int nbuf = small_bufs(ctx->batch_cells, ctx->batch_cluster, ctx->batch_smem);
     launch_small_solve(ctx->batch_items, (int)list.size(), ctx->batch_cluster, nbuf, ctx->batch_smem + (size_t)nbuf * 8192,
-                       ctx->stream);
+                       false, ctx->stream);
     count_launch(ctx);
     check_launch("poisson_solve_batch");
 }
@@ -1853,7 +1858,7 @@ void poisson_solve(pic_ctx *ctx, Instance &in, const double walls[4]) {
     const bool singular = in.cfg.bc_x == PIC_BC_PERIODIC && in.cfg.bc_y == PIC_BC_PERIODIC;
     if (in.small_item) {
         const int nbuf = small_bufs((int)n, in.small_cluster, in.small_smem);
-        launch_small_solve(in.small_item, 1, in.small_cluster, nbuf, in.small_smem + (size_t)nbuf * 8192, s);
+        launch_small_solve(in.small_item, 1, in.small_cluster, nbuf, in.small_smem + (size_t)nbuf * 8192, in.small_cg, s);
         count_launch(ctx);
         check_launch("poisson_solve");
         in.mg_on_device = true;
