@@ -895,7 +895,7 @@ __device__ void sm_coarse_direct(const SmallLevel &L, const double *inv, float *
 // stopped at 1e-3), in place by Gauss-Jordan without pivoting (the operator is symmetric and
 // positive definite).  Singular: A + alpha 1 1^T is inverted and the constant's image taken out
 // again, so that the mean of the right-hand side does not matter.  1024 threads; `tmp` 2 n words.
-__device__ __noinline__ void sm_build_inverse(const SmallLevel &L, float *M, bool singular, float *tmp) {
+__device__ __forceinline__ void form_inverse(const SmallLevel &L, float *M, bool singular, float *tmp) {
     const int n = L.n, ld = n | 1, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     float *rowk = tmp, *colk = tmp + n;
     const float alpha = singular ? __frcp_rn(L.dinv[0]) / (float)n : 0.0f;
@@ -933,6 +933,11 @@ __device__ __noinline__ void sm_build_inverse(const SmallLevel &L, float *M, boo
             for (int j = tx; j < n; j += 32) M[i * ld + j] -= c;
         __syncthreads();
     }
+}
+
+// (out of line in the solve kernel, whose registers it would take)
+__device__ __noinline__ void sm_build_inverse(const SmallLevel &L, float *M, bool singular, float *tmp) {
+    form_inverse(L, M, singular, tmp);
 }
 
 // ---- levels stored by colour --------------------------------------------------------------
@@ -1254,7 +1259,7 @@ __global__ void __launch_bounds__(1024, 1) k_coarse_inverse(const __grid_constan
                                                             float *__restrict__ out) {
     extern __shared__ __align__(16) float sm[];
     __shared__ float tmp[2 * kDirectN];
-    sm_build_inverse(L, sm, singular != 0, tmp);
+    form_inverse(L, sm, singular != 0, tmp);
     for (int k = threadIdx.x; k < L.n * (L.n | 1); k += 1024) out[k] = sm[k];
 }
 
