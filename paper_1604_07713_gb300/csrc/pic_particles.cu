@@ -122,19 +122,22 @@ struct DepositArgs {
     double chi[2];           // dt^2 q_s^2 / (m_s eps0)
 };
 
-// From the records (after a load, an adaptation or split/merge): a warp sums `per` consecutive
-// leaves one after another, and lane i then forms leaf i's charge and right-hand side.  With
-// one leaf a warp, every warp issued the ~25 FP64 instructions of a leaf for itself (an SM's
-// FP64 pipe takes two lanes a clock).  Streamer of 8.8e7 records on 9e5 leaves, ten steps of
-// which the first deposits this way: 0.14 -> 0.061 ms per step.
+// From the records (after a load, an adaptation or split/merge): a warp sums `per` leaves one after
+// another, and lane i then forms its i-th leaf's charge and right-hand side.  With one leaf a warp,
+// every warp issued the ~25 FP64 instructions of a leaf for itself (an SM's FP64 pipe takes two
+// lanes a clock).  Streamer of 8.8e7 records on 9e5 leaves, ten steps of which the first deposits
+// this way: 0.14 -> 0.060 ms per step.  A warp's leaves lie apart, so that long lists side by side
+// (a beam) go to different warps: 3e6 records per species in 120 of 810,000 leaves 1.13 ms with one
+// leaf a warp, 6.83 with `per` consecutive ones, 0.28 so; even lists on 512 x 512 leaves 0.084 -> 0.089.
 template <typename R>
 __global__ void __launch_bounds__(kT) k_deposit(DepositArgs a, int per) {
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t L0 = warp * per; L0 < a.nleaf; L0 += nw * per) {
-        const int m = (int)min((int64_t)per, a.nleaf - L0);
-        const int64_t L = L0 + lane;
+    const int64_t each = (a.nleaf + per - 1) / per;  // a warp's leaves are this far apart
+    for (int64_t L0 = warp; L0 < each; L0 += nw) {
+        const int m = (int)((a.nleaf - L0 + each - 1) / each);
+        const int64_t L = L0 + lane * each;
         double total = 0.0, chi = 0.0;
         for (int s = 0; s < a.nsp; ++s) {
             const int32_t f = lane < m ? a.start[s][L] : 0, e = lane < m ? a.end[s][L] : 0;
@@ -1209,11 +1212,13 @@ template <typename R> __global__ void __launch_bounds__(512) k_sort_big(const __
     pdl_chain();
     extern __shared__ unsigned long long bk[];
     __shared__ R red_hi[16], red_lo[16];
+    // (both counts read at once; one copy of the sort's code)
     const int32_t n0 = P.e[0].a.big[P.e[0].a.nleaf], n1 = nsp > 1 ? P.e[1].a.big[P.e[1].a.nleaf] : 0;
-    if (n0 > 0) sort_big_leaves<R>(P.e[0].a, P.e[0].d, P.e[0].t, blockIdx.x, gridDim.x, bk, red_hi, red_lo);
-    if (n1 > 0)
-        sort_big_leaves<R>(P.e[1].a, P.e[1].d, P.e[1].t, (blockIdx.x + gridDim.x - (uint32_t)n0 % gridDim.x) % gridDim.x,
-                           gridDim.x, bk, red_hi, red_lo);
+#pragma unroll 1
+    for (int s = n0 > 0 ? 0 : 1; s < (n1 > 0 ? 2 : 1); ++s) {
+        const int32_t first = s ? (blockIdx.x + gridDim.x - (uint32_t)n0 % gridDim.x) % gridDim.x : blockIdx.x;
+        sort_big_leaves<R>(P.e[s].a, P.e[s].d, P.e[s].t, first, gridDim.x, bk, red_hi, red_lo);
+    }
 }
 
 // ---- the sorts of every (instance, species) of an ensemble, one launch per pass ----------
