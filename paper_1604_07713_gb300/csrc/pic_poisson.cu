@@ -1702,26 +1702,29 @@ double *coarse_inverse(pic_ctx *ctx, Instance &in, bool singular) {
     for (int i = 0; i < n; ++i) Inv[(size_t)i * n + i] = 1.0;
     double amax = 0.0;
     for (double a : A) amax = std::max(amax, std::fabs(a));
+    // (left of the pivot A is the identity already, and right of it the inverse's rows are zero
+    // until rows are exchanged: setting a mesh of 11 x 11 cells 0.95 -> 0.64 ms)
+    int used = 0;  // the inverse's columns from `used` on are zero in the rows that eliminate
     for (int k = 0; k < n; ++k) {
         int piv = k;
         for (int i = k + 1; i < n; ++i)
             if (std::fabs(at(i, k)) > std::fabs(at(piv, k))) piv = i;
         if (!(std::fabs(at(piv, k)) > 1e-12 * amax)) return nullptr;
-        if (piv != k)
-            for (int j = 0; j < n; ++j) {
-                std::swap(at(k, j), at(piv, j));
-                std::swap(Inv[(size_t)k * n + j], Inv[(size_t)piv * n + j]);
-            }
-        const double p = 1.0 / at(k, k);
-        for (int j = 0; j < n; ++j) { at(k, j) *= p; Inv[(size_t)k * n + j] *= p; }
+        used = piv != k ? n : std::max(used, k + 1);
+        double *ak = A.data() + (size_t)k * n, *ik = Inv.data() + (size_t)k * n;
+        if (piv != k) {
+            std::swap_ranges(ak, ak + n, A.data() + (size_t)piv * n);
+            std::swap_ranges(ik, ik + n, Inv.data() + (size_t)piv * n);
+        }
+        const double p = 1.0 / ak[k];
+        for (int j = k; j < n; ++j) ak[j] *= p;
+        for (int j = 0; j < used; ++j) ik[j] *= p;
         for (int i = 0; i < n; ++i) {
-            if (i == k) continue;
-            const double f = at(i, k);
-            if (f == 0.0) continue;
-            for (int j = 0; j < n; ++j) {
-                at(i, j) -= f * at(k, j);
-                Inv[(size_t)i * n + j] -= f * Inv[(size_t)k * n + j];
-            }
+            double *ai = A.data() + (size_t)i * n, *ii = Inv.data() + (size_t)i * n;
+            const double f = ai[k];
+            if (i == k || f == 0.0) continue;
+            for (int j = k; j < n; ++j) ai[j] -= f * ak[j];
+            for (int j = 0; j < used; ++j) ii[j] -= f * ik[j];
         }
     }
     for (int i = 0; i < n; ++i)
