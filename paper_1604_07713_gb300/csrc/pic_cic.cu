@@ -9,7 +9,7 @@
 // weight folds into it); periodic directions wrap.
 //
 // Deposit: one warp per leaf sums its particles' charge into the 3 x 3 block of cells around
-// it (FP64 per lane, lanes combined by a fixed shuffle tree), then one thread per cell adds
+// it (FP64 per lane, the lanes in a fixed order), then one thread per cell adds
 // the contributions of its 9 neighbours in a fixed order: no atomics, the same bits every run.
 //
 // Field: for each leaf and each quarter (qx, qy) of it, the field over that quarter is a
@@ -139,7 +139,7 @@ __device__ __forceinline__ void add_either(bool first, double &a, double &b, dou
 // One warp per leaf.  A particle's weights on the three columns around its cell are
 // (a, 1 - a - c, c) with a = max(1/2 - u, 0), c = max(u - 1/2, 0) (one of them zero), and
 // likewise on the rows, so the nine sums 1, a, c, a', c', aa', ca', ac', cc' (times q w) give the
-// nine cells: 10 FP64 operations per particle instead of the ~55 of nine predicated accumulators
+// nine cells: 8 to 10 FP64 operations per particle instead of the ~55 of nine predicated accumulators
 // per centre; the lanes are combined through shared memory, three lanes per sum.  The FP64 pipe
 // bounds it.  512 x 16 FP32 discharge: the deposit 0.258 ms per step with nine predicated accumulators,
 // 0.119 with the nine sums, 0.089 with one addition for either sum and the conversions off the

@@ -181,7 +181,7 @@ struct Diag {
     int64_t nleaf = 0;
     double *leaf = nullptr;                 // [4 nleaf]: sum w_e, sum w_i, sum w_e eps [eV], sum phi
     double *eedf = nullptr;                 // [nbins] sum of electron weights per energy bin
-    double *part = nullptr;                 // per-warp partial histograms of one step
+    double *part = nullptr;                 // per bin the blocks' partial sums of one step
     DeviceArena mem;
 };
 
@@ -222,7 +222,7 @@ struct Instance {
     double mg_res_max = 0;         // host-driven solves: worst relative residual since reset
     bool mg_on_device = false;     // last solve ran its loop on the device (stats below)
     double *mg_stats = nullptr;    // device: [cycles, rel. residual, max rel. since reset]
-    double *coarse_inv = nullptr;        // coarsest multigrid level: dense FP64 inverse (small levels)
+    double *coarse_inv = nullptr;        // coarsest multigrid level: dense FP64 inverse (up to 128 cells)
     double *coarse_build = nullptr;      // implicit multi-block solves: the inverse of this step's operator (FP32)
     double *coarse_inv_mem = nullptr;    // its memory, kept over mesh rebuilds, and the root grid
     std::array<int, 4> coarse_inv_key = {0, 0, 0, 0};  // (nx, ny, walls) it was formed for

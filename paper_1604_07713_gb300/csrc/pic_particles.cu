@@ -80,8 +80,8 @@ __device__ __forceinline__ float abs_f32(double x) {
 
 template <typename R> __device__ __forceinline__ R u24(uint32_t r) { return (R)(r >> 8) * (R)(1.0 / 16777216.0); }
 
-// Compensated accumulation (Kahan) of one lane, and an error-free combination of the lanes'
-// (sum, -compensation) pairs: every lane ends with the same (hi, lo).
+// Compensated accumulation (Kahan) of one lane, and an error-free combination (Knuth's two-sum) of
+// the lanes' (sum, -compensation) pairs: every lane ends with the same (hi, lo).
 template <typename R> __device__ __forceinline__ void kahan_add(R &sum, R &c, R x) {
     const R y = x - c;
     const R t = sum + y;
@@ -292,10 +292,11 @@ template <typename R> struct PushArgs {
     R ng_dt, sig_el, sig_iz0, eps_th, half_m_over_qe, two_qe_over_m, two_m_over_mn;
     R vt_gas;       // neutral thermal speed sqrt(T qe / M)
     R red_a, red_m, red_mn;  // ions: M / (m + M), m / (m + M), M / (m + M)
-    R g_partner_max, g_pad;  // ions: bound on the partner speed (8.2 v_t), rounding margin
-    R p_pad;                 // rounding margin of the linear bound on the collision probability
-    // the bound test of the pass: electrons sigma_el / sc, sigma_iz0 / sc, (n dt sc p_pad)^2 with
-    // sc the larger nonzero cross section scale; ions 1 / (n dt sigma_el g_pad p_pad)
+    R g_partner_max;  // ions: bound on the partner speed (8.2 v_t)
+    // the bound test of the pass, with rounding margins of 1e-4 on the linear bound of the collision
+    // probability and 1e-3 on the partner speed: electrons sigma_el / sc, sigma_iz0 / sc,
+    // (n dt sc 1.0001)^2 with sc the larger nonzero cross section scale; ions
+    // 1 / (n dt sigma_el 1.001 1.0001)
     R bnd_el, bnd_iz, bnd_q, bnd_inv;
     // FP64 state: the same bound in FP32 (f_ok: its constants lie in FP32's range; else every
     // particle goes on to the exact test): electrons n dt sc, m / (2 qe), the threshold (a little
@@ -1486,8 +1487,6 @@ template <typename R> PushArgs<R> push_args(Instance &in, int s, int64_t step) {
     a.red_m = (R)(c.m[s] / mt);
     a.red_mn = (R)(c.neutral_mass / mt);
     a.g_partner_max = (R)(8.2 * std::sqrt(c.gas_temperature_ev * c.qe / c.neutral_mass));
-    a.g_pad = (R)1.001;
-    a.p_pad = (R)1.0001;
     {
         const double sc = c.sigma_el > 0.0 ? c.sigma_el : (c.sigma_iz0 > 0.0 ? c.sigma_iz0 : 1.0);
         const double A = c.gas_density * c.dt * sc * 1.0001;

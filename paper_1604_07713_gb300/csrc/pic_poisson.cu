@@ -3,12 +3,15 @@
 // phi += e are FP64 (iterative refinement); each correction e comes from one FP32
 // geometric-multigrid V-cycle over the tree-clamped and root-coarsened levels, with two
 // red-black Gauss-Seidel sweeps before and after the coarse correction, summed restriction
-// and piecewise-constant prolongation; the coarsest level (at most 64 cells) is solved by its
-// dense inverse, built on the host in FP64, or else by conjugate gradients.  Levels of at
-// most 8192 cells live in one block's shared memory; when every level does, the whole solve
-// (FP64 residual, V-cycles, convergence test) is a single launch of a thread-block cluster
-// that spreads the FP64 work over its SMs (one CTA per instance in a batch).  Larger meshes
-// run one CUDA graph per solve whose WHILE node repeats the cycle until the device decides.
+// and piecewise-constant prolongation.  The coarsest level, up to 128 cells, is solved by its
+// dense inverse: the explicit scheme's in FP64, formed on the host once per root grid and walls;
+// the implicit scheme's, whose operator changes every step, in FP32 on the device once per
+// solve.  A larger one, or one that is singular between Neumann walls, goes to conjugate
+// gradients.  Levels of at most 8192 cells live in one block's shared memory; when every level
+// does, the whole solve (FP64 residual, V-cycles, convergence test) is a single launch of
+// thread-block clusters, one per instance of a batch, that spread the FP64 work over their SMs.
+// Larger meshes run one CUDA graph per solve whose WHILE node repeats the cycle until the
+// device decides.
 #include <algorithm>
 #include <array>
 #include <cmath>
@@ -646,7 +649,7 @@ struct SmallDesc {
     SmallLevel lv[kMaxSmallLevels];
     int32_t off_cg;  // smem offset of the coarsest CG vectors r, p, q (3 n)
     int32_t smem_floats;  // a multiple of 4
-    const double *cinv;  // coarsest level: dense FP64 inverse (n rows of n | 1 words), or null (CG)
+    const double *cinv;  // coarsest level: dense inverse (n rows of n | 1 words; FP64, or FP32 with build 2), or null
     int32_t build;       // FP32 inverse (sm_build_inverse): 1: formed by each launch, 2: in cinv, formed once per solve
     int32_t inv_words;   // FP64 words of the inverse in shared memory, else 0
 };
