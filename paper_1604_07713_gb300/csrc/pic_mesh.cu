@@ -337,30 +337,26 @@ template <typename T> struct FieldView {
             const int32_t i = sI[top], j = sJ[top];
             const T wt = sw[top];
             const int32_t LL = L.at(i - 1, j - 1), LR = L.at(i, j - 1), UL = L.at(i - 1, j), UR = L.at(i, j);
-            // the node's distance along that edge; 0 where a leaf as wide as a periodic domain meets
-            // itself across the wrap: the node is then the leaf's corner, not inside its edge
-            int32_t q = -1, off = 0;
+            // (on the domain's first and last line a node is a corner of every leaf it touches: where
+            // the same leaf lies on both sides there, it is as wide as the periodic domain and meets
+            // itself across the wrap)
+            const bool in_i = i > 0 && i < L.NX, in_j = j > 0 && j < L.NY;
+            int32_t q = -1;
             bool horiz = false;
-            auto inside_x = [&](int32_t c) {
-                off = (((i - L.ix[c]) % L.NX) + L.NX) % L.NX;
-                return off != 0;
-            };
-            auto inside_y = [&](int32_t c) {
-                off = (((j - L.iy[c]) % L.NY) + L.NY) % L.NY;
-                return off != 0;
-            };
-            if (UL >= 0 && UL == UR && inside_x(UL)) { q = UL; horiz = true; }
-            else if (LL >= 0 && LL == LR && inside_x(LL)) { q = LL; horiz = true; }
-            else if (LL >= 0 && LL == UL && inside_y(LL)) { q = LL; horiz = false; }
-            else if (LR >= 0 && LR == UR && inside_y(LR)) { q = LR; horiz = false; }
+            if (UL >= 0 && UL == UR && in_i) { q = UL; horiz = true; }
+            else if (LL >= 0 && LL == LR && in_i) { q = LL; horiz = true; }
+            else if (LL >= 0 && LL == UL && in_j) { q = LL; horiz = false; }
+            else if (LR >= 0 && LR == UR && in_j) { q = LR; horiz = false; }
             if (q >= 0 && top + 2 <= 24) {
                 const int32_t s = L.side(q);
                 if (horiz) {
-                    sI[top] = i - off; sJ[top] = j; sw[top] = (T)0.5 * wt; ++top;
-                    sI[top] = i - off + s; sJ[top] = j; sw[top] = (T)0.5 * wt; ++top;
+                    const int32_t x = L.ix[q];
+                    sI[top] = x; sJ[top] = j; sw[top] = (T)0.5 * wt; ++top;
+                    sI[top] = x + s; sJ[top] = j; sw[top] = (T)0.5 * wt; ++top;
                 } else {
-                    sI[top] = i; sJ[top] = j - off; sw[top] = (T)0.5 * wt; ++top;
-                    sI[top] = i; sJ[top] = j - off + s; sw[top] = (T)0.5 * wt; ++top;
+                    const int32_t y = L.iy[q];
+                    sI[top] = i; sJ[top] = y; sw[top] = (T)0.5 * wt; ++top;
+                    sI[top] = i; sJ[top] = y + s; sw[top] = (T)0.5 * wt; ++top;
                 }
                 continue;
             }
